@@ -139,17 +139,17 @@ void pc_destroy(pc_handle *h);
  *                 default 128) run on the staged kernel, which holds
  *                 corr[adj(u), adj(u)] in shared memory; the rest read corr
  *                 from L2 (0 = staged kernel off)
- *   "stage_loop"  1 = problems of p <= 128 (not batched) run the stage loop in
- *                 one cooperative kernel, a grid-wide barrier where the captured
- *                 loop has a kernel boundary (tests, commit, degrees, next stage,
- *                 and in the reversed order the precision blocks); it runs the
- *                 complement tests and the direct tests of stages with at most
- *                 12 conditioning members and at most 16 tests per warp of its
- *                 grid, a warp each; from the first stage it does not take
- *                 (larger direct stages, or a stage the proposal may score) on,
- *                 the captured loop (default; skipped on a device without
- *                 cooperative launches).  0 = the captured loop throughout.
- *                 The results are the same either way.
+ *   "stage_loop"  1 = problems of p <= 128 (not batched) run the whole search in
+ *                 one cooperative kernel, a CTA per node that keeps the node's
+ *                 precision block, the FP32 correlations and the graph in its
+ *                 shared memory; the CTAs exchange the pairs they separated once
+ *                 per stage.  It hands over to the captured loop at the first
+ *                 stage it does not take: a node with more than 16384 tests,
+ *                 direct tests of more than 12 conditioning members, a stage
+ *                 the proposal may score, more FP64 re-decisions than its queue
+ *                 holds, or a stage above the budget (default; skipped on a
+ *                 device without cooperative launches).  0 = the captured loop
+ *                 throughout.  The results are the same either way.
  *   "comp_fp32"   1 = complement tests (reversed order) in FP32 first from the
  *                 FP64 precision blocks, decided there when a first-order
  *                 error bound with validity checks shows the FP64 decision is
@@ -320,11 +320,12 @@ int64_t pc_kernel_launches(void);
  * with CUDA events on its stream, grouped by kernel class: 0 correlation,
  * 1 closed-form stage l=p-2, 2 neighbourhood precision builds and downdates,
  * 3 direct CI tests, 4 complement CI tests, 5 stage bookkeeping (neighbour
- * lists, counts, scans, commit), 6 proposal scoring, ordering and the FP64
+ * lists, counts, scans, commit, the expansion of the skeleton), 6 proposal scoring, ordering and the FP64
  * re-test of the sepsets found in the proposal order, 7 the correlation GEMM
  * kernels alone (the tensor-core product and its split-K reduce, or the SIMT
- * Gram kernel; a part of class 0), 8 the stage loop in one kernel (option
- * "stage_loop": every class of work of the stages it runs).  Writes per-class
+ * Gram kernel; a part of class 0), 8 the search in one kernel (option
+ * "stage_loop": every class of work of the stages it runs, the closed-form one
+ * included).  Writes per-class
  * device milliseconds and launch-group counts accumulated since the last reset
  * (reset != 0 clears them afterwards).  ms and count have 9 entries; either may
  * be NULL. */

@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <cstddef>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -65,7 +66,7 @@ struct pc_handle {
     int lane_chunk = 8, lane_rounds = 32, lane_blocks = 8, direct_warps = 8;
     int node_dmax = fpc::NODE_DMAX;   // staged small-stage kernel: largest node degree (0: off)
     int comp_fp32 = 1;                // complement tests in FP32 first (FP32 modes)
-    int stage_loop = 1;               // reversed order, p <= LOOP_PMAX: complement-only stages in one kernel
+    int stage_loop = 1;               // p <= NL_PMAX: the search in one kernel (node_loop.cu)
     int coop = -1;                    // device supports cooperative launches (-1: not asked yet)
     int pair_warp = 1;                // stages 1-2: warp-per-pair kernel for the larger nodes
     int pair_warp_dmin = fpc::PAIRWARP_DMIN;
@@ -104,8 +105,19 @@ struct pc_handle {
     ull *binom = nullptr;
     double *rq_tab = nullptr;         // per stage l: tanh(q / sqrt(n - l - 3)), the |r| threshold
     long long opair_cap = 0;
-    LevelInfo *info_h = nullptr;     // pinned mirror
-    DevCounters *ctr_h = nullptr;    // pinned mirror
+    // the search's scalars, counters and the GEMM's error flag lie together on the device,
+    // with one pinned mirror: one copy brings them all
+    struct HostView {
+        LevelInfo info;
+        DevCounters ctr;
+        int tc_err;
+    };
+    HostView *view_d = nullptr, *view_h = nullptr;
+    LevelInfo *info_h = nullptr;     // into view_h
+    DevCounters *ctr_h = nullptr;
+    unsigned long long *nl_xch = nullptr;   // exchange words of the one-kernel search
+    bool loop_ran = false;           // the current search started in that kernel
+    uint8_t *adj_early = nullptr;    // device output to expand the skeleton into right behind it
     ull *sepcnt_h = nullptr;
     // orientation (Phase II): arrowhead bitsets, two rounds' worth, and a flag
     uint32_t *or_mk = nullptr;
@@ -356,14 +368,18 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
     A(dalloc(h, &g.prec_mem, (size_t)p * fpc::PREC_MAX * sizeof(int)));
     A(dalloc(h, &g.prec_pos, pp * sizeof(short)));
     A(dalloc(h, &g.prec_need, (size_t)p * sizeof(int)));
-    A(dalloc(h, &g.info, sizeof(LevelInfo)));
-    A(dalloc(h, &g.ctr, sizeof(DevCounters)));
+    A(dalloc(h, &h->view_d, sizeof(pc_handle::HostView)));
+    if (e == cudaSuccess) {
+        g.info = &h->view_d->info;
+        g.ctr = &h->view_d->ctr;
+        h->tc_err = &h->view_d->tc_err;
+    }
+    if (p <= fpc::NL_PMAX && !batch) A(dalloc(h, &h->nl_xch, fpc::node_loop_xch_bytes(p)));
     A(dalloc(h, &h->mean, (size_t)p * sizeof(double)));
     A(dalloc(h, &h->rsd, (size_t)p * sizeof(double)));
     A(dalloc(h, &h->C64, h->c_elems * sizeof(double)));
     A(dalloc(h, &h->C32, h->c_elems * sizeof(float)));
     A(dalloc(h, &h->singular, sizeof(int)));
-    A(dalloc(h, &h->tc_err, sizeof(int)));
     A(dalloc(h, &h->mlp_err, sizeof(int)));
     h->rq_cap = 1ull << 24;
     A(dalloc(h, &h->rq, (size_t)h->rq_cap * sizeof(ull)));
@@ -375,8 +391,11 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
     A(dalloc(h, &h->grad, (size_t)fpc::mlp_nparam() * sizeof(float)));
     A(dalloc(h, &h->wpack, fpc::mlp_pack_bytes()));
     A(dalloc(h, &h->work, (size_t)(2 * p + 16) * sizeof(double)));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&h->info_h, sizeof(LevelInfo));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&h->ctr_h, sizeof(DevCounters));
+    if (e == cudaSuccess) e = cudaMallocHost((void **)&h->view_h, sizeof(pc_handle::HostView));
+    if (e == cudaSuccess) {
+        h->info_h = &h->view_h->info;
+        h->ctr_h = &h->view_h->ctr;
+    }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->br_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev0);
@@ -528,8 +547,7 @@ extern "C" void pc_destroy(pc_handle *h)
         if (cl.s) cudaStreamSynchronize(cl.s);
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
-    if (h->info_h) cudaFreeHost(h->info_h);
-    if (h->ctr_h) cudaFreeHost(h->ctr_h);
+    if (h->view_h) cudaFreeHost(h->view_h);
     if (h->sepcnt_h) cudaFreeHost(h->sepcnt_h);
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
@@ -1042,10 +1060,13 @@ extern "C" pc_status pc_corr_get(pc_handle *h, float *C32, double *C64)
 }
 
 // ---------------------------------------------------------------- skeleton
+// scalars, counters and the GEMM's error flag in one copy
 static pc_status read_info(pc_handle *h)
 {
-    CK(cudaMemcpyAsync(h->info_h, h->g.info, sizeof(LevelInfo), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->view_h, h->view_d, sizeof(pc_handle::HostView), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    if (h->used_tc && h->view_h->tc_err)
+        return fail(h, (pc_status)h->view_h->tc_err, "tensor-core correlation GEMM: a bounded wait expired");
     return PC_OK;
 }
 
@@ -1321,6 +1342,38 @@ static pc_status skeleton_enqueue(pc_handle *h)
         g.rows_cap = 0;
         g.scored = nullptr;
     }
+    // problems of p <= NL_PMAX: the whole search in one kernel, a CTA per node; the captured
+    // loop (or the host loop) goes on from the first stage it does not take
+    h->loop_ran = false;
+    bool loop = h->stage_loop && p <= fpc::NL_PMAX && !h->nblk;
+    if (loop && h->coop < 0) {
+        int dev = 0, v = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&v, cudaDevAttrCooperativeLaunch, dev));
+        h->coop = v;
+    }
+    const bool stage_a = h->order == 1 && h->stage_a && n - p - 1 > 0;
+    if (loop && h->coop) {
+        CK(cudaMemsetAsync(h->view_d, 0, offsetof(pc_handle::HostView, tc_err), s));
+        CK(cudaEventRecord(h->ev0, s));
+        cudaError_t e;
+        {
+            Timed t(h, 8);
+            e = fpc::launch_node_loop(g, tp, h->C32, h->C64, h->ldc, h->Pbuf, h->nl_xch, h->budget, level_cap(h),
+                                      stage_a, s);
+        }
+        if (e != cudaErrorCooperativeLaunchTooLarge) {
+            CK(e);
+            CK(cudaEventRecord(h->ev1, s));
+            if (h->adj_early) {
+                Timed t(h, 5);
+                CK(fpc::launch_expand_adj(g, h->adj_early, s));
+            }
+            h->loop_ran = true;
+            return PC_OK;
+        }
+        cudaGetLastError();                            // not resident: the loop below runs it all
+    }
     if (graph) {
         if (pc_status r = ensure_graph(h)) return r;
     }
@@ -1339,14 +1392,12 @@ static pc_status skeleton_enqueue(pc_handle *h)
     CK(cudaMemsetAsync(h->singular, 0, sizeof(int), s));
     CK(cudaEventRecord(h->ev0, s));
 
-    int stage_a_launched = 0;
     {
         Timed t(h, 5);
         CK(fpc::launch_level_degrees(g, s));
         CK(fpc::launch_tail(g, tp, level_cap(h), 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, s));
     }
-    if (h->order == 1 && h->stage_a && n - p - 1 > 0) {
-        stage_a_launched = 1;
+    if (stage_a) {
         {
             Timed t(h, 1);
             CK(cudaMemcpyAsync(h->Pbuf, h->C64, (size_t)p * h->ldc * sizeof(double),
@@ -1362,39 +1413,13 @@ static pc_status skeleton_enqueue(pc_handle *h)
     }
     {
         Timed t(h, 5);
-        CK(fpc::launch_tail(g, tp, level_cap(h), 1, h->singular, stage_a_launched, h->hcond, 0, fpc::StageConds{},
-                            s));
+        CK(fpc::launch_tail(g, tp, level_cap(h), 1, h->singular, stage_a, h->hcond, 0, fpc::StageConds{}, s));
     }
-    // the stage loop in one kernel for small problems (the reversed order's precision
-    // blocks, when it has them, included)
-    bool loop = h->stage_loop && p <= fpc::LOOP_PMAX && !h->nblk;
-    if (loop && h->coop < 0) {
-        int dev = 0, v = 0;
-        CK(cudaGetDevice(&dev));
-        CK(cudaDeviceGetAttribute(&v, cudaDevAttrCooperativeLaunch, dev));
-        h->coop = v;
-    }
-    loop = loop && h->coop;
     if (h->order == 1 && h->complement) {
         Timed t(h, 2);
         // after the closed-form stage: blocks from its inverse, then one downdate each
-        // (in the stage loop kernel when it runs)
-        if (stage_a_launched && p <= fpc::PREC_MAX) CK(fpc::launch_prec_seed(g, h->Pbuf, h->ldc, s));
-        if (!loop) CK(fpc::launch_prec_update(g, tp, h->C64, h->ldc, s));
-    }
-    if (loop) {
-        // the first blocks and the stages in one cooperative kernel; the captured loop (or
-        // the host loop) goes on from the first stage the kernel does not take
-        const bool blocks = h->order == 1 && h->complement;
-        Timed t(h, 8);
-        cudaError_t e = fpc::launch_stage_loop(g, tp, h->C32, h->C64, h->ldc, h->budget, level_cap(h),
-                                               blocks ? 1 : 0, s);
-        if (e == cudaErrorCooperativeLaunchTooLarge) {
-            cudaGetLastError();                        // not resident: the captured loop runs it all
-            if (blocks) CK(fpc::launch_prec_update(g, tp, h->C64, h->ldc, s));
-        } else {
-            CK(e);
-        }
+        if (stage_a && p <= fpc::PREC_MAX) CK(fpc::launch_prec_seed(g, h->Pbuf, h->ldc, s));
+        CK(fpc::launch_prec_update(g, tp, h->C64, h->ldc, s));
     }
 
     if (graph) CK(cudaGraphLaunch(h->gexec, s));
@@ -1411,10 +1436,15 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
     *overflow = false;
     const bool timed = h->timing != 0;
     const bool graph = h->use_graph && !timed;
-    // the stage loop
+    // the stage loop; more: work was issued after the first driver's
+    bool more = false;
     for (int guard_iter = 0; guard_iter < 4 * p + 16; ++guard_iter) {
         if (graph) {
-            if (guard_iter > 0) CK(cudaGraphLaunch(h->gexec, s));
+            if (guard_iter > 0) {
+                if (pc_status r = ensure_graph(h)) return r;
+                CK(cudaGraphLaunch(h->gexec, s));
+                more = true;
+            }
             if (pc_status r = read_info(h)) return r;
         } else {
             if (pc_status r = read_info(h)) return r;
@@ -1427,6 +1457,7 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
                     mmax = fpc::DIRECT_MMAX;
                 }
                 if (pc_status r = enqueue_level(h, s, mmax, false, timed)) return r;
+                more = true;
                 continue;
             }
         }
@@ -1435,6 +1466,8 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
             *overflow = true;
             return PC_OK;
         }
+        if (I.error == PC_ERR_TIMEOUT)
+            return fail(h, PC_ERR_TIMEOUT, "skeleton search: a bounded wait between its CTAs expired");
         if (I.error) {
             return fail(h, (pc_status)I.error,
                         "stage l=" + std::to_string(I.l) + " schedules " +
@@ -1453,19 +1486,25 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
                                 std::to_string(fpc::DIRECT_MMAX) + "); use the conventional order");
             if (pc_status r = clear_halt(h)) return r;
             if (pc_status r = enqueue_level(h, s, I.l + 2, false, timed)) return r;
+            more = true;
         }
     }
-    CK(cudaEventRecord(h->ev1, s));
+    if (!h->loop_ran || more) {
+        CK(cudaEventRecord(h->ev1, s));
+        if (h->adj_early) {
+            Timed t(h, 5);
+            CK(fpc::launch_expand_adj(g, h->adj_early, s));
+        }
+    }
     if (h->learned && h->learned_lmax >= 1) {
         // largest stage run: the first one in the reversed order, the last one conventionally
         Timed tm(h, h->timing ? 6 : -1);
         const int lmax = h->order == 1 ? h->info_h->first_level : h->info_h->l - 1;
         CK(fpc::launch_reverify(g, tp, h->C32, h->C64, h->ldc, lmax, s));
     }
-    if (pc_status r = read_info(h)) return r;
+    if (!h->loop_ran || more || h->learned)
+        if (pc_status r = read_info(h)) return r;
     if (!h->info_h->done) return fail(h, PC_ERR_INTERNAL, "stage loop did not finish");
-    CK(cudaMemcpyAsync(h->ctr_h, g.ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     const DevCounters &c = *h->ctr_h;
     const LevelInfo &I = *h->info_h;
     // the captured body counts the kernels its conditional nodes actually ran
@@ -1763,14 +1802,23 @@ extern "C" pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats
 {
     if (!h) return PC_ERR_ARG;
     if (!h->have_corr) return fail(h, PC_ERR_STATE, "pc_skeleton before pc_corr");
-    if (pc_status r = check_tc(h)) return r;
     pc_stats st;
-    pc_status r = h->path_pool ? skeleton_pathpool(h, &st) : skeleton_run(h, &st);
+    pc_status r;
+    // a device output is expanded right behind the search, before its one wait
+    const bool early = adj_out && !h->path_pool && is_device_ptr(adj_out);
+    if (h->path_pool) {
+        if (pc_status c = check_tc(h)) return c;
+        r = skeleton_pathpool(h, &st);
+    } else {
+        h->adj_early = early ? adj_out : nullptr;
+        r = skeleton_run(h, &st);
+        h->adj_early = nullptr;
+    }
     if (r != PC_OK) return r;
     h->last = st;
     h->have_skel = true;
     if (stats) *stats = st;
-    if (adj_out) return copy_adj(h, adj_out);
+    if (adj_out && !early) return copy_adj(h, adj_out);
     return PC_OK;
 }
 
@@ -1780,6 +1828,7 @@ static pc_status copy_adj(pc_handle *h, uint8_t *adj_out)
 {
     const size_t bytes = (size_t)h->p * h->p;
     cudaStream_t s = h->stream;
+    Timed t(h, 5);
     if (is_device_ptr(adj_out)) {
         CK(fpc::launch_expand_adj(h->g, adj_out, s));
     } else {

@@ -18,20 +18,13 @@
 //               the sequential canonical order
 #include "internal.h"
 #include "device_util.cuh"
+#include "ci_test.cuh"
 #include <algorithm>
 #include <cooperative_groups.h>
 
 namespace fpc {
 
 namespace cg = cooperative_groups;
-
-typedef unsigned long long ull;
-
-__device__ __forceinline__ ull sat_add(ull a, ull b)
-{
-    ull c = a + b;
-    return c < a ? KEY_NONE : c;
-}
 
 
 // small-stage kernel instantiation that runs stage l (l <= LANE_LMAX)
@@ -40,22 +33,6 @@ __host__ __device__ __forceinline__ int lane_range_of_dev(int l)
     return l <= 2 ? 0 : (l <= 4 ? 1 : (l <= 6 ? 2 : (l <= 8 ? 3 : (l <= 10 ? 4 : 5))));
 }
 int lane_range_of(int l) { return lane_range_of_dev(l); }
-
-// samples behind the tests of node u (batched problems: its instance's n)
-__device__ __forceinline__ long long n_of(const TestParams &tp, int u)
-{
-    return tp.nvec ? __ldg(tp.nvec + u) : tp.n;
-}
-
-// node u has tests at stage l only while n_u - l - 3 > 0 (one problem: the
-// stage cap n - 4 already ensures it; batched problems differ in n)
-__device__ __forceinline__ bool dof_ok(const TestParams &tp, int u, int l)
-{
-    return !tp.nvec || n_of(tp, u) - l - 3 > 0;
-}
-
-// the stage loop has finished or has been halted: nothing to do
-__device__ __forceinline__ bool stopped(const LevelInfo *I) { return I->done || I->halt; }
 
 // ---------------------------------------------------------------- frozen graph
 // The complete graph (Algorithm 1/2 input): every bit v != u of row u set.
@@ -82,16 +59,15 @@ __global__ void init_adj_kernel(GraphDev g)
 
 // Degrees and ascending neighbour lists of the current graph, one warp per node.
 // Frozen neighbour list (ascending) and degree of node u from its adjacency row, by
-// the calling warp.  l2: read the row through L2 (words other CTAs of the running
-// kernel cleared with atomics).
-__device__ __forceinline__ void node_degree(const GraphDev &g, int u, int lane, bool l2)
+// the calling warp.
+__device__ __forceinline__ void node_degree(const GraphDev &g, int u, int lane)
 {
-    const int old = lane == 0 ? (l2 ? __ldcg(g.deg + u) : g.deg[u]) : 0;
+    const int old = lane == 0 ? g.deg[u] : 0;
     const uint32_t *row = g.adj + (long long)u * g.W;
     int base = 0;
     for (int w0 = 0; w0 < g.W; w0 += 32) {
         const int w = w0 + lane;
-        uint32_t bits = (w < g.W) ? (l2 ? __ldcg(row + w) : row[w]) : 0u;
+        uint32_t bits = (w < g.W) ? row[w] : 0u;
         const int c = __popc(bits);
         int incl = c;
         for (int off = 1; off < 32; off <<= 1) {
@@ -117,7 +93,7 @@ __global__ void degrees_kernel(GraphDev g)
     const int lane = threadIdx.x & 31;
     const int u = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     if (u >= g.p || stopped(g.info)) return;
-    node_degree(g, u, lane, false);
+    node_degree(g, u, lane);
 }
 
 __device__ void tail_body(GraphDev g, TestParams tp, int cap, int mode, const int *stagea_singular,
@@ -132,7 +108,7 @@ __global__ void __launch_bounds__(256) degrees_tail_kernel(GraphDev g, TestParam
 {
     const int lane = threadIdx.x & 31;
     const int u = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-    if (u < g.p && !stopped(g.info)) node_degree(g, u, lane, false);
+    if (u < g.p && !stopped(g.info)) node_degree(g, u, lane);
     __shared__ int last;
     __threadfence();
     __syncthreads();
@@ -166,12 +142,6 @@ __device__ __forceinline__ ull node_chunk(const TestParams &tp, ull T, int dg)
 {
     const ull fair = T * (ull)dg / NODE_THREADS;       // T * dg < 2^64: T <= C(127, 12), dg <= 128
     return fair < (ull)tp.lane_chunk ? (fair > 0 ? fair : 1ull) : (ull)tp.lane_chunk;
-}
-
-__device__ __forceinline__ bool comp_eligible(int d, int l, const TestParams &tp)
-{
-    const int k = d - l;
-    return tp.reversed && tp.complement && d >= l && k <= KC_MAX && k < l && d + 2 <= PREC_MAX;
 }
 
 // One CTA after the degrees: ordered-pair offsets, L* = max |adj(u)\{v}|, edge
@@ -589,290 +559,11 @@ __device__ __forceinline__ void locate_test(const GraphDev &g, const ull *noff, 
 
 size_t scan_ws_bytes(long long n) { return 64 + 0 * n; }
 
-// ---------------------------------------------------------------- warp test
-// Cholesky of the leading l x l block of the (l+2) x (l+2) lower triangle M
-// (row stride ms; order S..., u, v).  Lanes own rows.  After l steps the
-// trailing 2x2 holds H = H0 - H1 H2^{-1} H1^T (Sec. 4).  pmin is the smallest
-// of the l pivots (conditional variances of S_k given S_1..S_{k-1}), h11, h22.
-// bad: a pivot, h11 or h22 <= DEGEN (the FP64 degeneracy rule) or not finite.
-template <typename T>
-__device__ __forceinline__ void warp_chol_test(T *M, int m, int ms, int l, T &r, T &pmin, bool &bad)
-{
-    const int lane = threadIdx.x & 31;
-    pmin = (T)1e30;
-    bad = false;
-    for (int k = 0; k < l; ++k) {
-        const T piv = M[k * ms + k];
-        pmin = piv < pmin ? piv : pmin;
-        if (!(piv > (T)DEGEN)) {
-            bad = true;
-            break;
-        }
-        const T rl = (T)1 / sqrt(piv);
-        for (int i = k + 1 + lane; i < m; i += 32) M[i * ms + k] *= rl;
-        __syncwarp();
-        for (int i = k + 1 + lane; i < m; i += 32) {
-            const T lik = M[i * ms + k];
-            for (int c = k + 1; c <= i; ++c) M[i * ms + c] -= lik * M[c * ms + k];
-        }
-        __syncwarp();
-    }
-    if (bad) {
-        r = (T)0;
-        return;
-    }
-    const T h11 = M[l * ms + l], h22 = M[(l + 1) * ms + l + 1], h12 = M[(l + 1) * ms + l];
-    pmin = h11 < pmin ? h11 : pmin;
-    pmin = h22 < pmin ? h22 : pmin;
-    if (!(h11 > (T)DEGEN) || !(h22 > (T)DEGEN)) {
-        bad = true;
-        r = (T)0;
-        return;
-    }
-    r = h12 / sqrt(h11 * h22);
-}
-
-struct WarpAcc {
-    ull tests, red, band, guard, degen, fl32, fl64;
-    float maxdz;
-};
-
 // per-thread counters of the small-stage kernel (32-bit: a thread runs far fewer
 // than 2^32 tests of one stage); its FP32 flops are tests x F(L), formed at the end
 struct LaneAcc {
     unsigned tests, band, guard;
 };
-
-__device__ __forceinline__ ull flops_direct(int l)
-{
-    ull L = (ull)l;
-    return (L * L * L) / 3 + 2 * L * L + 6 * L + 10;
-}
-
-// Fills the FP64 correlations the lower triangle of corr[nd, nd] needs (lazy
-// mode): every missing entry is computed once by a whole warp -- lane t sums
-// samples t, t+32, ... in order, a fixed butterfly adds the lanes -- and
-// published with a fence before its flag, so racing warps write equal values.
-__device__ __noinline__ void ensure_c64(const int *nd, int m, const TestParams &tp, double *C64, int ldc)
-{
-    const int lane = threadIdx.x & 31;
-    const int ne = m * (m + 1) / 2;
-    volatile unsigned char *valid = tp.c64_valid;
-    for (int e0 = 0; e0 < ne; e0 += 32) {
-        const int e = e0 + lane;
-        bool miss = false;
-        int a = 0, b = 0;
-        if (e < ne) {
-            int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-            while (i * (i + 1) / 2 > e) --i;
-            while ((i + 1) * (i + 2) / 2 <= e) ++i;
-            const int c = e - i * (i + 1) / 2;
-            a = nd[i];
-            b = nd[c];
-            miss = a != b && valid[cidx(tp.prow, tp.p, a, b)] != 1;
-        }
-        unsigned bal = __ballot_sync(0xffffffffu, miss);
-        while (bal) {
-            const int src = __ffs(bal) - 1;
-            const int aa = __shfl_sync(0xffffffffu, a, src), bb = __shfl_sync(0xffffffffu, b, src);
-            const double *xa = tp.xs64 + (long long)aa * tp.ldk, *xb = tp.xs64 + (long long)bb * tp.ldk;
-            const long long na = n_of(tp, aa);
-            // rows start 512-byte aligned (ldk is a multiple of 64): 16-byte loads,
-            // four independent FMA chains per lane
-            const double2 *xa2 = (const double2 *)xa, *xb2 = (const double2 *)xb;
-            const long long nh = na >> 1;
-            double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
-            long long t = lane;
-            for (; t + 32 < nh; t += 64) {
-                const double2 a0 = __ldg(xa2 + t), b0 = __ldg(xb2 + t);
-                const double2 a1 = __ldg(xa2 + t + 32), b1 = __ldg(xb2 + t + 32);
-                acc0 = fma(a0.x, b0.x, acc0);
-                acc1 = fma(a0.y, b0.y, acc1);
-                acc2 = fma(a1.x, b1.x, acc2);
-                acc3 = fma(a1.y, b1.y, acc3);
-            }
-            if (t < nh) {
-                const double2 a0 = __ldg(xa2 + t), b0 = __ldg(xb2 + t);
-                acc0 = fma(a0.x, b0.x, acc0);
-                acc1 = fma(a0.y, b0.y, acc1);
-            }
-            if ((na & 1) && lane == 0) acc0 = fma(xa[na - 1], xb[na - 1], acc0);
-            double acc = (acc0 + acc1) + (acc2 + acc3);
-            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (lane == 0) {
-                const double v = acc / (double)na;
-                C64[cidx(tp.prow, ldc, aa, bb)] = v;
-                C64[cidx(tp.prow, ldc, bb, aa)] = v;
-                __threadfence();
-                valid[cidx(tp.prow, tp.p, aa, bb)] = 1;
-                valid[cidx(tp.prow, tp.p, bb, aa)] = 1;
-            }
-            bal &= bal - 1;
-        }
-        __syncwarp();
-    }
-    __threadfence_block();
-    __syncwarp();
-}
-
-// ---------------------------------------------------------------- FP32 trust rule
-// The FP32 trailing block (h11, h12, h22) of a test is the exact Schur
-// complement of corr + E, where E holds the correlation step's entry errors
-// (|E_ij| <= eps_c) and the backward error of the FP32 factorisation (every
-// row of the Cholesky factor of a correlation matrix has unit norm, so each
-// entry of that backward error is below a few m eps32; 4 m eps32 is taken).
-// With b_u = corr_SS^{-1} corr_Su and b_v the regression coefficients of u
-// and v on S, to first order in eps = eps_c + 4 m eps32
-//   |dh12| <= eps A_u A_v,  |dh11| <= eps A_u^2,  |dh22| <= eps A_v^2,
-//   A_u = 1 + |b_u|_1,  A_v = 1 + |b_v|_1,
-// hence |dr| <= eps (A_u A_v / sqrt(h11 h22) + |r|/2 (A_u^2/h11 + A_v^2/h22)).
-// The expansion is used only while eps A_u^2/h11, eps A_v^2/h22 and
-// m eps |corr_SS^{-1}| (kap) stay below 0.05, and the bound is doubled to
-// cover the higher-order terms and the rounding of the final ratio.  A test
-// is trusted when |r| clears the threshold r_q = tanh(q / sqrt(n-l-3)) by
-// more than that bound (then the FP64 decision of Eq. 1 is the same) and the
-// statistic lies at least `band` from q; otherwise it is re-decided in FP64.
-// Returns 0 trusted, 1 band (re-decide), 2 guard (re-decide); dr_out: the bound.
-constexpr float EPS32 = 5.96e-8f;
-
-__device__ __forceinline__ int fp32_trust(const TestParams &tp, int m, float sqf, float rq, float a, float h11,
-                                          float h22, float ih, float Au, float Av, float kap, float &dr_out)
-{
-    const float eps = tp.eps_c + (4.0f * (float)m) * EPS32;
-    const float i11 = __frcp_rn(h11), i22 = __frcp_rn(h22);
-    const float qu = eps * Au * Au * i11, qv = eps * Av * Av * i22;
-    dr_out = INFINITY;
-    if (fmaxf(fmaxf(qu, qv), kap) > 0.05f) return 2;
-    const float dr = 2.0f * eps * (Au * Av * ih + 0.5f * a * (Au * Au * i11 + Av * Av * i22)) + 8.0f * EPS32;
-    dr_out = dr;
-    if (dr > tp.dr_max) return 2;
-    // |z - q| >= sqf |a - rq| / (1 - min(a, rq)^2) (mean-value theorem on atanh)
-    const float gap = fabsf(a - rq), mn = fminf(a, rq);
-    if (gap <= dr || sqf * gap < (float)tp.band * (1.0f - mn * mn)) return 1;
-    return 0;
-}
-
-// l1 norms of the regression coefficients b_u = corr_SS^{-1} corr_Su and b_v
-// from the factor warp_chol_test left in M (column k below the diagonal holds
-// L_ik, the diagonal the pivots L_kk^2, rows l and l+1 hold L^{-1} corr_Su and
-// L^{-1} corr_Sv): back substitution L^T b = y by the warp, column by column.
-// Overwrites the first l entries of rows l and l+1.
-__device__ __forceinline__ void warp_beta_l1(float *M, int ms, int l, float &bu, float &bv)
-{
-    const int lane = threadIdx.x & 31;
-    float *yu = M + (long long)l * ms, *yv = M + (long long)(l + 1) * ms;
-    float su = 0.f, sv = 0.f;
-    for (int k = l - 1; k >= 0; --k) {
-        __syncwarp();
-        const float rl = rsqrtf(M[k * ms + k]);
-        const float b_u = yu[k] * rl, b_v = yv[k] * rl;
-        su += fabsf(b_u);
-        sv += fabsf(b_v);
-        for (int j = lane; j < k; j += 32) {
-            const float lkj = M[k * ms + j];
-            yu[j] -= lkj * b_u;
-            yv[j] -= lkj * b_v;
-        }
-    }
-    __syncwarp();
-    bu = su;
-    bv = sv;
-}
-
-// One CI test for node ids nd[0..m) (S..., u, v) by the calling warp.
-// Returns independent; writes r and z (of the path that decided).
-template <bool F64>
-__device__ __forceinline__ bool warp_test(const int *nd, int m, int l, const float *C32,
-                                          const double *C64, int ldc, const TestParams &tp,
-                                          double sq, float sqf, void *Mbuf, int ms, WarpAcc &acc,
-                                          double &r_out, float &z_out)
-{
-    const int lane = threadIdx.x & 31;
-    bool need64 = F64, indep = false;
-    float zf = 0.f, rf = 0.f;
-    bool f32ok = false;
-    if (!F64) {
-        float *M = (float *)Mbuf;
-        for (int i = 0; i < m; ++i)
-            for (int c = lane; c <= i; c += 32) M[i * ms + c] = C32[cidx(tp.prow, ldc, nd[i], nd[c])];
-        __syncwarp();
-        float pmin;
-        bool bad;
-        warp_chol_test<float>(M, m, ms, l, rf, pmin, bad);
-        __syncwarp();
-        acc.fl32 += flops_direct(l);
-        if (bad || pmin < (float)tp.guard) {
-            need64 = true;
-            ++acc.guard;
-        } else {
-            const float h11 = M[l * ms + l], h22 = M[(l + 1) * ms + l + 1];
-            float bu, bv, dr;
-            warp_beta_l1(M, ms, l, bu, bv);
-            const float ih = rsqrtf(h11 * h22);
-            const float a = fabsf(rf);
-            const float rq = tanhf(tp.qf / sqf);
-            // kap is not formed here (it would need corr_SS^{-1}); the pivot guard
-            // and the two first-order ratios bound the expansion instead
-            const int t = fp32_trust(tp, m, sqf, rq, a, h11, h22, ih, 1.0f + bu, 1.0f + bv, 0.0f, dr);
-            zf = a < 1.0f ? sqf * atanhf(a) : INFINITY;
-            if (t == 2) {
-                need64 = true;
-                ++acc.guard;
-            } else if (t == 1) {
-                need64 = true;
-                ++acc.band;
-            } else {
-                indep = a <= rq;
-                f32ok = true;
-            }
-        }
-    }
-    double r = rf;
-    float z = zf;
-    if (need64) {
-        double *M = (double *)Mbuf;
-        if (tp.lazy) ensure_c64(nd, m, tp, (double *)C64, ldc);
-        for (int i = 0; i < m; ++i)
-            for (int c = lane; c <= i; c += 32) {
-                const long long o = cidx(tp.prow, ldc, nd[i], nd[c]);
-                M[i * ms + c] = tp.lazy ? ((volatile const double *)C64)[o] : C64[o];
-            }
-        __syncwarp();
-        double pmin;
-        bool bad;
-        warp_chol_test<double>(M, m, ms, l, r, pmin, bad);
-        __syncwarp();
-        acc.fl64 += flops_direct(l);
-        if (bad) {
-            indep = true;
-            r = 0.0;
-            z = 0.f;
-            ++acc.degen;
-        } else {
-            double z64 = fabs(r) < 1.0 ? sq * fabs(atanh(r)) : INFINITY;
-            indep = z64 <= tp.q;
-            if (!F64 && isfinite(zf) && zf > 0.f) acc.maxdz = fmaxf(acc.maxdz, (float)fabs(zf - z64));
-            z = (float)z64;
-        }
-        if (!F64) ++acc.red;
-    }
-    (void)f32ok;
-    r_out = r;
-    z_out = z;
-    return indep;
-}
-
-__device__ __forceinline__ void flush_acc(const WarpAcc &acc, DevCounters *ctr)
-{
-    if (acc.tests) atomicAdd(&ctr->tests_executed, acc.tests);
-    if (acc.red) atomicAdd(&ctr->redecided, acc.red);
-    if (acc.band) atomicAdd(&ctr->band_hits, acc.band);
-    if (acc.guard) atomicAdd(&ctr->guard_hits, acc.guard);
-    if (acc.degen) atomicAdd(&ctr->degenerate, acc.degen);
-    if (acc.fl32) atomicAdd(&ctr->flops, acc.fl32);
-    if (acc.fl64) atomicAdd(&ctr->flops64_direct, acc.fl64);
-    if (acc.maxdz > 0.f) atomic_max_float_pos(&ctr->max_dz_bits, acc.maxdz);
-}
 
 // Candidate position x of the ordered pair (u, j) (d candidates) -> node id:
 // position x of adj(u)\{v} in ascending order (v sits at index j of nbr[u]), or
@@ -961,57 +652,6 @@ __global__ void __launch_bounds__(256) ci_direct_kernel(GraphDev g, TestParams t
     if (lane == 0) flush_acc(acc, g.ctr);
 }
 
-
-// bytes of one warp's buffer in the stage loop's direct tests: the FP64 matrix of
-// LOOP_MMAX x (LOOP_MMAX + 1) and the member and position lists
-__host__ __device__ constexpr size_t loop_direct_bytes()
-{
-    return ((size_t)LOOP_MMAX * (LOOP_MMAX + 1) * sizeof(double) + 2 * LOOP_MMAX * sizeof(int) + 15) / 16 * 16;
-}
-
-// The stage loop's direct tests of a small stage (l + 2 <= LOOP_MMAX): one warp per
-// test as ci_direct_kernel, located by the CTA's own plan (doff: per-node offsets in
-// shared memory, doff[p] = their total); mine: the warp's buffer of loop_direct_bytes.
-template <bool F64>
-__device__ __noinline__ void loop_direct_body(const GraphDev &g, const TestParams &tp, int l, const ull *doff,
-                                              const float *C32, const double *C64, int ldc, unsigned char *mine)
-{
-    const int lane = threadIdx.x & 31;
-    const int m = l + 2, ms = LOOP_MMAX + 1;
-    double *Mbuf = (double *)mine;
-    int *nd = (int *)(mine + (size_t)LOOP_MMAX * ms * sizeof(double));
-    int *pos = nd + LOOP_MMAX;
-    const ull total = doff[g.p];
-    const long long gw = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const double sq = sqrt((double)(tp.n - l - 3));
-    const float sqf = (float)sq;
-    WarpAcc acc = {0, 0, 0, 0, 0, 0, 0, 0.f};
-    for (ull t = gw; t < total; t += nw) {
-        int u, j, d;
-        ull rank;
-        locate_test(g, doff, l, t, u, j, d, rank);
-        const int v = g.nbr[nidx(g, u) + j];
-        const int side = u > v;
-        const ull key = ((ull)side << 62) | rank;
-        ull *bp = g.best + pidx(g, min(u, v), max(u, v));
-        if (*(volatile ull *)bp < key) continue;   // an earlier set already separates
-        if (lane == 0) {
-            unrank_lex(rank, d, l, g.binom, g.ldb, pos);
-            for (int i = 0; i < l; ++i) nd[i] = g.nbr[nidx(g, u) + pos[i] + (pos[i] >= j)];
-            nd[l] = u;
-            nd[l + 1] = v;
-        }
-        __syncwarp();
-        double r;
-        float z;
-        ++acc.tests;
-        const bool ind = warp_test<F64>(nd, m, l, C32, C64, ldc, tp, sq, sqf, Mbuf, ms, acc, r, z);
-        if (ind && lane == 0) atomicMin(bp, key);
-        __syncwarp();
-    }
-    if (lane == 0) flush_acc(acc, g.ctr);
-}
 
 // ---------------------------------------------------------------- direct path, small stages
 // One thread per chunk of tp.lane_chunk consecutive sets of one ordered pair
@@ -1956,25 +1596,18 @@ constexpr int COMP_OFF_MAX = 2048;    // per-node offsets staged in shared memor
 // The complement tests of CTA `cta` of `ncta`.  sb: the unranking table (loaded by
 // the caller); soff: shared room for soff_cap per-node test offsets, used when they
 // fit (the searches in both are chains of dependent loads).
-// planned: soff already holds this CTA's own copy of the stage's offsets (soff[p] =
-// the total) and the stage is unscored (the stage loop's stages have no direct tests).
-// sdeg, sT: with planned, the degree and C(d, l) of every node (shared), so that a
-// test is located without global loads.
 __device__ __noinline__ void complement_body(const GraphDev &g, const TestParams &tp, const ull *sb, ull *soff,
-                                                int soff_cap, int cta, int ncta, bool planned = false,
-                                                const int *sdeg = nullptr, const ull *sT = nullptr)
+                                                int soff_cap, int cta, int ncta)
 {
-    if (!planned && stopped(g.info)) return;
+    if (stopped(g.info)) return;
     const int l = g.info->l;
-    const bool prop = !planned && stage_prop(g, l);
-    const ull total = planned ? soff[g.p] : g.info->total_comp;
+    const bool prop = stage_prop(g, l);
+    const ull total = g.info->total_comp;
     if ((ull)cta >= total) return;                       // no test reaches this CTA
-    const bool off_sm = planned || g.p < soff_cap;
-    if (!planned) {
-        if (off_sm)
-            for (int i = threadIdx.x; i <= g.p; i += blockDim.x) soff[i] = g.cn_off[i];
-        __syncthreads();
-    }
+    const bool off_sm = g.p < soff_cap;
+    if (off_sm)
+        for (int i = threadIdx.x; i <= g.p; i += blockDim.x) soff[i] = g.cn_off[i];
+    __syncthreads();
     const ull *noff = off_sm ? soff : g.cn_off;
     // |r| threshold of the stage: z <= q  <=>  |r| <= tanh(q / sqrt(n - l - 3)) (from the
     // host's table); tests within a relative 1e-12 of it are decided by z itself, exactly
@@ -1989,18 +1622,9 @@ __device__ __noinline__ void complement_body(const GraphDev &g, const TestParams
     // spreads its FP64 work (the bound of a test) over every SM
     for (ull t = (ull)threadIdx.x * ncta + cta; t < total; t += nthr) {
         int u, j, d;
-        ull rank, T;
-        if (sdeg) {
-            u = (int)(upper_bound_dev(noff, (long long)g.p + 1, t) - 1);
-            d = sdeg[u] - 1;
-            T = sT[u];
-            const ull w = t - noff[u], jj = w / T;
-            j = (int)jj;
-            rank = w - jj * T;
-        } else {
-            locate_test(g, noff, l, t, u, j, d, rank);
-            T = g.binom[(long long)d * g.ldb + l];
-        }
+        ull rank;
+        locate_test(g, noff, l, t, u, j, d, rank);
+        const ull T = g.binom[(long long)d * g.ldb + l];
         const int v = g.nbr[nidx(g, u) + j];
         const int k = d - l;
         const int side = u > v;
@@ -2145,15 +1769,11 @@ constexpr int PREC_SHARE_MIN = 16;    // from this many removals one CTA of the 
 // slot map, so that chunk 0 can retire R (slot map entry -1) at once; members
 // retired earlier are skipped.  A requested block (chunk 0) is built by a
 // symmetric sweep of corr[F,F], F = adj(u) u {u}.
-// Node u, chunk `chunk` of `nchunks` (smd: the dynamic shared memory).  CL: the
-// chunks of a node are one thread-block cluster (the kernel below), which shares
-// a large factor through distributed shared memory and retires R in place; else
-// every chunk with rows factors P_RR itself and prec_retire retires R once every
-// chunk is done.
-template <bool CL>
-// need: the node's build request (-1: read it from the tail's flags in memory).
+// Node u, chunk `chunk` of `nchunks` (smd: the dynamic shared memory); the chunks of a
+// node are one thread-block cluster, which shares a large factor through distributed
+// shared memory and retires R in place.
 __device__ __forceinline__ void prec_body(const GraphDev &g, const TestParams &tp, const double *C64, int ldc, int u,
-                                          int chunk, int nchunks, double *smd, int need = -1)
+                                          int chunk, int nchunks, double *smd)
 {
     if (stopped(g.info)) return;
     __shared__ int mem[PREC_MAX];
@@ -2219,18 +1839,16 @@ __device__ __forceinline__ void prec_body(const GraphDev &g, const TestParams &t
             if (chunk == 0 && threadIdx.x == 0) g.prec_m[u] = -2;
             return;
         }
-        if constexpr (CL) {
-            // every chunk of the node's cluster has read the slot map (the exits above are
-            // the same in all of them): chunk 0 retires R while the others go on
-            cg::this_cluster().sync();
-            if (chunk == 0)
-                for (int i = threadIdx.x; i < nr; i += blockDim.x) g.prec_pos[pidx(g, u, pm[rem[i]])] = -1;
-        }
+        // every chunk of the node's cluster has read the slot map (the exits above are
+        // the same in all of them): chunk 0 retires R while the others go on
+        cg::this_cluster().sync();
+        if (chunk == 0)
+            for (int i = threadIdx.x; i < nr; i += blockDim.x) g.prec_pos[pidx(g, u, pm[rem[i]])] = -1;
         const int per = (nt + nchunks - 1) / nchunks;
         const int t0 = chunk * per, t1 = min(nt, t0 + per);
         // many removals in a cluster: rank 0 factors P_RR and the others copy the factor
         // (distributed shared memory); else every chunk with rows factors it itself
-        const bool share = CL && nr >= PREC_SHARE_MIN;   // the same in every chunk
+        const bool share = nr >= PREC_SHARE_MIN;   // the same in every chunk
         if (!share && t0 >= t1) return;                // no kept rows in this chunk
         // P_RR = L D L^T, right-looking with one barrier per pivot: the trailing update of
         // pivot k reads the unscaled column k (times 1/D_k); column k-1 is scaled to L in
@@ -2281,20 +1899,18 @@ __device__ __forceinline__ void prec_body(const GraphDev &g, const TestParams &t
         }
         __syncthreads();
         }
-        if constexpr (CL) {
-            if (share) {
-                __shared__ int fac_bad;
-                if (chunk == 0 && threadIdx.x == 0) fac_bad = brk;
-                cg::cluster_group cl = cg::this_cluster();
-                cl.sync();                                 // rank 0's factor and flag are ready
-                if (chunk != 0) {
-                    brk = *cl.map_shared_rank(&fac_bad, 0) != 0;
-                    const double *A0 = cl.map_shared_rank(smd, 0);
-                    if (!brk)
-                        for (int e = threadIdx.x; e < nr * nr + nr; e += blockDim.x) smd[e] = A0[e];   // L, then 1/D
-                }
-                cl.sync();                                 // rank 0 keeps its shared memory until every copy is done
+        if (share) {
+            __shared__ int fac_bad;
+            if (chunk == 0 && threadIdx.x == 0) fac_bad = brk;
+            cg::cluster_group cl = cg::this_cluster();
+            cl.sync();                                 // rank 0's factor and flag are ready
+            if (chunk != 0) {
+                brk = *cl.map_shared_rank(&fac_bad, 0) != 0;
+                const double *A0 = cl.map_shared_rank(smd, 0);
+                if (!brk)
+                    for (int e = threadIdx.x; e < nr * nr + nr; e += blockDim.x) smd[e] = A0[e];   // L, then 1/D
             }
+            cl.sync();                                 // rank 0 keeps its shared memory until every copy is done
         }
         if (brk) {
             // P_RR is a principal block of an SPD inverse; a pivot at the floor means the
@@ -2350,7 +1966,7 @@ __device__ __forceinline__ void prec_body(const GraphDev &g, const TestParams &t
             atomicAdd(&g.ctr->flops_prec, (ull)nr * nr * nr / 3 + 2ull * nt * nr * (nr + nt));
         return;
     }
-    if (chunk != 0 || !(need < 0 ? g.prec_need[u] : need)) return;
+    if (chunk != 0 || !g.prec_need[u]) return;
     const int m = g.deg[u] + 1;
     if (threadIdx.x == 0) {
         bad = 0;
@@ -2403,23 +2019,7 @@ __global__ void __cluster_dims__(1, PREC_CHUNKS, 1) __launch_bounds__(512)
     prec_update_kernel(GraphDev g, TestParams tp, const double *C64, int ldc)
 {
     extern __shared__ double smd[];
-    prec_body<true>(g, tp, C64, ldc, blockIdx.x, blockIdx.y, PREC_CHUNKS, smd);
-}
-
-// After prec_body<false> of every chunk: the slots of node u's maintained block
-// whose members the commit deleted leave the slot map (entry -1).  A dropped
-// block (prec_m <= 0) keeps its stale map until it is rebuilt.
-__device__ __forceinline__ void prec_retire(const GraphDev &g, int u)
-{
-    const int m0 = g.prec_m[u];
-    if (m0 <= 0) return;
-    const int *pm = g.prec_mem + (long long)u * PREC_MAX;
-    short *pos = g.prec_pos + pidx(g, u, 0);
-    const uint32_t *row = g.adj + (long long)u * g.W;
-    for (int sl = threadIdx.x; sl < m0; sl += blockDim.x) {
-        const int w = pm[sl];
-        if (w != u && pos[w] >= 0 && !((row[w >> 5] >> (w & 31)) & 1u)) pos[w] = -1;
-    }
+    prec_body(g, tp, C64, ldc, blockIdx.x, blockIdx.y, PREC_CHUNKS, smd);
 }
 
 // The first stage's blocks from the closed-form stage's inverse P = corr^{-1}: node
@@ -2457,10 +2057,8 @@ __global__ void __launch_bounds__(256) prec_seed_kernel(GraphDev g, const double
 // key, and count the tests of the sequential canonical order:
 // key (0, rank) -> rank+1; key (1, rank) -> C(d_u,l) + rank+1; none -> both sides.
 // The commit of CTA `cta` of `ncta` (sb: the small binomial table, loaded).
-// soo: when given, a shared copy of the ordered-pair offsets (p+1 entries): the
-// owner of a pair is found there instead of in the head's owner table.
 __device__ __forceinline__ void commit_body(const GraphDev &g, int l_fixed, int explicit_sets, int count_canonical,
-                                            const ull *sb, int cta, int ncta, const long long *soo = nullptr)
+                                            const ull *sb, int cta, int ncta)
 {
     const int l = l_fixed >= 0 ? l_fixed : g.info->l;
     const bool prop = stage_prop(g, l);
@@ -2478,8 +2076,7 @@ __device__ __forceinline__ void commit_body(const GraphDev &g, int l_fixed, int 
         ull rank = 0, off = 0;
         if (o < nop) {
             // owner node: the head kernel's table inside the stage loop, else a search
-            const int u = soo ? (int)(upper_bound_dev(soo, (long long)p + 1, o) - 1)
-                              : l_fixed < 0 ? g.opu[o] : (int)(upper_bound_dev(g.ooff, (long long)p + 1, o) - 1);
+            const int u = l_fixed < 0 ? g.opu[o] : (int)(upper_bound_dev(g.ooff, (long long)p + 1, o) - 1);
             const int j = (int)(o - g.ooff[u]);
             const int v = g.nbr[nidx(g, u) + j];
             if (u < v) {
@@ -2649,191 +2246,6 @@ __global__ void commit_kernel(GraphDev g, int l_fixed, int explicit_sets, int co
     load_small_binom(g, sb);
     __syncthreads();
     commit_body(g, l_fixed, explicit_sets, count_canonical, sb, blockIdx.x, gridDim.x);
-}
-
-// ---------------------------------------------------------------- stage loop in one kernel
-// Every CTA of the stage loop plans stage l itself, as the head does: the
-// complement and direct tests' per-node offsets in shared memory (soff, sdoff;
-// entry p holds the total).  True when the stage is one for the loop: direct tests
-// only of at most LOOP_MMAX - 2 members and outside the proposal's stages, nothing
-// saturated, within the budget (the captured loop's head reports the others).
-// sh: 64 words of scratch; sdeg, sT receive every node's degree and C(d, l).
-__device__ __forceinline__ bool loop_stage_plan(const GraphDev &g, const TestParams &tp, int l, double budget,
-                                                ull *soff, ull *sh, int *sdeg, ull *sT, ull *sdoff)
-{
-    const int t = threadIdx.x, p = g.p;                // p <= LOOP_PMAX < blockDim.x
-    ull v[2] = {0ull, 0ull};
-    bool sat = false;
-    if (t < p) {
-        const int dg = g.deg[t], d = dg - 1;
-        const ull T = (dg > 0 && d >= l && dof_ok(tp, t, l)) ? g.binom[(long long)d * g.ldb + l] : 0ull;
-        sdeg[t] = dg;
-        sT[t] = T;
-        const ull tot = sat_mul(T, (ull)dg);
-        sat = tot == KEY_NONE;
-        if (T && comp_eligible(d, l, tp) && g.prec_m[t] > 0) v[0] = tot;
-        else v[1] = tot;
-    }
-    const int ssat = __syncthreads_or(sat);
-    ull ex[2], tot[2];
-    block_scan_sat<2>(v, ex, tot, sh);
-    if (t < p) {
-        soff[t] = ex[0];
-        sdoff[t] = ex[1];
-    }
-    if (t == 0) {
-        soff[p] = tot[0];
-        sdoff[p] = tot[1];
-    }
-    __syncthreads();
-    // direct tests only where the warp buffer holds them, where no proposal order could
-    // apply (the captured loop scores such stages), and at most LOOP_DIRECT_ROUNDS per
-    // warp of the grid (larger stages run faster on the small-stage kernels)
-    const ull nwarps = (ull)gridDim.x * (blockDim.x >> 5);
-    const bool direct_ok = tot[1] == 0 || (l + 2 <= LOOP_MMAX && tot[1] <= LOOP_DIRECT_ROUNDS * nwarps &&
-                                           !(g.row_off && l >= 1 && l <= tp.learned_lmax));
-    return !ssat && tot[0] != KEY_NONE && tot[1] != KEY_NONE && direct_ok &&
-           (double)tot[0] + (double)tot[1] <= budget;
-}
-
-// Every CTA of the stage loop forms the tail's results it needs from the degrees
-// of the new frozen graph (stage l just committed): the ordered-pair offsets
-// (soo[p] = their total), and per node the precision-block request for the next
-// stage min(l - 1, L*) (reversed order), as the tail does.  CTA 0's tail writes
-// the same into memory for the captured loop.  sh: 32 words of scratch.
-// Also the list of nodes whose blocks have work this stage (a maintained block whose
-// node lost neighbours, or a build request): sact[0..*nact).
-__device__ __forceinline__ void loop_tail_plan(const GraphDev &g, const TestParams &tp, int l, long long *soo,
-                                               int *sneed, ull *sh, int *sact, int *nact)
-{
-    __shared__ int smx[32];
-    const int t = threadIdx.x, p = g.p, lane = t & 31, w = t >> 5;
-    const int dg = t < p ? __ldcg(g.deg + t) : 0;
-    ull v[1] = {(ull)dg}, ex[1], tot[1];
-    block_scan_sat<1>(v, ex, tot, sh);
-    int mx = dg;
-    for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (lane == 0) smx[w] = mx;
-    if (t < p) soo[t] = (long long)ex[0];
-    if (t == 0) soo[p] = (long long)tot[0];
-    __syncthreads();
-    int lmax = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) lmax = max(lmax, smx[i]);
-    const int nl = min(l - 1, lmax - 1);
-    bool act = false;
-    if (t < p) {
-        const int pm = g.prec_m[t];
-        const int nd = nl >= 0 && dg > 0 && comp_eligible(dg - 1, nl, tp) && (pm == 0 || pm == -2);
-        sneed[t] = nd;
-        act = nd || (pm > 0 && __ldcg(g.dchg + t) != 0);
-    }
-    __syncthreads();                                    // sh free again
-    ull va[1] = {act ? 1ull : 0ull}, exa[1], tota[1];
-    block_scan_sat<1>(va, exa, tota, sh);
-    if (act) sact[exa[0]] = t;
-    if (t == 0) *nact = (int)tota[0];
-    __syncthreads();
-}
-
-// Small problems in the reversed order (Algorithm 2) spend most of a stage on the
-// latency of its launches, not on its tests.  This cooperative kernel runs the
-// stages whose tests all take the complement path, one after the other, with a
-// grid-wide barrier where the captured loop has a kernel boundary:
-//   plan (every CTA: the head's offsets, in its shared memory), complement tests,
-//   the previous stage's retirement of deleted block members | commit (the
-//   owner of a pair found in a shared copy of the pair offsets) | degrees |
-//   tail (CTA 0 into memory; every CTA forms the offsets and block requests it
-//   needs itself) and precision downdates and builds.
-// Stages with direct tests of at most LOOP_MMAX - 2 members run them too, a warp per
-// test beside the complement tests.  It returns at the first stage it does not take
-// (larger direct tests, or stages the proposal may score: the captured loop, whose
-// head recomputes that stage, runs it and the rest), or when the search ends or halts.
-// The exits are taken by all CTAs together: `done` and `halt` are written only in
-// the commit and the last phase (the tail), each followed by a barrier, and every
-// CTA plans the stage from the same data.  The stage l is read once per pass, at
-// its start: the tail moves it on in the last phase.
-// pre: first the first stage's block builds and downdates (the seeded blocks drop
-// their non-neighbours), in place of the cluster kernel.
-__global__ void __launch_bounds__(LOOP_THREADS, 1) stage_loop_kernel(GraphDev g, TestParams tp, const float *C32,
-                                                                     const double *C64, int ldc, double budget,
-                                                                     int cap, int chunks, int pre)
-{
-    cg::grid_group grid = cg::this_grid();
-    extern __shared__ double lsm[];
-    __shared__ ull sb[SB_ROWS * SB_COLS];
-    __shared__ ull soff[LOOP_PMAX + 1];
-    __shared__ ull sh[2 * 32];
-    __shared__ long long soo[LOOP_PMAX + 1];
-    __shared__ int sdeg[LOOP_PMAX];
-    __shared__ ull sT[LOOP_PMAX];
-    __shared__ ull sdoff[LOOP_PMAX + 1];
-    __shared__ int sneed[LOOP_PMAX];
-    __shared__ int sact[LOOP_PMAX];
-    __shared__ int nact;
-    LevelInfo *I = g.info;
-    load_small_binom(g, sb);
-    for (int i = threadIdx.x; i <= g.p; i += blockDim.x) soo[i] = g.ooff[i];   // the first stage's, from the tail
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwg = (int)((gridDim.x * blockDim.x) >> 5);
-    if (pre) {
-        // the tail scheduled the requests; every CTA lists the nodes with block work
-        const int t = threadIdx.x;
-        bool act = false;
-        if (t < g.p) {
-            const int nd = g.prec_need[t], pm = g.prec_m[t];
-            sneed[t] = nd;
-            act = nd || (pm > 0 && g.dchg[t] != 0);
-        }
-        ull va[1] = {act ? 1ull : 0ull}, exa[1], tota[1];
-        block_scan_sat<1>(va, exa, tota, sh);
-        if (act) sact[exa[0]] = t;
-        if (t == 0) nact = (int)tota[0];
-        __syncthreads();
-        const int ch = max(1, min(chunks, (int)gridDim.x / max(1, nact)));
-        for (int item = blockIdx.x; item < nact * ch; item += gridDim.x) {
-            const int u = sact[item / ch];
-            prec_body<false>(g, tp, C64, ldc, u, item % ch, ch, lsm, sneed[u]);
-            __syncthreads();
-        }
-        grid.sync();
-    }
-    for (int it = 0; it <= g.p; ++it) {                 // one pass per stage, at most p stages
-        if (stopped(I)) break;
-        const int lcur = I->l;                          // moved on only by the tail below
-        if (!loop_stage_plan(g, tp, lcur, budget, soff, sh, sdeg, sT, sdoff)) break;
-        if (sdoff[g.p] > 0) {                           // the stage's direct tests, a warp each
-            unsigned char *mine = (unsigned char *)lsm + (size_t)(threadIdx.x >> 5) * loop_direct_bytes();
-            if (tp.precision == 0) loop_direct_body<true>(g, tp, lcur, sdoff, C32, C64, ldc, mine);
-            else loop_direct_body<false>(g, tp, lcur, sdoff, C32, C64, ldc, mine);
-        }
-        complement_body(g, tp, sb, soff, LOOP_PMAX + 1, blockIdx.x, gridDim.x, true, sdeg, sT);
-        // then the previous downdates' deletions leave the slot maps (the complement tests
-        // read only the slots of current neighbours; repeating it is harmless)
-        for (int u = blockIdx.x; u < g.p; u += gridDim.x) prec_retire(g, u);
-        grid.sync();
-        if (!stopped(I)) commit_body(g, -1, 1, 1, sb, blockIdx.x, gridDim.x, soo);
-        grid.sync();
-        if (!stopped(I))
-            for (int u = gw; u < g.p; u += nwg) node_degree(g, u, lane, true);
-        grid.sync();
-        // the tail: CTA 0 in memory (next stage, loop end, offsets, requests), every
-        // CTA for itself what the downdates and the next commit need
-        if (blockIdx.x == 0) tail_body(g, tp, cap, 0, nullptr, 0, 0, 0, StageConds{}, true);
-        loop_tail_plan(g, tp, lcur, soo, sneed, sh, sact, &nact);
-        // the nodes with work only, each node's kept rows over as many CTAs as leave one
-        // item per CTA (up to `chunks`): a CTA's items run one after the other
-        const int ch = max(1, min(chunks, (int)gridDim.x / max(1, nact)));
-        for (int item = blockIdx.x; item < nact * ch; item += gridDim.x) {
-            const int u = sact[item / ch];
-            prec_body<false>(g, tp, C64, ldc, u, item % ch, ch, lsm, sneed[u]);
-            __syncthreads();                            // the body's shared arrays are reused
-        }
-        grid.sync();
-    }
-    // the last stage's deletions, also when the loop ran out of passes (no barrier
-    // needed: nothing else runs in the kernel any more)
-    for (int u = blockIdx.x; u < g.p; u += gridDim.x) prec_retire(g, u);
 }
 
 // ---------------------------------------------------------------- re-verification
@@ -3448,28 +2860,6 @@ cudaError_t launch_prec_seed(GraphDev g, const double *P, int ldp, cudaStream_t 
     if (g.p > PREC_MAX) return cudaErrorInvalidValue;
     prec_seed_kernel<<<g.p, 256, 0, s>>>(g, P, ldp); note_launch();
     return cudaGetLastError();
-}
-
-cudaError_t launch_stage_loop(GraphDev g, TestParams tp, const float *C32, const double *C64, int ldc,
-                              double budget, int cap, int pre, cudaStream_t s)
-{
-    if (g.p > LOOP_PMAX) return cudaErrorInvalidValue;
-    // the downdates' and builds' block, or the direct tests' warp buffers
-    const size_t smem = std::max(prec_smem_bytes(g.p), (size_t)(LOOP_THREADS / 32) * loop_direct_bytes());
-    cudaError_t e = cudaFuncSetAttribute(stage_loop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stage_loop_kernel, LOOP_THREADS, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-    const int grid = num_sms() * std::min(per_sm, 2);   // every CTA resident (cooperative launch)
-    // a node's kept rows over PREC_CHUNKS CTAs (consecutive items: different SMs), so
-    // that the FP64 work of a large downdate is spread
-    int chunks = PREC_CHUNKS;
-    void *args[] = {&g, &tp, (void *)&C32, (void *)&C64, &ldc, &budget, &cap, &chunks, &pre};
-    e = cudaLaunchCooperativeKernel((const void *)stage_loop_kernel, dim3(grid), dim3(LOOP_THREADS), args, smem, s);
-    note_launch();
-    return e;
 }
 
 cudaError_t launch_commit(GraphDev g, long long n_opairs_cap, int l_fixed, int explicit_sets,
