@@ -111,6 +111,7 @@ struct pc_handle {
         LevelInfo info;
         DevCounters ctr;
         int tc_err;
+        int orient[2];               // pc_orient's rounds and error (pinned side only)
     };
     HostView *view_d = nullptr, *view_h = nullptr;
     LevelInfo *info_h = nullptr;     // into view_h
@@ -119,11 +120,11 @@ struct pc_handle {
     bool loop_ran = false;           // the current search started in that kernel
     uint8_t *adj_early = nullptr;    // device output to expand the skeleton into right behind it
     ull *sepcnt_h = nullptr;
-    // orientation (Phase II): arrowhead bitsets, two rounds' worth, and a flag
-    uint32_t *or_mk = nullptr;
-    int *or_changed = nullptr;
+    // orientation (Phase II): arrowhead bitsets, a round's additions and its control words
+    void *or_ws = nullptr;
     int8_t *or_codes = nullptr;
     bool have_skel = false;
+    long long skel_edges = 0;        // of that skeleton
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     pc_stats last{};
     std::vector<void *> allocs;
@@ -1654,6 +1655,7 @@ extern "C" pc_status pc_autotune(pc_handle *h, int32_t reps, pc_tune_result *out
     cudaEventDestroy(e1);
     if (rs != PC_OK) return rs;
     h->have_skel = true;
+    h->skel_edges = (long long)h->last.edges_kept;
     if (out) {
         out->lane_chunk = h->lane_chunk;
         out->lane_rounds = h->lane_rounds;
@@ -1817,6 +1819,7 @@ extern "C" pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats
     if (r != PC_OK) return r;
     h->last = st;
     h->have_skel = true;
+    h->skel_edges = (long long)st.edges_kept;
     if (stats) *stats = st;
     if (adj_out && !early) return copy_adj(h, adj_out);
     return PC_OK;
@@ -1878,6 +1881,7 @@ extern "C" pc_status pc_skeleton_many(pc_handle **hs, int32_t count, uint8_t **a
         if (st[i] == PC_OK) {
             h->last = one;
             h->have_skel = true;
+            h->skel_edges = (long long)one.edges_kept;
             if (adj_out && adj_out[i]) st[i] = copy_adj(h, adj_out[i]);
         }
         if (stats) stats[i] = one;
@@ -1963,34 +1967,22 @@ extern "C" pc_status pc_orient(pc_handle *h, int8_t *codes_out, int32_t *rounds_
     if (!codes_out) return fail(h, PC_ERR_ARG, "pc_orient: codes_out is null");
     cudaStream_t s = h->stream;
     const size_t words = (size_t)h->p * h->g.W;
-    if (!h->or_mk) {
-        CK(dalloc(h, &h->or_mk, 4 * words * sizeof(uint32_t)));
-        CK(dalloc(h, &h->or_changed, sizeof(int)));
-    }
-    uint32_t *ah = h->or_mk, *at = ah + words, *ah2 = at + words, *at2 = ah2 + words;
-    CK(fpc::launch_orient_colliders(h->g, ah, at, s));
-    // each round that changes something adds a mark; there are at most 32 W p marks
-    const long long max_rounds = (long long)words * 32 + 1;
-    int32_t rounds = 0;
-    for (;;) {
-        CK(fpc::launch_orient_round(h->g, ah, at, ah2, at2, h->or_changed, s));
-        int changed = 0;
-        CK(cudaMemcpyAsync(&changed, h->or_changed, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        std::swap(ah, ah2);
-        std::swap(at, at2);
-        if (!changed) break;
-        if (++rounds > max_rounds) return fail(h, PC_ERR_INTERNAL, "pc_orient: rules did not settle");
-    }
+    if (!h->or_ws) CK(dalloc(h, &h->or_ws, fpc::orient_ws_bytes(h->g)));
     const size_t pp = (size_t)h->p * h->p;
     int8_t *dst = codes_out;
     if (!is_device_ptr(codes_out)) {
         if (!h->or_codes) CK(dalloc(h, &h->or_codes, pp));
         dst = h->or_codes;
     }
-    CK(fpc::launch_orient_codes(h->g, ah, at, dst, s));
+    // each round that changes something adds a mark; there are at most 32 W p marks
+    int *ctl = nullptr, *res = h->view_h->orient;
+    CK(fpc::launch_orient(h->g, h->skel_edges, h->or_ws, (long long)words * 32, dst, &ctl, s));
+    CK(cudaMemcpyAsync(res, ctl + 3, sizeof(h->view_h->orient), cudaMemcpyDeviceToHost, s));
     if (dst != codes_out) CK(cudaMemcpyAsync(codes_out, dst, pp, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    if (res[1]) return fail(h, (pc_status)res[1], "pc_orient: a bounded wait between its CTAs expired");
+    const int32_t rounds = res[0];
+    if (rounds > (long long)words * 32) return fail(h, PC_ERR_INTERNAL, "pc_orient: rules did not settle");
     if (rounds_out) *rounds_out = rounds;
     return PC_OK;
 }

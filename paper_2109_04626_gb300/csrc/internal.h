@@ -278,11 +278,10 @@ cudaError_t launch_ci_lane(GraphDev g, TestParams tp, const float *C32, const do
                            int range, bool prop, cudaStream_t s);
 int lane_range_of(int l);
 cudaError_t launch_prec_update(GraphDev g, TestParams tp, const double *C64, int ldc, cudaStream_t s);
-// ---- orientation, Algorithm 1 Phase II (orient.cu): arrowhead bitsets ah/at (p x W)
-cudaError_t launch_orient_colliders(GraphDev g, uint32_t *ah, uint32_t *at, cudaStream_t s);
-cudaError_t launch_orient_round(GraphDev g, const uint32_t *ah, const uint32_t *at, uint32_t *ah2, uint32_t *at2,
-                                int *changed, cudaStream_t s);
-cudaError_t launch_orient_codes(GraphDev g, const uint32_t *ah, const uint32_t *at, int8_t *out, cudaStream_t s);
+// ---- orientation, Algorithm 1 Phase II, in one cooperative kernel (orient.cu)
+size_t orient_ws_bytes(const GraphDev &g);
+cudaError_t launch_orient(GraphDev g, long long edges, void *ws, long long max_rounds, int8_t *out, int **ctl,
+                          cudaStream_t s);
 // degrees of the frozen graph, then (last CTA) the stage tail of mode 0 in the same kernel
 cudaError_t launch_degrees_tail(GraphDev g, TestParams tp, int cap, cudaGraphConditionalHandle hc, int use_cond,
                                 StageConds sc, cudaStream_t s);

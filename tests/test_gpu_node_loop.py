@@ -8,6 +8,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+import oracle                                                            # noqa: E402
 from paper_2109_04626_gb300 import sem                                   # noqa: E402
 from test_gpu_parity import _check_skeleton, _run_gpu, _sem_case, fp     # noqa: E402,F401
 
@@ -54,6 +55,25 @@ def test_duplicate_and_constant_columns(fp):                             # noqa:
     X[:, 11] = 2.5
     _check_skeleton(fp, X, order=1)
     _check_skeleton(fp, X, order=0)
+
+
+@pytest.mark.parametrize("p, prob, cap", [(2, 1.0, -1), (33, 0.2, -1), (128, 0.04, -1), (64, 0.9, 0), (128, 0.5, 0),
+                                          (129, 0.05, -1)])
+def test_orient_small_and_dense(fp, p, prob, cap):                       # noqa: F811
+    """Phase II in one CTA (p <= 128, mean degree <= 16) and on the whole GPU (denser or
+    larger graphs) against the oracle on the same skeleton and sets."""
+    X = _sem_case(900 + p, p, 4000, prob)
+    with fp.PC(X.shape[0], p, 0.01, cap, order=0) as pc:
+        pc.corr(torch.from_numpy(X).cuda())
+        adj, _ = pc.skeleton()
+        seps = pc.sepsets()
+        codes, rounds = pc.orient()
+        dev = torch.empty((p, p), dtype=torch.int8, device="cuda")
+        pc.orient(dev)
+    want, want_rounds = oracle.orient(adj, seps)
+    np.testing.assert_array_equal(codes, want)
+    np.testing.assert_array_equal(dev.cpu().numpy(), want)
+    assert rounds == want_rounds
 
 
 def test_budget_and_repeated_calls(fp):                                  # noqa: F811
