@@ -84,7 +84,10 @@ void pc_destroy(pc_handle *h);
  *   "stage_a"     1 = run the l = p-2 stage in closed form when n-p-1 > 0 (default)
  *   "precision"   0 = FP64 everywhere; 1 = FP32 SIMT correlation GEMM + FP32 tests
  *                 with FP64 re-decision; 2 = split-precision BF16x3 tensor-core
- *                 correlation GEMM + FP32 tests with FP64 re-decision (default)
+ *                 correlation GEMM + FP32 tests with FP64 re-decision (default).
+ *                 0, and 2 in the reversed order or with p <= 128, form all FP64
+ *                 correlations by exact integer products on the tensor cores;
+ *                 2 then rounds them to FP32 for the search
  *   "band"        FP64 re-decision band on |z - q| (default 1e-3)
  *   "guard"       pivot-ratio guard: FP32 tests whose smallest Cholesky pivot is
  *                 below it are re-decided in FP64 (default 1e-3)
@@ -336,7 +339,10 @@ pc_status pc_timing(pc_handle *h, double *ms, int64_t *count, int32_t reset);
  * reserved up front by their own pool or budget, and latency-critical loops
  * in which a cudaMalloc would synchronise the device.  The paper has no
  * counterpart; it computes what pc_corr computes in FP64 (corr = Xs^T Xs / n
- * of the FP64-standardised columns, unit diagonal), with no handle.
+ * of the FP64-standardised columns, unit diagonal), with no handle: exact
+ * integer products on the tensor cores, accumulated in C_out itself.  A product
+ * that could not finish (a bounded wait on the device) leaves NaN off the
+ * diagonal.
  *   X      device pointer, n x p row-major, row stride ld >= p, dtype PC_F32 or
  *          PC_F64 (caller-owned, read only)
  *   C_out  device pointer, p x p row-major FP64, row stride ldc >= p

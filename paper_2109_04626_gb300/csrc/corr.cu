@@ -4,51 +4,14 @@
 #include "internal.h"
 #include <cuda_bf16.h>
 #include <algorithm>
+#include <cooperative_groups.h>
 
 namespace fpc {
 
+namespace cg = cooperative_groups;
+
 template <typename T>
 __device__ __forceinline__ double ld_as_double(const T *p) { return (double)__ldg(p); }
-
-// Column mean and reciprocal population standard deviation, two passes in FP64.
-// Block: 32 columns x 8 row phases; a warp reads 32 consecutive columns of one row.
-template <typename T>
-__global__ void __launch_bounds__(256) col_stats_kernel(const T *__restrict__ X, long long n, int p,
-                                                        long long ld, double *mean, double *rsd)
-{
-    __shared__ double red[8][33];
-    __shared__ double mu_s[32];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int col = blockIdx.x * 32 + tx;
-    const bool ok = col < p;
-    double s = 0.0;
-    if (ok)
-        for (long long t = ty; t < n; t += 8) s += ld_as_double(X + t * ld + col);
-    red[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0) {
-        double a = 0.0;
-        for (int k = 0; k < 8; ++k) a += red[k][tx];
-        mu_s[tx] = a / (double)n;
-    }
-    __syncthreads();
-    const double mu = mu_s[tx];
-    double q = 0.0;
-    if (ok)
-        for (long long t = ty; t < n; t += 8) {
-            double d = ld_as_double(X + t * ld + col) - mu;
-            q += d * d;
-        }
-    red[ty][tx] = q;
-    __syncthreads();
-    if (ty == 0 && ok) {
-        double a = 0.0;
-        for (int k = 0; k < 8; ++k) a += red[k][tx];
-        double var = a / (double)n;
-        mean[col] = mu;
-        rsd[col] = var > 0.0 ? 1.0 / sqrt(var) : 0.0;   // constant column -> zero column
-    }
-}
 
 // Column statistics over row chunks: CTA (column tile, chunk) computes the
 // chunk's count, mean and sum of squared deviations (two passes over the
@@ -192,6 +155,120 @@ __device__ __forceinline__ double f2d(float x)
     if (e == 0u || e == 0xffu) return (double)x;
     const unsigned hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
     return __hiloint2double((int)hi, (int)((b & 7u) << 29));
+}
+
+// Column mean and reciprocal population sd without a workspace (pc_corr_noalloc): a cluster
+// of CS_CLUSTER CTAs per 32 columns splits the rows, and the CTAs' sums meet through
+// distributed shared memory, in a fixed order, between the two passes (the second mostly
+// hits L2).  A lane owns a column.  FP32 input in double-single sums (col_sum_f32_kernel,
+// col_m2_f32_kernel below), FP64 input in FP64.  It also clears what the exact product adds
+// into: C above the diagonal, and its error flag.
+constexpr int CS_CLUSTER = 8, CS_WARPS = 8;
+
+template <typename T>
+__global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WARPS)
+    col_stats_cluster_kernel(const T *__restrict__ X, long long n, int p, long long ld, double *mean, double *rsd,
+                             double *C, long long ldc, int *err)
+{
+    __shared__ double red[CS_WARPS][33];
+    __shared__ double part[2][32];                       // this CTA's sums of the two passes
+    cg::cluster_group cl = cg::this_cluster();
+    const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int col = blockIdx.x * 32 + tx;
+    const bool ok = col < p;
+    const long long r0 = (long long)cl.block_rank() * CS_WARPS + w, step = CS_CLUSTER * CS_WARPS;
+    const T *x = X + (ok ? col : 0);
+    for (int a = blockIdx.x * CS_CLUSTER + (int)cl.block_rank(); a < p; a += gridDim.x * CS_CLUSTER)
+        for (int b = a + 1 + threadIdx.x; b < p; b += blockDim.x) C[(long long)a * ldc + b] = 0.0;
+    if (blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
+    // the warps' values -> the cluster's total, the same in every CTA
+    auto total = [&](double v, int pass) -> double {
+        red[w][tx] = v;
+        __syncthreads();
+        if (w == 0) {
+            double s = 0.0;
+            for (int k = 0; k < CS_WARPS; ++k) s += red[k][tx];
+            part[pass][tx] = s;
+        }
+        cl.sync();
+        double s = 0.0;
+        for (int k = 0; k < CS_CLUSTER; ++k) s += cl.map_shared_rank(&part[pass][0], k)[tx];
+        return s;
+    };
+    double v = 0.0;
+    if constexpr (sizeof(T) == 4) {
+        float hi = 0.f, lo = 0.f;
+        for (long long r = r0; r < n; r += 8 * step) {
+            float f[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                float e;
+                two_sum_f(hi, f[u], hi, e);
+                lo = __fadd_rn(lo, e);
+                if (u & 1) two_sum_f(hi, lo, hi, lo);
+            }
+        }
+        v = f2d(hi) + f2d(lo);
+    } else {
+        double s0 = 0.0, s1 = 0.0;
+        for (long long r = r0; r < n; r += 8 * step) {
+            double f[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; u += 2) {
+                s0 += f[u];
+                s1 += f[u + 1];
+            }
+        }
+        v = s0 + s1;
+    }
+    const double mu = total(v, 0) / (double)n;
+    double m2;
+    if constexpr (sizeof(T) == 4) {
+        const float mh = (float)mu;
+        double Q = 0.0;
+        for (long long r = r0; r < n; r += 8 * step) {
+            float f[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : mh;
+            float hi = 0.f, lo = 0.f, sm = 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {                // (f - mh)^2 exactly, a missing row adds 0
+                float sd, e, ee;
+                two_sum_f(f[u], -mh, sd, e);
+                const float pp = __fmul_rn(sd, sd), pe = __fmaf_rn(sd, sd, -pp);
+                sm = __fadd_rn(sm, __fmaf_rn(e, e, __fmaf_rn(__fmul_rn(2.f, sd), e, pe)));
+                two_sum_f(hi, pp, hi, ee);
+                lo = __fadd_rn(lo, ee);
+            }
+            Q += f2d(hi) + (f2d(lo) + f2d(sm));
+        }
+        const double ml = mu - (double)mh;
+        m2 = total(Q, 1) - (double)n * ml * ml;
+    } else {
+        double q0 = 0.0, q1 = 0.0;
+        for (long long r = r0; r < n; r += 8 * step) {
+            double f[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : mu;
+#pragma unroll
+            for (int u = 0; u < 8; u += 2) {
+                const double d0 = f[u] - mu, d1 = f[u + 1] - mu;
+                q0 = fma(d0, d0, q0);
+                q1 = fma(d1, d1, q1);
+            }
+        }
+        m2 = total(q0 + q1, 1);
+    }
+    if (cl.block_rank() == 0 && w == 0 && ok) {
+        const double var = m2 / (double)n;
+        mean[col] = mu;
+        rsd[col] = var > 0.0 ? 1.0 / sqrt(var) : 0.0;    // constant column -> zero column
+    }
+    cl.sync();                                           // no CTA leaves while another reads its sums
 }
 
 // Work layout of the FP32 statistics passes: CTA (column tile of ST_COLS, row
@@ -728,13 +805,15 @@ cudaError_t launch_cast_block(const double *C64, float *C32, int ldc, int o, int
 }
 
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
-                             double *mean, double *rsd, cudaStream_t s)
+                             double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s)
 {
-    dim3 g((p + 31) / 32);
+    const dim3 g((p + 31) / 32, CS_CLUSTER);
     if (dtype == 1)
-        col_stats_kernel<double><<<g, 256, 0, s>>>((const double *)X, n, p, ld, mean, rsd);
+        col_stats_cluster_kernel<double><<<g, 32 * CS_WARPS, 0, s>>>((const double *)X, n, p, ld, mean, rsd, C,
+                                                                        ldc, err);
     else
-        col_stats_kernel<float><<<g, 256, 0, s>>>((const float *)X, n, p, ld, mean, rsd);
+        col_stats_cluster_kernel<float><<<g, 32 * CS_WARPS, 0, s>>>((const float *)X, n, p, ld, mean, rsd, C,
+                                                                       ldc, err);
     note_launch();
     return cudaGetLastError();
 }

@@ -100,6 +100,17 @@ struct pc_handle {
     size_t Xstage_bytes = 0;
     bool have_corr = false;
     bool used_tc = false;
+    bool c32_rounded = false;        // C32 is the FP32 rounding of full FP64 correlations
+    // pc_ci_batch returns r from the split-precision product: beside a rounded C32 it is
+    // formed on demand, from a copy of X
+    void *Xkeep = nullptr;
+    size_t Xkeep_bytes = 0;
+    const void *keep_x = nullptr;    // Xkeep, or the staging buffer of a host X
+    int keep_dtype = 0;
+    long long keep_ld = 0;
+    unsigned char *c32tc_ws = nullptr;
+    float *C32tc = nullptr;          // into c32tc_ws
+    bool c32tc_valid = false;
     // graph state
     GraphDev g{};
     ull *binom = nullptr;
@@ -286,7 +297,7 @@ static TestParams make_tp(const pc_handle *h)
     tp.rq_tab = h->rq_tab;
     tp.band = h->band;
     tp.guard = h->guard;
-    tp.eps_c = h->used_tc ? 1.0e-6f : 1.2e-7f;
+    tp.eps_c = h->used_tc && !h->c32_rounded ? 1.0e-6f : 1.2e-7f;
     tp.dr_max = 1.0f;            // skeleton: only the decision is returned (no bound on r itself)
     tp.lane_chunk = h->lane_chunk;
     tp.lane_rounds = h->lane_rounds;
@@ -798,6 +809,50 @@ static pc_status alloc_c64_list(pc_handle *h)
     return PC_OK;
 }
 
+// the standardised planes (zero: the padding samples stay so)
+static pc_status alloc_planes(pc_handle *h, cudaStream_t s)
+{
+    const size_t plane = (size_t)h->p * h->ldk;
+    if (!h->Xs64) {
+        CK(dalloc(h, &h->Xs64, plane * sizeof(double)));
+        CK(dalloc(h, &h->Xs32, plane * sizeof(float)));
+        CK(dalloc(h, &h->Xhi, plane * sizeof(uint16_t)));
+        CK(dalloc(h, &h->Xlo, plane * sizeof(uint16_t)));
+        CK(cudaMemsetAsync(h->Xs64, 0, plane * sizeof(double), s));
+        CK(cudaMemsetAsync(h->Xs32, 0, plane * sizeof(float), s));
+        CK(cudaMemsetAsync(h->Xhi, 0, plane * sizeof(uint16_t), s));
+        CK(cudaMemsetAsync(h->Xlo, 0, plane * sizeof(uint16_t), s));
+    }
+    return PC_OK;
+}
+
+// The split-precision product beside a rounded C32, once per pc_corr, for the raw tests.
+// Its planes, workspaces and matrix are one allocation, made at the first such call.
+static pc_status ensure_c32tc(pc_handle *h)
+{
+    if (h->c32tc_valid) return PC_OK;
+    cudaStream_t s = h->stream;
+    const int p = h->p;
+    const size_t plane = (size_t)p * h->ldk * sizeof(uint16_t);
+    const size_t c32 = ((size_t)p * h->ldc * sizeof(float) + 255) / 256 * 256;
+    const size_t sws = (fpc::col_stats_ws_bytes(h->n, p) + 255) / 256 * 256;
+    const size_t tws = fpc::corr_bf16x3_ws_bytes(h->n, p);
+    if (!h->c32tc_ws) {
+        CK(dalloc(h, &h->c32tc_ws, 2 * plane + c32 + sws + tws));
+        CK(cudaMemsetAsync(h->c32tc_ws, 0, 2 * plane, s));    // the padding samples stay zero
+        h->C32tc = (float *)(h->c32tc_ws + 2 * plane);
+    }
+    uint16_t *hi = (uint16_t *)h->c32tc_ws, *lo = (uint16_t *)(h->c32tc_ws + plane);
+    double *st = (double *)(h->c32tc_ws + 2 * plane + c32);
+    float *ws = (float *)(h->c32tc_ws + 2 * plane + c32 + sws);
+    CK(fpc::launch_col_stats_split(h->keep_x, h->keep_dtype, h->n, p, h->keep_ld, h->mean, h->rsd, st, s));
+    CK(fpc::launch_standardize(h->keep_x, h->keep_dtype, h->n, p, h->keep_ld, h->mean, h->rsd, st, nullptr, nullptr,
+                               hi, lo, h->ldk, s));
+    CK(fpc::launch_corr_bf16x3(hi, lo, h->n, h->ldk, p, h->C32tc, h->ldc, ws, tws, h->tc_err, s));
+    h->c32tc_valid = true;
+    return PC_OK;
+}
+
 // Standardisation and correlation GEMM of one problem, or of instance blk of a
 // batched handle (its columns are rows [o, o+p) of the planes, its block of
 // corr the diagonal block there).
@@ -831,18 +886,52 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
         CK(cudaMemcpyAsync(Xstage, X, bytes, cudaMemcpyHostToDevice, s));
         Xd = Xstage;
     }
-    const size_t plane = (size_t)h->p * h->ldk;
-    if (!h->Xs64) {
-        CK(dalloc(h, &h->Xs64, plane * sizeof(double)));
-        CK(dalloc(h, &h->Xs32, plane * sizeof(float)));
-        CK(dalloc(h, &h->Xhi, plane * sizeof(uint16_t)));
-        CK(dalloc(h, &h->Xlo, plane * sizeof(uint16_t)));
-        CK(cudaMemsetAsync(h->Xs64, 0, plane * sizeof(double), s));
-        CK(cudaMemsetAsync(h->Xs32, 0, plane * sizeof(float), s));
-        CK(cudaMemsetAsync(h->Xhi, 0, plane * sizeof(uint16_t), s));
-        CK(cudaMemsetAsync(h->Xlo, 0, plane * sizeof(uint16_t), s));
+    // One problem that needs all FP64 correlations (FP64 tests, the reversed order), or is
+    // small enough that they cost no more than the split-precision product with its planes
+    // and the FP64 entries formed on demand: the exact product from X itself, C32 its
+    // rounding.
+    if (blk < 0 && fpc::tc_gemm_available() &&
+        (h->precision == 0 || (h->precision == 2 && (h->order == 1 || p <= fpc::NL_PMAX)))) {
+        Timed tm(h, 0);
+        if (h->precision == 2) {
+            h->keep_dtype = dtype;
+            h->keep_x = Xd;
+            h->keep_ld = ld;
+            if (Xd == X) {
+                const size_t bytes = (size_t)n * p * esz;
+                if (bytes > h->Xkeep_bytes) {
+                    dfree(h, h->Xkeep);
+                    h->Xkeep = nullptr;
+                    h->Xkeep_bytes = 0;
+                    CK(dalloc(h, &h->Xkeep, bytes));
+                    h->Xkeep_bytes = bytes;
+                }
+                h->keep_x = h->Xkeep;
+                h->keep_ld = p;
+                if (ld == p) CK(cudaMemcpyAsync(h->Xkeep, X, bytes, cudaMemcpyDeviceToDevice, s));
+                else CK(cudaMemcpy2DAsync(h->Xkeep, (size_t)p * esz, X, (size_t)ld * esz, (size_t)p * esz, n,
+                                          cudaMemcpyDeviceToDevice, s));
+            }
+        }
+        h->c32tc_valid = false;
+        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean, h->rsd, h->C64, h->ldc, h->tc_err, s));
+        {
+            Timed tg(h, 7);
+            CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean, h->rsd, h->C64, h->ldc, h->C32, h->ldc,
+                                      h->tc_err, s));
+        }
+        h->used_tc = true;
+        h->c32_rounded = true;
+        h->c64_full = true;
+        if (!h->Pbuf) CK(dalloc(h, &h->Pbuf, (size_t)p * h->ldc * sizeof(double)));
+        h->have_corr = true;
+        h->have_skel = false;
+        return PC_OK;
     }
+    h->c32_rounded = false;
+    if (pc_status r = alloc_planes(h, s)) return r;
     Timed tm(h, lane ? -1 : 0);
+    const size_t po = (size_t)o * h->ldk;                  // first plane row of this problem
     const size_t sws = fpc::col_stats_ws_bytes(n, p);
     if (sws > stats_ws_bytes) {
         dfree(h, stats_ws);
@@ -850,7 +939,6 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
         CK(dalloc(h, &stats_ws, sws));
         stats_ws_bytes = sws;
     }
-    const size_t po = (size_t)o * h->ldk;                  // first plane row of this problem
     CK(fpc::launch_col_stats_split(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, stats_ws, s));
     const bool want_bf16 = h->precision == 2 && fpc::tc_gemm_available();
     CK(fpc::launch_standardize(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, stats_ws, h->Xs64 + po,
@@ -965,17 +1053,7 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
     Timed tm(h, 0);
     // what the instances share, on the handle's stream before the fork: the
     // standardised planes, the FP64-validity flags, the GEMM's error flag
-    const size_t plane = (size_t)h->p * h->ldk;
-    if (!h->Xs64) {
-        CK(dalloc(h, &h->Xs64, plane * sizeof(double)));
-        CK(dalloc(h, &h->Xs32, plane * sizeof(float)));
-        CK(dalloc(h, &h->Xhi, plane * sizeof(uint16_t)));
-        CK(dalloc(h, &h->Xlo, plane * sizeof(uint16_t)));
-        CK(cudaMemsetAsync(h->Xs64, 0, plane * sizeof(double), s));
-        CK(cudaMemsetAsync(h->Xs32, 0, plane * sizeof(float), s));
-        CK(cudaMemsetAsync(h->Xhi, 0, plane * sizeof(uint16_t), s));
-        CK(cudaMemsetAsync(h->Xlo, 0, plane * sizeof(uint16_t), s));
-    }
+    if (pc_status r = alloc_planes(h, s)) return r;
     if (!h->c64_valid) {
         CK(dalloc(h, &h->c64_valid, (h->pair_elems + 7) / 4 * 4));
         CK(cudaMemsetAsync(h->c64_valid, 0, (h->pair_elems + 7) / 4 * 4, s));
@@ -1242,7 +1320,7 @@ static pc_status enqueue_level(pc_handle *h, cudaStream_t s, int mmax, bool use_
 static std::vector<double> graph_key(const pc_handle *h)
 {
     return {(double)h->order, (double)h->complement, (double)h->precision, h->band, h->guard,
-            (double)h->used_tc, (double)h->c64_full, (double)h->learned, (double)(uintptr_t)h->perm, (double)h->rows_cap, h->learned_min, h->learned_ratio, (double)(uintptr_t)h->rq,
+            (double)h->used_tc, (double)h->c32_rounded, (double)h->c64_full, (double)h->learned, (double)(uintptr_t)h->perm, (double)h->rows_cap, h->learned_min, h->learned_ratio, (double)(uintptr_t)h->rq,
             h->budget, (double)level_cap(h), (double)(uintptr_t)h->g.pool, (double)h->g.pool_cap,
             (double)(uintptr_t)h->C32, (double)(uintptr_t)h->C64, (double)h->lane_chunk,
             (double)h->lane_rounds, (double)h->lane_blocks, (double)h->direct_warps, (double)h->stage_conds,
@@ -1999,10 +2077,17 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     if ((h->nblk ? h->n_min : h->n) - l - 3 <= 0) return fail(h, PC_ERR_DOF, "n - l - 3 <= 0");
     if (b == 0) return PC_OK;
     cudaStream_t s = h->stream;
+    // r itself is returned: from the split-precision product, as at every size
+    const float *C32 = h->C32;
+    if (h->c32_rounded && h->precision == 2) {
+        if (pc_status r = ensure_c32tc(h)) return r;
+        C32 = h->C32tc;
+    }
     TestParams tp = make_tp(h);
-    tp.dr_max = 5e-6f;                                   // r itself is returned
+    if (C32 != h->C32) tp.eps_c = 1.0e-6f;
+    tp.dr_max = 5e-6f;
     CK(cudaMemsetAsync(h->g.ctr, 0, sizeof(DevCounters), s));
-    CK(fpc::launch_ci_list(ij, S, l, b, h->C32, h->C64, h->ldc, h->p, tp, r_out, indep_out, z_out,
+    CK(fpc::launch_ci_list(ij, S, l, b, C32, h->C64, h->ldc, h->p, tp, r_out, indep_out, z_out,
                            h->g.ctr, h->g.blk_lo, h->g.blk_hi, s));
     CK(cudaMemcpyAsync(h->ctr_h, h->g.ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

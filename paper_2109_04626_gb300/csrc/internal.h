@@ -219,8 +219,9 @@ struct TestParams {
 void note_launch();
 
 // ---- correlation (corr.cu)
+// without a workspace; also clears C above the diagonal and err for launch_gram_exact
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
-                             double *mean, double *rsd, cudaStream_t s);
+                             double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s);
 cudaError_t launch_col_stats_split(const void *X, int dtype, long long n, int p, long long ld,
                                    double *mean, double *rsd, double *ws, cudaStream_t s);
 size_t col_stats_ws_bytes(long long n, int p);
@@ -233,6 +234,12 @@ cudaError_t launch_standardize(const void *X, int dtype, long long n, int p, lon
 cudaError_t launch_syrk_f64(const double *Xs, long long n, long long ldk, int p, double *C64,
                             int ldc, double *ws, size_t ws_bytes, cudaStream_t s);
 size_t syrk_f64_ws_bytes(long long n, int p);
+// FP64 correlations of X by exact integer products on the tensor cores (gram_exact.cu): C
+// (p x p, fully written), and their FP32 rounding C32 when given; mean, rsd and the cleared
+// C and err as launch_col_stats left them; no workspace
+cudaError_t launch_gram_exact(const void *X, int dtype, long long n, int p, long long ld, const double *mean,
+                              const double *rsd, double *C, long long ldc, float *C32, int ldc32, int *err,
+                              cudaStream_t s);
 cudaError_t launch_syrk_f32(const float *Xs, long long n, long long ldk, int p, float *C32,
                             int ldc, cudaStream_t s);
 cudaError_t launch_c64_lazy_init(double *C64, int ldc, unsigned char *valid, int p, cudaStream_t s);
