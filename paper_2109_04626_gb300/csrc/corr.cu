@@ -2,6 +2,7 @@
 // corr = Xs^T Xs / n (Sec. 4, the matrix corr): FP64 column statistics, FP64
 // and FP32 Gram kernels on the CUDA cores, and the FP64 -> FP32 cast.
 #include "internal.h"
+#include "device_util.cuh"
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cooperative_groups.h>
@@ -141,20 +142,6 @@ __device__ __forceinline__ void dev_split(float x, float mh, float ml, float &sd
     float e;
     two_sum_f(x, -mh, sd, e);
     two_sum_f(e, -ml, dl, dll);
-}
-
-// float -> double without the FP64 pipe: the IEEE-754 binary32 fields moved into
-// binary64 (exponent rebiased by 1023 - 127 = 896, fraction shifted by 52 - 23).
-// Exact for normal numbers and zeros; subnormals, infinities and NaNs take the
-// conversion instruction.
-__device__ __forceinline__ double f2d(float x)
-{
-    const unsigned b = __float_as_uint(x);
-    const unsigned e = (b >> 23) & 0xffu;
-    if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)(b & 0x80000000u), 0);
-    if (e == 0u || e == 0xffu) return (double)x;
-    const unsigned hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
-    return __hiloint2double((int)hi, (int)((b & 7u) << 29));
 }
 
 // Column mean and reciprocal population sd without a workspace (pc_corr_noalloc): a cluster

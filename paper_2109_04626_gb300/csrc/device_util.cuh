@@ -32,6 +32,58 @@ __device__ __forceinline__ double rcp_newton(double v)
     return x;
 }
 
+// float -> double without the FP64 pipe: the IEEE-754 binary32 fields moved into
+// binary64 (exponent rebiased by 1023 - 127 = 896, fraction shifted by 52 - 23).
+// Exact for normal numbers and zeros; subnormals, infinities and NaNs take the
+// conversion instruction.
+__device__ __forceinline__ double f2d(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    const unsigned e = (b >> 23) & 0xffu;
+    if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)(b & 0x80000000u), 0);
+    if (e == 0u || e == 0xffu) return (double)x;
+    const unsigned hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
+    return __hiloint2double((int)hi, (int)((b & 7u) << 29));
+}
+
+// FP64 -> FP32 by rounding the significand in integer registers (the conversion
+// instruction runs on the FP64 pipe).  Values below the FP32 normal range become 0.
+__device__ __forceinline__ float round_f32(double x)
+{
+    const long long b = __double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    if (e <= 0) return __uint_as_float(sign);
+    if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
+    uint32_t v = ((uint32_t)e << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
+    v += (uint32_t)(b >> 28) & 1u;
+    return __uint_as_float(sign | v);
+}
+
+// 1/v and 1/sqrt(v) of a pivot (1e-12 < v < 1e30) with 4 and 7 FP64 instructions: the FP32
+// approximation, conversions in integer registers, and two Newton steps each (relative
+// error 2^-22 -> 2^-43 -> below the FP64 rounding).
+__device__ __forceinline__ double rcp_pivot(double v)
+{
+    float a;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(round_f32(v)));
+    double x = f2d(a);
+    x = fma(x, fma(-v, x, 1.0), x);
+    x = fma(x, fma(-v, x, 1.0), x);
+    return x;
+}
+__device__ __forceinline__ double rsqrt_pivot(double v)
+{
+    double y = f2d(rsqrtf(round_f32(v)));
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double e = fma(-(v * y), y, 1.0);          // 1 - v y^2
+        const double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
+        y = fma(h, e, y);
+    }
+    return y;
+}
+
 // Symmetric sweep of every pivot of an SPD matrix in shared memory:
 // A <- -A^{-1}.  Pivot k is used without row exchanges, so it equals the
 // conditional variance of k given 0..k-1 (the degeneracy test of the oracle's

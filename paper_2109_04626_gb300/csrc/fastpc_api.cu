@@ -2079,13 +2079,15 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     cudaStream_t s = h->stream;
     // r itself is returned: from the split-precision product, as at every size
     const float *C32 = h->C32;
-    if (h->c32_rounded && h->precision == 2) {
-        if (pc_status r = ensure_c32tc(h)) return r;
-        C32 = h->C32tc;
-    }
     TestParams tp = make_tp(h);
-    if (C32 != h->C32) tp.eps_c = 1.0e-6f;
     tp.dr_max = 5e-6f;
+    if (h->c32_rounded && h->precision == 2) {
+        tp.eps_c = 1.0e-6f;
+        if (fpc::ci_list_uses_fp32(l, tp)) {
+            if (pc_status r = ensure_c32tc(h)) return r;
+            C32 = h->C32tc;
+        }
+    }
     CK(cudaMemsetAsync(h->g.ctr, 0, sizeof(DevCounters), s));
     CK(fpc::launch_ci_list(ij, S, l, b, C32, h->C64, h->ldc, h->p, tp, r_out, indep_out, z_out,
                            h->g.ctr, h->g.blk_lo, h->g.blk_hi, s));

@@ -331,6 +331,8 @@ cudaError_t launch_reverify(GraphDev g, TestParams tp, const float *C32, const d
                             cudaStream_t s);
 
 // ---- raw test batches (level.cu)
+// does a batch of l-member sets read C32 (else FP64 throughout)?
+bool ci_list_uses_fp32(int l, const TestParams &tp);
 cudaError_t launch_ci_list(const int *ij, const int *S, int l, long long b, const float *C32,
                            const double *C64, int ldc, int p, TestParams tp, double *r_out,
                            uint8_t *indep_out, float *z_out, DevCounters *ctr, const int *blk_lo,

@@ -21,6 +21,7 @@
 #include "ci_test.cuh"
 #include <algorithm>
 #include <cooperative_groups.h>
+#include <type_traits>
 
 namespace fpc {
 
@@ -2370,6 +2371,326 @@ __global__ void __launch_bounds__(256) ci_list_kernel(const int *ij, const int *
     if (lane == 0) flush_acc(acc, ctr);
 }
 
+// One test per thread (sets of at most LT_MAX members, FP64 correlations all present).
+// FP64 is what bounds a raw batch -- the error bound of 5e-6 on r sends nearly every test
+// with two members or more there -- and GB300 issues an FP64 instruction of a warp every 64
+// clocks of a scheduler whether one lane or 32 are active: a warp per test (lanes on the
+// rows of one small matrix) filled 3 to 6 lanes of each.  A thread factors its own
+// (l+2) x (l+2) matrix row by row; each entry takes its products in the order of
+// warp_chol_test, so the FP32 values are the same bits.  The matrix lives in registers for
+// l <= 4, else in shared memory, entry-major (neighbouring threads on neighbouring
+// words).  Measured, 1 M tests of 3 members at p = 500: 7.4 ms -> 187 us; 50 thousand of 14 at
+// p = 200: 1.62 ms -> 155 us.  From about 24 members on a warp's lanes fill, and the matrix
+// outgrows a thread's share of shared memory: the warp kernel runs those.
+constexpr int LT_MAX = 24;
+
+// Storage of a thread's factor: the packed rows 0..l-1, then the rows of u and v; the FP32
+// factor keeps the pivots on its diagonal and their reciprocal roots behind, the FP64
+// factor (L D L^T) the pivots' reciprocals on its diagonal.
+template <typename T, int N>
+struct RegStore {
+    T a[N > 0 ? N : 1];
+    __device__ __forceinline__ T &operator()(int e) { return a[e]; }
+};
+template <typename T>
+struct SmemStore {                       // one 8-byte cell per entry: both types use the same cells
+    unsigned char *base;
+    int stride;
+    __device__ __forceinline__ T &operator()(int e) { return *(T *)(base + (size_t)e * stride); }
+};
+__host__ __device__ constexpr int lt_cells(int l) { return l * (l + 1) / 2 + 2 * l; }
+__host__ __device__ constexpr int lt_cells32(int l) { return lt_cells(l) + l; }
+
+// FP32: Cholesky of the S block and the trailing 2 x 2, the same operations on the same
+// operands as warp_chol_test, entry by entry.  C(i, j): the correlation of members i and j
+// (order S..., u, v).  false: a pivot, h11 or h22 <= DEGEN.
+template <int LT, class St, class Get>
+__device__ __forceinline__ bool lt_factor32(St &M, const Get &C, int l_rt, float &h11, float &h22, float &h12,
+                                            float &pmin)
+{
+    const int l = LT >= 0 ? LT : l_rt;
+    const int ru = l * (l + 1) / 2, rv = ru + l, rr = rv + l;
+    pmin = 1e30f;
+#pragma unroll
+    for (int i = 0; i < (LT >= 0 ? LT : l); ++i) {
+        const int ri = i * (i + 1) / 2;
+        float d = C(i, i);
+#pragma unroll
+        for (int c = 0; c < i; ++c) {
+            float t = C(i, c);
+#pragma unroll
+            for (int q = 0; q < c; ++q) t = __fmaf_rn(-M(ri + q), M(c * (c + 1) / 2 + q), t);
+            t = __fmul_rn(t, M(rr + c));
+            M(ri + c) = t;
+            d = __fmaf_rn(-t, t, d);
+        }
+        pmin = d < pmin ? d : pmin;
+        if (!(d > (float)DEGEN)) return false;
+        M(ri + i) = d;
+        M(rr + i) = 1.0f / sqrtf(d);
+    }
+    h11 = C(l, l);
+    h22 = C(l + 1, l + 1);
+    h12 = C(l + 1, l);
+#pragma unroll
+    for (int c = 0; c < (LT >= 0 ? LT : l); ++c) {
+        float a = C(l, c), b = C(l + 1, c);
+        const int rc = c * (c + 1) / 2;
+#pragma unroll
+        for (int q = 0; q < c; ++q) {
+            a = __fmaf_rn(-M(ru + q), M(rc + q), a);
+            b = __fmaf_rn(-M(rv + q), M(rc + q), b);
+        }
+        a = __fmul_rn(a, M(rr + c));
+        b = __fmul_rn(b, M(rr + c));
+        M(ru + c) = a;
+        M(rv + c) = b;
+        h11 = __fmaf_rn(-a, a, h11);
+        h12 = __fmaf_rn(-b, a, h12);
+        h22 = __fmaf_rn(-b, b, h22);
+    }
+    pmin = h11 < pmin ? h11 : pmin;
+    pmin = h22 < pmin ? h22 : pmin;
+    return h11 > (float)DEGEN && h22 > (float)DEGEN;
+}
+
+// d > DEGEN without the FP64 pipe: positive finite doubles order as their bits
+__device__ __forceinline__ bool above_floor(double d)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    return b > 0x3d719799812dea11ull && b < 0x7ff0000000000000ull;      // bits of 1e-12; below infinity
+}
+
+// FP64: L D L^T of the S block (the same pivots, no roots: a reciprocal is 4 FP64
+// instructions, a reciprocal root 7) and the trailing 2 x 2.  Two rows at a time: they
+// share the loads of the earlier rows, and their sums are independent chains.
+template <int LT, class St, class Get>
+__device__ __forceinline__ bool lt_factor64(St &M, const Get &C, int l_rt, double &h11, double &h22, double &h12)
+{
+    const int l = LT >= 0 ? LT : l_rt;
+    const int ru = l * (l + 1) / 2, rv = ru + l;
+    // row i against rows c < n: unscaled sums t_ic = C_ic - sum_q t_iq L_cq into M(ri + c)
+    // (and row i2's beside it)
+    auto sums = [&](int i, int i2, int ri, int ri2, int n) {
+#pragma unroll
+        for (int c = 0; c < n; ++c) {
+            double a = C(i, c), b = C(i2, c);
+            const int rc = c * (c + 1) / 2;
+#pragma unroll
+            for (int q = 0; q < c; ++q) {
+                const double x = M(rc + q);
+                a = fma(-M(ri + q), x, a);
+                b = fma(-M(ri2 + q), x, b);
+            }
+            M(ri + c) = a;
+            M(ri2 + c) = b;
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < (LT >= 0 ? LT : l); i += 2) {
+        const int ri = i * (i + 1) / 2, ri2 = ri + i + 1, i2 = i + 1;
+        const bool two = i2 < l;
+        if (two) {
+            sums(i, i2, ri, ri2, i);
+        } else {
+#pragma unroll
+            for (int c = 0; c < i; ++c) {
+                double a = C(i, c);
+                const int rc = c * (c + 1) / 2;
+#pragma unroll
+                for (int q = 0; q < c; ++q) a = fma(-M(ri + q), M(rc + q), a);
+                M(ri + c) = a;
+            }
+        }
+        // row i: L_ic = t_ic / D_c, D_i; row i2's last sum needs row i's L
+        double d = C(i, i), e = two ? C(i2, i) : 0.0;
+#pragma unroll
+        for (int c = 0; c < i; ++c) {
+            const double t = M(ri + c), L = t * M(c * (c + 1) / 2 + c);
+            d = fma(-t, L, d);
+            if (two) e = fma(-M(ri2 + c), L, e);
+            M(ri + c) = L;
+        }
+        if (!above_floor(d)) return false;
+        M(ri + i) = rcp_pivot(d);
+        if (two) {
+            M(ri2 + i) = e;
+            double d2 = C(i2, i2);
+#pragma unroll
+            for (int c = 0; c < i2; ++c) {
+                const double t = M(ri2 + c), L = t * M(c * (c + 1) / 2 + c);
+                d2 = fma(-t, L, d2);
+                M(ri2 + c) = L;
+            }
+            if (!above_floor(d2)) return false;
+            M(ri2 + i2) = rcp_pivot(d2);
+        }
+    }
+    sums(l, l + 1, ru, rv, l);
+    h11 = C(l, l);
+    h22 = C(l + 1, l + 1);
+    h12 = C(l + 1, l);
+#pragma unroll
+    for (int c = 0; c < (LT >= 0 ? LT : l); ++c) {
+        const double a = M(ru + c), b = M(rv + c), rD = M(c * (c + 1) / 2 + c), L = a * rD;
+        h11 = fma(-a, L, h11);
+        h12 = fma(-b, L, h12);
+        h22 = fma(-b, b * rD, h22);
+    }
+    return above_floor(h11) && above_floor(h22);
+}
+
+// sq |atanh r| to about 1e-9 of its value (it is returned as FP32).  atanh r = atanh c +
+// atanh((r - c) / (1 - r c)) with c = tanh(0.34 k), k the nearest by FP32, leaves an
+// argument below 0.17, whose odd Taylor series to the 17th power runs in FP32 beyond its
+// first term (below 1 % of it): 9 FP64 instructions for every lane.  (The library function
+// takes about 60, and one lane of a warp with |r| > 0.17 is enough to pay them: the batch
+// of 1 M tests above ran at 271 us with it there, at 187 without.)
+constexpr int FISHER_K = 19;
+__constant__ double c_fisher[FISHER_K] = {0.0, 0.32747739480870536, 0.5915193954318165, 0.7698665359089004,
+                                          0.8763930674728229, 0.935409070603099, 0.9667472877842368, 0.9830142742967113,
+                                          0.9913585329601762, 0.9956127332865825, 0.9977749279342794, 0.9988721215826155,
+                                          0.9994284385983162, 0.9997103964478165, 0.9998532714367244, 0.9999256621257943,
+                                          0.9999623384790944, 0.9999809198562816, 0.9999903336294768};
+
+__device__ __forceinline__ double lt_fisher(double r, double sq)
+{
+    const double a = fabs(r);
+    const int k = __float2int_rn(atanhf(fminf(round_f32(a), 0.99999f)) * (1.0f / 0.34f));
+    if (k >= FISHER_K) return a < 1.0 ? sq * atanh(a) : INFINITY;
+    const double c = c_fisher[k];
+    const double y = (a - c) * rcp_pivot(fma(-a, c, 1.0));
+    const float g = round_f32(y), x = g * g;
+    float s = 1.0f / 17.0f;
+    s = fmaf(s, x, 1.0f / 15.0f);
+    s = fmaf(s, x, 1.0f / 13.0f);
+    s = fmaf(s, x, 1.0f / 11.0f);
+    s = fmaf(s, x, 1.0f / 9.0f);
+    s = fmaf(s, x, 1.0f / 7.0f);
+    s = fmaf(s, x, 1.0f / 5.0f);
+    s = fmaf(s, x, 1.0f / 3.0f);
+    return sq * (fma(y, f2d(s * x), y) + 0.34 * f2d((float)k));
+}
+
+// f32: FP32 first under the trust rule (warp_test); else FP64 throughout, `skip32` telling
+// why: 0 the FP64 mode, 1 no test of this size can be trusted (counted as guard hits)
+template <int LT>
+__global__ void __launch_bounds__(128) ci_list_thread_kernel(const int *ij, const int *S, int l_rt, long long b,
+                                                             const float *C32, const double *C64, int ldc, int p,
+                                                             TestParams tp, double *r_out, uint8_t *indep_out,
+                                                             float *z_out, DevCounters *ctr, const int *blk_lo,
+                                                             const int *blk_hi, int f32, int skip32)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int l = LT >= 0 ? LT : l_rt, m = l + 2;
+    const int bd = blockDim.x, tid = threadIdx.x;
+    // node ids: registers, or behind the cells
+    int ndr[LT >= 0 ? LT + 2 : 1] = {};
+    unsigned short *nds = (unsigned short *)(smem_raw + (size_t)(f32 ? lt_cells32(l) : lt_cells(l)) * bd * 8) + tid;
+    auto nd = [&](int i) -> int { return LT >= 0 ? ndr[LT >= 0 ? i : 0] : (int)nds[i * bd]; };
+    const double sq0 = sqrt((double)(tp.n - l - 3));
+    WarpAcc acc = {0, 0, 0, 0, 0, 0, 0, 0.f};
+    for (long long t = blockIdx.x * (long long)bd + tid; t < b; t += (long long)gridDim.x * bd) {
+        bool ok = true;
+#pragma unroll
+        for (int i = 0; i < (LT >= 0 ? LT + 2 : m); ++i) {
+            const int x = i < l ? S[t * l + i] : ij[2 * t + (i - l)];
+            ok = ok && x >= 0 && x < p;
+            if (LT >= 0) ndr[LT >= 0 ? i : 0] = x;
+            else nds[i * bd] = (unsigned short)x;             // p <= 32768
+        }
+        const int u = nd(l), v = nd(l + 1);
+        ok = ok && u != v;
+        if (ok && blk_lo) {
+            const int lo = blk_lo[u], hi = blk_hi[u];
+#pragma unroll
+            for (int i = 0; i < (LT >= 0 ? LT + 2 : m); ++i) ok = ok && nd(i) >= lo && nd(i) < hi;
+        }
+        if (!ok) {
+            ctr->status = 1;
+            continue;
+        }
+        ++acc.tests;
+        const double sq = tp.nvec ? sqrt((double)(n_of(tp, u) - l - 3)) : sq0;
+        bool need64 = true, ind = false;
+        double r = 0.0;
+        float z = 0.f;
+        acc.guard += skip32;
+        acc.red += skip32;
+        if (f32) {
+            typename std::conditional<LT >= 0, RegStore<float, lt_cells32(LT >= 0 ? LT : 0)>, SmemStore<float>>::type M;
+            if constexpr (LT < 0) M = {smem_raw + (size_t)tid * 8, bd * 8};
+            float h11, h22, h12, pmin;
+            const bool good = lt_factor32<LT>(
+                M, [&](int i, int c) { return __ldg(C32 + cidx(tp.prow, ldc, nd(i), nd(c))); }, l, h11, h22, h12, pmin);
+            if (!good || pmin < (float)tp.guard) {
+                ++acc.guard;
+            } else {
+                // |b_u|_1, |b_v|_1 by back substitution (warp_beta_l1)
+                const int ru = l * (l + 1) / 2, rv = ru + l;
+                float bu = 0.f, bv = 0.f;
+#pragma unroll
+                for (int k = (LT >= 0 ? LT : l) - 1; k >= 0; --k) {
+                    const int rk = k * (k + 1) / 2;
+                    const float rl = rsqrtf(M(rk + k));
+                    const float b_u = __fmul_rn(M(ru + k), rl), b_v = __fmul_rn(M(rv + k), rl);
+                    bu = __fadd_rn(bu, fabsf(b_u));
+                    bv = __fadd_rn(bv, fabsf(b_v));
+#pragma unroll
+                    for (int j = 0; j < k; ++j) {
+                        M(ru + j) = __fmaf_rn(-M(rk + j), b_u, M(ru + j));
+                        M(rv + j) = __fmaf_rn(-M(rk + j), b_v, M(rv + j));
+                    }
+                }
+                const float rf = h12 / sqrtf(h11 * h22), sqf = (float)sq;
+                const float ih = rsqrtf(h11 * h22), a = fabsf(rf), rq = tanhf(tp.qf / sqf);
+                float dr;
+                const int tr = fp32_trust(tp, m, sqf, rq, a, h11, h22, ih, 1.0f + bu, 1.0f + bv, 0.0f, dr);
+                if (tr == 0) {
+                    need64 = false;
+                    r = (double)rf;
+                    z = a < 1.0f ? sqf * atanhf(a) : INFINITY;
+                    ind = a <= rq;
+                } else if (tr == 1) {
+                    ++acc.band;
+                } else {
+                    ++acc.guard;
+                }
+            }
+            acc.red += need64;
+        }
+        if (need64) {
+            typename std::conditional<LT >= 0, RegStore<double, lt_cells(LT >= 0 ? LT : 0)>, SmemStore<double>>::type M;
+            if constexpr (LT < 0) M = {smem_raw + (size_t)tid * 8, bd * 8};
+            double h11, h22, h12;
+            if (!lt_factor64<LT>(
+                    M, [&](int i, int c) { return __ldg(C64 + cidx(tp.prow, ldc, nd(i), nd(c))); }, l, h11, h22, h12)) {
+                ind = true;
+                ++acc.degen;
+            } else {
+                r = h12 * rsqrt_pivot(h11 * h22);
+                const double z64 = lt_fisher(r, sq);
+                z = round_f32(z64);
+                if (fabsf(z - tp.qf) > 1e-5f * tp.qf) {
+                    ind = z < tp.qf;
+                } else {                                 // the decision on the function itself
+                    const double ze = fabs(r) < 1.0 ? sq * fabs(atanh(r)) : INFINITY;
+                    ind = ze <= tp.q;
+                    z = (float)ze;
+                }
+            }
+        }
+        if (r_out) r_out[t] = r;
+        if (z_out) z_out[t] = z;
+        if (indep_out) indep_out[t] = ind ? 1 : 0;
+    }
+    ull c5[5] = {acc.tests, acc.red, acc.band, acc.guard, acc.degen};
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+        for (int off = 16; off > 0; off >>= 1) c5[k] += __shfl_xor_sync(0xffffffffu, c5[k], off);
+    if ((tid & 31) == 0) flush_acc({c5[0], c5[1], c5[2], c5[3], c5[4], 0, 0, 0.f}, ctr);
+}
+
 // ---------------------------------------------------------------- launchers
 static int g_num_sms = 0;
 static int num_sms()
@@ -2886,11 +3207,55 @@ cudaError_t launch_reverify(GraphDev g, TestParams tp, const float *C32, const d
     return cudaGetLastError();
 }
 
+// Can an FP32 test of l members be trusted at all?  fp32_trust's bound is at least
+// 2 (eps_c + 4 m eps32) + 8 eps32 (A_u, A_v >= 1, h11, h22 <= 1); one part in 1e6 of slack
+// covers its rounding.
+bool ci_list_uses_fp32(int l, const TestParams &tp)
+{
+    const double least = 2.0 * ((double)tp.eps_c + 4.0 * (l + 2) * (double)EPS32) + 8.0 * (double)EPS32;
+    return tp.precision != 0 && least * (1.0 - 1e-6) <= (double)tp.dr_max;
+}
+
+template <int LT>
+static cudaError_t list_thread_launch(const int *ij, const int *S, int l, long long b, const float *C32,
+                                      const double *C64, int ldc, int p, TestParams tp, double *r_out,
+                                      uint8_t *indep_out, float *z_out, DevCounters *ctr, const int *blk_lo,
+                                      const int *blk_hi, cudaStream_t s)
+{
+    const int f32 = ci_list_uses_fp32(l, tp), skip32 = tp.precision != 0 && !f32;
+    // shared memory: a warp per CTA, as many as fit an SM
+    const size_t per = LT >= 0 ? 0 : (size_t)(f32 ? lt_cells32(l) : lt_cells(l)) * 8 + (size_t)(l + 2) * 2;
+    const int threads = LT >= 0 ? 128 : 32;
+    const size_t smem = per * threads;
+    cudaError_t e = cudaFuncSetAttribute(ci_list_thread_kernel<LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    const long long blocks = std::min<long long>((b + threads - 1) / threads, (long long)num_sms() * (LT >= 0 ? 64 : 512));
+    ci_list_thread_kernel<LT><<<(unsigned)blocks, threads, smem, s>>>(ij, S, l, b, C32, C64, ldc, p, tp, r_out,
+                                                                      indep_out, z_out, ctr, blk_lo, blk_hi, f32,
+                                                                      skip32);
+    note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_ci_list(const int *ij, const int *S, int l, long long b, const float *C32,
                            const double *C64, int ldc, int p, TestParams tp, double *r_out,
                            uint8_t *indep_out, float *z_out, DevCounters *ctr, const int *blk_lo,
                            const int *blk_hi, cudaStream_t s)
 {
+    if (l <= LT_MAX && !tp.lazy) {
+        // (with FP64 entries formed on demand a warp forms each missing one)
+#define LT_GO(L) list_thread_launch<L>(ij, S, l, b, C32, C64, ldc, p, tp, r_out, indep_out, z_out, ctr, blk_lo, blk_hi, s)
+        switch (l) {
+        case 0: return LT_GO(0);
+        case 1: return LT_GO(1);
+        case 2: return LT_GO(2);
+        case 3: return LT_GO(3);
+        case 4: return LT_GO(4);
+        default: return LT_GO(-1);
+        }
+#undef LT_GO
+    }
     int ms, per_warp, wpc;
     direct_shape(l + 2, ms, per_warp, wpc);
     size_t smem = (size_t)wpc * per_warp;

@@ -89,22 +89,6 @@ __device__ __forceinline__ int tri_row(int e)
     return r;
 }
 
-// FP64 -> FP32 by rounding the significand in integer registers: the conversion
-// instruction runs on the FP64 pipe, which the block updates need.  Values below the
-// FP32 normal range become 0 (|P_ij| of a precision matrix that small is far below
-// every rounding term of the tests' error bound).
-__device__ __forceinline__ float round_f32(double x)
-{
-    const long long b = __double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
-    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-    if (e <= 0) return __uint_as_float(sign);
-    if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
-    uint32_t v = ((uint32_t)e << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
-    v += (uint32_t)(b >> 28) & 1u;
-    return __uint_as_float(sign | v);
-}
-
 // clocks of dropping a block's members from nl down to nt one by one (two barriers and
 // n^2/2 FMAs at 2 per clock each), and of a sweep build of m members
 __device__ __forceinline__ float drop_clocks(int nt, int nl)
