@@ -165,6 +165,8 @@ struct pc_handle {
     uint8_t *wpack = nullptr;
     int *mlp_err = nullptr;
     double *mlp_loss = nullptr;
+    float *mlp_ws = nullptr;         // the groups' parts of a gradient
+    unsigned char *mlp_h = nullptr;  // pinned mirror of the block at grad
     bool have_params = false;
     int adam_step = 0;
     unsigned long long *row_off = nullptr;
@@ -330,6 +332,9 @@ static TestParams make_tp(const pc_handle *h)
 // ---------------------------------------------------------------- create / destroy
 // pmax: largest problem size (binomial table), batch: block-diagonal batch
 // layout (no precision blocks, conventional order only)
+// bytes of the gradient (padded to 8), the loss (double) and the error flag (with padding)
+static size_t mlp_block_bytes() { return ((size_t)fpc::mlp_nparam() * sizeof(float) + 7) / 8 * 8 + 16; }
+
 static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_level, int32_t pmax,
                              long long pool_cap, bool batch, size_t packed, pc_handle **out)
 {
@@ -392,15 +397,18 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
     A(dalloc(h, &h->C64, h->c_elems * sizeof(double)));
     A(dalloc(h, &h->C32, h->c_elems * sizeof(float)));
     A(dalloc(h, &h->singular, sizeof(int)));
-    A(dalloc(h, &h->mlp_err, sizeof(int)));
     h->rq_cap = 1ull << 24;
     A(dalloc(h, &h->rq, (size_t)h->rq_cap * sizeof(ull)));
     A(dalloc(h, &h->rq_len, sizeof(ull)));
-    A(dalloc(h, &h->mlp_loss, sizeof(double)));
     A(dalloc(h, &h->theta, (size_t)fpc::mlp_nparam() * sizeof(float)));
     A(dalloc(h, &h->adam_m, (size_t)fpc::mlp_nparam() * sizeof(float)));
     A(dalloc(h, &h->adam_v, (size_t)fpc::mlp_nparam() * sizeof(float)));
-    A(dalloc(h, &h->grad, (size_t)fpc::mlp_nparam() * sizeof(float)));
+    // gradient, loss and the network's error flag together: one copy brings them
+    A(dalloc(h, &h->grad, mlp_block_bytes()));
+    if (e == cudaSuccess) {
+        h->mlp_loss = (double *)((char *)h->grad + mlp_block_bytes() - 16);
+        h->mlp_err = (int *)(h->mlp_loss + 1);
+    }
     A(dalloc(h, &h->wpack, fpc::mlp_pack_bytes()));
     A(dalloc(h, &h->work, (size_t)(2 * p + 16) * sizeof(double)));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&h->view_h, sizeof(pc_handle::HostView));
@@ -560,6 +568,7 @@ extern "C" void pc_destroy(pc_handle *h)
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
     if (h->view_h) cudaFreeHost(h->view_h);
+    if (h->mlp_h) cudaFreeHost(h->mlp_h);
     if (h->sepcnt_h) cudaFreeHost(h->sepcnt_h);
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
@@ -2201,38 +2210,58 @@ static void mlp_work_free(pc_handle *h, MlpWork &w)
     dfree(h, w.h1);
 }
 
+// the tensor-core gradient's workspace, kept with the handle
+static pc_status mlp_grad_ws(pc_handle *h)
+{
+    if (!h->mlp_ws) CK(dalloc(h, &h->mlp_ws, fpc::mlp_grad_ws_bytes()));
+    return PC_OK;
+}
+
 extern "C" pc_status pc_mlp_grad(pc_handle *h, const float *feats, const float *labels, int64_t R, float *grad_out,
                                  double *loss)
 {
     if (!h || R <= 0 || !feats || !labels) return PC_ERR_ARG;
     if (!h->have_params) return fail(h, PC_ERR_STATE, "no parameters set");
+    cudaStream_t s = h->stream;
+    const size_t block = mlp_block_bytes(), gbytes = (size_t)fpc::mlp_nparam() * sizeof(float);
+    if (!h->mlp_h) CK(cudaMallocHost((void **)&h->mlp_h, block));
     MlpWork w;
-    pc_status st = mlp_work(h, R, w);
-    if (st == PC_OK) st = mlp_forward(h, feats, R, w.scores, w.h1, w.h2);
-    if (st == PC_OK) {
-        cudaError_t e = cudaMemsetAsync(h->mlp_loss, 0, sizeof(double), h->stream);
-        if (e == cudaSuccess)
-            e = h->mlp_bwd_tc
-                    ? fpc::launch_mlp_backward_tc(feats, labels, w.scores, w.h1, w.h2, R, 1.0f / (float)R, h->theta,
-                                                  h->wpack, h->grad, h->mlp_loss, h->mlp_err, h->stream)
-                    : fpc::launch_mlp_backward(feats, labels, w.scores, w.h1, w.h2, R, 1.0f / (float)R, h->theta,
-                                               h->grad, h->mlp_loss, h->stream);
-        if (e != cudaSuccess) st = cuda_fail(h, e, "pc_mlp_grad");
+    pc_status st = PC_OK;
+    // loss and error flag
+    CK(cudaMemsetAsync(h->mlp_loss, 0, 16, s));
+    if (h->mlp_bwd_tc) {
+        if (pc_status r = mlp_grad_ws(h)) return r;
+        CK(fpc::launch_mlp_grad(feats, labels, R, 1.0f / (float)R, h->theta, h->wpack, h->mlp_ws, h->grad, h->mlp_loss,
+                                h->mlp_err, s));
+    } else {
+        st = mlp_work(h, R, w);
+        if (st == PC_OK) st = mlp_forward(h, feats, R, w.scores, w.h1, w.h2);
+        if (st == PC_OK) {
+            cudaError_t e = fpc::launch_mlp_backward(feats, labels, w.scores, w.h1, w.h2, R, 1.0f / (float)R, h->theta,
+                                                     h->grad, h->mlp_loss, s);
+            if (e != cudaSuccess) st = cuda_fail(h, e, "pc_mlp_grad");
+        }
     }
-    if (st == PC_OK) st = mlp_check_err(h);
-    if (st == PC_OK && grad_out) {
-        cudaError_t e = cudaMemcpy(grad_out, h->grad, (size_t)fpc::mlp_nparam() * sizeof(float), cudaMemcpyDefault);
+    if (st == PC_OK) {
+        cudaError_t e = cudaMemcpyAsync(h->mlp_h, h->grad, block, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && grad_out && is_device_ptr(grad_out))
+            e = cudaMemcpyAsync(grad_out, h->grad, gbytes, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) st = cuda_fail(h, e, "pc_mlp_grad copy");
     }
-    if (st == PC_OK && loss) {
-        double ls = 0;
-        cudaError_t e = cudaMemcpy(&ls, h->mlp_loss, sizeof(double), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) st = cuda_fail(h, e, "pc_mlp_grad loss");
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess && st == PC_OK) st = cuda_fail(h, e, "pc_mlp_grad");
+    mlp_work_free(h, w);
+    if (st != PC_OK) return st;
+    int bad;
+    std::memcpy(&bad, h->mlp_h + block - 8, sizeof(bad));
+    if (bad) return fail(h, (pc_status)bad, "proposal network: a bounded wait of a tensor-core pass expired");
+    if (grad_out && !is_device_ptr(grad_out)) std::memcpy(grad_out, h->mlp_h, gbytes);
+    if (loss) {
+        double ls;
+        std::memcpy(&ls, h->mlp_h + block - 16, sizeof(ls));
         *loss = ls / (double)R;
     }
-    cudaStreamSynchronize(h->stream);
-    mlp_work_free(h, w);
-    return st;
+    return PC_OK;
 }
 
 extern "C" pc_status pc_mlp_train(pc_handle *h, const float *feats, const float *labels, int64_t R, int32_t epochs,
@@ -2242,21 +2271,23 @@ extern "C" pc_status pc_mlp_train(pc_handle *h, const float *feats, const float 
     if (!h->have_params) return fail(h, PC_ERR_STATE, "no parameters set");
     const long long B = std::min<long long>(batch, R);
     MlpWork w;
-    pc_status st = mlp_work(h, B, w);
+    pc_status st = h->mlp_bwd_tc ? mlp_grad_ws(h) : mlp_work(h, B, w);
     cudaStream_t s = h->stream;
     double last = 0.0;
     for (int ep = 0; ep < epochs && st == PC_OK; ++ep) {
-        cudaError_t e = cudaMemsetAsync(h->mlp_loss, 0, sizeof(double), s);
+        // the loss, and once the error flag behind it
+        cudaError_t e = cudaMemsetAsync(h->mlp_loss, 0, ep == 0 ? 16 : sizeof(double), s);
         for (long long b0 = 0; b0 < R && e == cudaSuccess && st == PC_OK; b0 += B) {
             const long long nb = std::min<long long>(B, R - b0);
-            st = mlp_forward(h, feats + b0 * 16, nb, w.scores, w.h1, w.h2);
-            if (st != PC_OK) break;
-            e = h->mlp_bwd_tc
-                    ? fpc::launch_mlp_backward_tc(feats + b0 * 16, labels + b0, w.scores, w.h1, w.h2, nb,
-                                                  1.0f / (float)nb, h->theta, h->wpack, h->grad, h->mlp_loss,
-                                                  h->mlp_err, s)
-                    : fpc::launch_mlp_backward(feats + b0 * 16, labels + b0, w.scores, w.h1, w.h2, nb,
-                                               1.0f / (float)nb, h->theta, h->grad, h->mlp_loss, s);
+            if (h->mlp_bwd_tc) {
+                e = fpc::launch_mlp_grad(feats + b0 * 16, labels + b0, nb, 1.0f / (float)nb, h->theta, h->wpack,
+                                         h->mlp_ws, h->grad, h->mlp_loss, h->mlp_err, s);
+            } else {
+                st = mlp_forward(h, feats + b0 * 16, nb, w.scores, w.h1, w.h2);
+                if (st != PC_OK) break;
+                e = fpc::launch_mlp_backward(feats + b0 * 16, labels + b0, w.scores, w.h1, w.h2, nb, 1.0f / (float)nb,
+                                             h->theta, h->grad, h->mlp_loss, s);
+            }
             if (e == cudaSuccess) e = fpc::launch_adam(h->theta, h->grad, h->adam_m, h->adam_v, (float)lr, ++h->adam_step, s);
             if (e == cudaSuccess) e = fpc::launch_mlp_pack(h->theta, h->wpack, s);
         }

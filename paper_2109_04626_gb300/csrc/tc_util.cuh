@@ -103,9 +103,9 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar)
                  : "memory");
 }
 
-__device__ __forceinline__ void tc_ld_32cols(uint32_t taddr, float *out)
+// 32 columns of this warp's TMEM lanes; the values are there after tc_ld_wait
+__device__ __forceinline__ void tc_ld_32cols_async(uint32_t taddr, uint32_t (&r)[32])
 {
-    uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -115,11 +115,28 @@ __device__ __forceinline__ void tc_ld_32cols(uint32_t taddr, float *out)
           "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
           "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// Waits for every load before it.  r passes through the statement so that its uses stay
+// behind the wait.
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28])
+                 :
+                 : "memory");
+    asm volatile("" : "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
+}
+__device__ __forceinline__ void tc_ld_32cols(uint32_t taddr, float *out)
+{
+    uint32_t r[32];
+    tc_ld_32cols_async(taddr, r);
+    tc_ld_wait(r);
 #pragma unroll
     for (int j = 0; j < 32; ++j) out[j] = __uint_as_float(r[j]);
 }
-
 
 __device__ __forceinline__ void tc_alloc(uint32_t *dst_smem, uint32_t ncols)
 {
