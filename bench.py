@@ -54,7 +54,7 @@ def dominant_class(tim):
 
 # the kernels behind each timing class that the roofline names
 CLASS_KERNELS = {
-    "ci_direct": "ci_pairwarp_kernel (l = 1, 2, degree > 32: a warp per ordered pair) + ci_node_kernel "
+    "ci_direct": "ci_pairgroup_kernel (l = 1, 2, degree > 32: groups of pairs of a node) + ci_node_kernel "
                  "(degree <= 128: corr block in shared memory) + ci_lane_kernel (other stages l <= 12) + "
                  "ci_direct_kernel (one warp per test) + ci_redecide_kernel (FP64 pass)",
     "ci_complement": "ci_complement_kernel (FP64, from neighbourhood precision blocks)",

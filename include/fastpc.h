@@ -136,8 +136,9 @@ void pc_destroy(pc_handle *h);
  *                 adj(u)\{v} of both endpoints (default).  Not with "learned" or
  *                 a batched handle.
  *   "pair_warp"   1 = at stages 1 and 2, the ordered pairs of nodes of degree
- *                 above "pair_warp_dmin" (default 32) run one warp per pair, the
- *                 32 lanes on 32 consecutive sets of the pair (default); 0 = off
+ *                 above "pair_warp_dmin" (default 32) run in groups of pairs
+ *                 of one node, the 32 lanes of a warp on 32 consecutive sets of
+ *                 its neighbourhood for every pair of the group (default); 0 = off
  *   "node_dmax"   the other small-stage nodes of degree <= node_dmax (0..128,
  *                 default 128) run on the staged kernel, which holds
  *                 corr[adj(u), adj(u)] in shared memory; the rest read corr

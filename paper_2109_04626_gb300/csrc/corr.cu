@@ -167,7 +167,7 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
     const T *x = X + (ok ? col : 0);
     for (int a = blockIdx.x * CS_CLUSTER + (int)cl.block_rank(); a < p; a += gridDim.x * CS_CLUSTER)
         for (int b = a + 1 + threadIdx.x; b < p; b += blockDim.x) C[(long long)a * ldc + b] = 0.0;
-    if (blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
+    if (err && blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
     // the warps' values -> the cluster's total, the same in every CTA
     auto total = [&](double v, int pass) -> double {
         red[w][tx] = v;

@@ -862,6 +862,23 @@ static pc_status ensure_c32tc(pc_handle *h)
     return PC_OK;
 }
 
+// Does the correlation step form all FP64 correlations by the exact product from X itself
+// (C32 their rounding)?  Always for FP64 tests; FP32-first where the search needs all of
+// them (the reversed order) or they cost no more than the split-precision product with its
+// planes and the FP64 entries formed on demand: problems of p <= NL_PMAX, and batches of
+// instances of p <= EXACT_BATCH_PMAX, whose products fill the chip side by side
+// (64 instances of 50-400 variables and 2000-20000 samples: 6.3 ms for 3.1 with the
+// split-precision product, and in return the search takes 8-9 ms for 19-66, its FP64 tests
+// being decided on the spot instead of queued, their entries formed and re-read).
+static bool exact_corr(const pc_handle *h)
+{
+    if (!fpc::tc_gemm_available() || h->precision == 1) return false;
+    if (h->precision == 0 || h->order == 1) return true;
+    int pm = h->nblk ? 0 : h->p;
+    for (int i = 0; i < h->nblk; ++i) pm = std::max(pm, h->boff[i + 1] - h->boff[i]);
+    return pm <= (h->nblk ? fpc::EXACT_BATCH_PMAX : fpc::NL_PMAX);
+}
+
 // Standardisation and correlation GEMM of one problem, or of instance blk of a
 // batched handle (its columns are rows [o, o+p) of the planes, its block of
 // corr the diagonal block there).
@@ -895,14 +912,9 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
         CK(cudaMemcpyAsync(Xstage, X, bytes, cudaMemcpyHostToDevice, s));
         Xd = Xstage;
     }
-    // One problem that needs all FP64 correlations (FP64 tests, the reversed order), or is
-    // small enough that they cost no more than the split-precision product with its planes
-    // and the FP64 entries formed on demand: the exact product from X itself, C32 its
-    // rounding.
-    if (blk < 0 && fpc::tc_gemm_available() &&
-        (h->precision == 0 || (h->precision == 2 && (h->order == 1 || p <= fpc::NL_PMAX)))) {
-        Timed tm(h, 0);
-        if (h->precision == 2) {
+    if (exact_corr(h)) {
+        Timed tm(h, lane ? -1 : 0);
+        if (h->precision == 2 && blk < 0) {
             h->keep_dtype = dtype;
             h->keep_x = Xd;
             h->keep_ld = ld;
@@ -923,17 +935,27 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
             }
         }
         h->c32tc_valid = false;
-        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean, h->rsd, h->C64, h->ldc, h->tc_err, s));
+        double *C64b = blk < 0 ? h->C64 : h->C64 + h->pbase[blk];
+        float *C32x = blk < 0 ? h->C32 : h->C32 + h->pbase[blk];
+        const int ldx = blk < 0 ? h->ldc : p;
+        // a batch's instances share the error flag: cleared with the first of them
+        if (blk == 0 && !lane) CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
+        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, blk < 0 ? h->tc_err : nullptr,
+                                 s));
         {
-            Timed tg(h, 7);
-            CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean, h->rsd, h->C64, h->ldc, h->C32, h->ldc,
-                                      h->tc_err, s));
+            Timed tg(h, lane ? -1 : 7);
+            CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, C32x, ldx, h->tc_err, s));
         }
         h->used_tc = true;
         h->c32_rounded = true;
-        h->c64_full = true;
-        if (!h->Pbuf) CK(dalloc(h, &h->Pbuf, (size_t)p * h->ldc * sizeof(double)));
         h->have_corr = true;
+        if (blk < 0) {
+            if (!h->Pbuf) CK(dalloc(h, &h->Pbuf, (size_t)p * h->ldc * sizeof(double)));
+        } else {
+            h->bdone[blk] = 1;
+            for (char d : h->bdone) h->have_corr = h->have_corr && d;
+        }
+        h->c64_full = h->have_corr;
         h->have_skel = false;
         return PC_OK;
     }
@@ -1052,7 +1074,8 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
     for (int i = 0; i < k; ++i)
         if (!X[i] || (dtype[i] != PC_F32 && dtype[i] != PC_F64) || ld[i] < h->boff[i + 1] - h->boff[i])
             return fail(h, PC_ERR_ARG, "pc_corr_blocks: bad X, dtype or ld of instance " + std::to_string(i));
-    if (h->precision == 0) {
+    const bool exact = exact_corr(h);
+    if (h->precision == 0 && !exact) {
         // the FP64 Gram shares one split-K workspace: one instance after the other
         for (int i = 0; i < k; ++i)
             if (pc_status r = corr_impl(h, X[i], dtype[i], ld[i], i)) return r;
@@ -1062,11 +1085,13 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
     Timed tm(h, 0);
     // what the instances share, on the handle's stream before the fork: the
     // standardised planes, the FP64-validity flags, the GEMM's error flag
-    if (pc_status r = alloc_planes(h, s)) return r;
-    if (!h->c64_valid) {
-        CK(dalloc(h, &h->c64_valid, (h->pair_elems + 7) / 4 * 4));
-        CK(cudaMemsetAsync(h->c64_valid, 0, (h->pair_elems + 7) / 4 * 4, s));
-        if (pc_status r = alloc_c64_list(h)) return r;
+    if (!exact) {
+        if (pc_status r = alloc_planes(h, s)) return r;
+        if (!h->c64_valid) {
+            CK(dalloc(h, &h->c64_valid, (h->pair_elems + 7) / 4 * 4));
+            CK(cudaMemsetAsync(h->c64_valid, 0, (h->pair_elems + 7) / 4 * 4, s));
+            if (pc_status r = alloc_c64_list(h)) return r;
+        }
     }
     CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
     const int nl = std::min(k, 8);
@@ -2092,7 +2117,9 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     tp.dr_max = 5e-6f;
     if (h->c32_rounded && h->precision == 2) {
         tp.eps_c = 1.0e-6f;
-        if (fpc::ci_list_uses_fp32(l, tp)) {
+        if (h->nblk) {
+            tp.precision = 0;                            // a batch keeps no X for that product: all in FP64
+        } else if (fpc::ci_list_uses_fp32(l, tp)) {
             if (pc_status r = ensure_c32tc(h)) return r;
             C32 = h->C32tc;
         }

@@ -62,7 +62,7 @@ struct LevelInfo {
     int kernels_run;                    // kernels the captured stage loop executed
     unsigned deg_ticket;                // CTAs of the stage's degrees kernel done (last one runs the tail)
     unsigned long long node_next;       // next work item of the staged small-stage kernel
-    unsigned long long pair_next;       // next ordered pair of the warp-per-pair kernel
+    unsigned long long pair_next;       // next pair group of the pair-group kernel
 };
 
 // Conditional nodes of the captured stage body: the head kernel picks one branch
@@ -73,6 +73,9 @@ struct StageConds {
     int use;                            // 1 inside the captured stage body
     int has_comp, has_score, has_prec;  // which kernels the body has
 };
+// Batched handles whose instances have at most this many variables form all FP64
+// correlations at once (the exact product); larger ones form them on demand.
+constexpr int EXACT_BATCH_PMAX = 512;
 constexpr int LANE_LMAX = 12;           // stages the lane-per-test kernel runs (FP32 modes)
 // Staged small-stage kernel: a node whose frozen degree is at most NODE_DMAX has
 // the block corr[adj(u), adj(u)] staged in shared memory by the CTA that runs
@@ -82,8 +85,8 @@ constexpr int NODE_THREADS = 256;
 constexpr unsigned long long NODE_ITEM_CHUNKS = 512;    // chunks per work item (two per thread)
 constexpr int NODE_ROUNDS_MAX = (int)NODE_ITEM_CHUNKS / 2 + 1;   // rank rounds an item spans (degree >= 2)
 // Stages 1 <= l <= PAIRWARP_LMAX: the pairs of nodes of degree above
-// pair_warp_dmin (default PAIRWARP_DMIN) run one warp per ordered pair, the
-// lanes on consecutive sets of the pair.
+// pair_warp_dmin (default PAIRWARP_DMIN) run in groups of pairs of one node, the
+// lanes of a warp on consecutive sets.
 constexpr int PAIRWARP_LMAX = 2;
 constexpr int PAIRWARP_DMIN = 32;
 constexpr int LANE_RANGES = 6;          // small-stage kernel instantiations: l 0-2, 3-4, 5-6, 7-8, 9-10, 11-12
@@ -132,7 +135,7 @@ struct GraphDev {
     unsigned long long *rn_off; // p+1: first remainder test of each node (small-stage kernel)
     unsigned long long *ia_off; // p+1: staged small-stage kernel, first items: one per staged node
     unsigned long long *it_off; // p+1: staged small-stage kernel, the nodes' further items
-    unsigned long long *wo_off; // p+1: warp-per-pair kernel, first ordered pair of each of its nodes
+    unsigned long long *wo_off; // p+1: pair-group kernel, first group of each of its nodes
     unsigned long long *best;   // p x p, best (side<<62 | rank) per unordered pair (a<b at a*p+b)
     const unsigned long long *binom;   // ldb x ldb saturating binomials
     int ldb;                    // p+1 (batched problems: largest instance p + 1)
@@ -190,7 +193,7 @@ struct TestParams {
     int node_dmax;      // stages 1 <= l <= LANE_LMAX: nodes of degree <= node_dmax run on the
                         // staged kernel (corr block in shared memory); 0: none
     int pair_warp;      // stages 1 <= l <= PAIRWARP_LMAX: the pairs of nodes of degree above
-                        // pair_warp_dmin one warp per pair (0: off)
+                        // pair_warp_dmin in groups of pairs (0: off)
     int pair_warp_dmin;
     int precision;      // 0 fp64, 1/2 fp32 tests with FP64 re-decision
     int comp_fp32;      // complement tests in FP32 first, FP64 where the bound does not decide
@@ -219,7 +222,7 @@ struct TestParams {
 void note_launch();
 
 // ---- correlation (corr.cu)
-// without a workspace; also clears C above the diagonal and err for launch_gram_exact
+// without a workspace; also clears C above the diagonal and err (nullptr: the caller has) for launch_gram_exact
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
                              double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s);
 cudaError_t launch_col_stats_split(const void *X, int dtype, long long n, int p, long long ld,

@@ -121,16 +121,35 @@ __global__ void __launch_bounds__(256) degrees_tail_kernel(GraphDev g, TestParam
     tail_body(g, tp, cap, 0, nullptr, 0, hc, use_cond, sc, true);
 }
 
-// Stages 1 and 2: the pairs of a node of degree above pair_warp_dmin run one
-// warp per pair.
+// Stages 1 and 2: the pairs of a node of degree above pair_warp_dmin run on the
+// pair-group kernel.
 __device__ __forceinline__ bool pair_warped(const TestParams &tp, int l, int dg)
 {
     return tp.pair_warp && l >= 1 && l <= PAIRWARP_LMAX && dg > tp.pair_warp_dmin;
 }
 
+constexpr int PG1_PAIRS = 8, PG_PAIRS = 32;              // pairs of a group at stages 1 and 2
+constexpr int PG_FIRST = 256;
+constexpr int PG_FLOATS = 12288;                         // rows corr[v, adj(u)] of a group: 48 KiB
+constexpr int PG_THREADS = 256;
+
+// pairs per group of a node of degree dg at stage l: equal groups; at stage 2 of pairs
+// whose rows fit the shared memory (nodes with larger rows: a warp per pair, from L2)
+__device__ __forceinline__ int pair_group(int l, int dg)
+{
+    const int most = l == 1 || dg > PG_FLOATS ? PG1_PAIRS : min(PG_PAIRS, PG_FLOATS / dg);
+    const int ng = (dg + most - 1) / most;
+    return (dg + ng - 1) / ng;
+}
+__device__ __forceinline__ int pair_groups(int l, int dg)
+{
+    const int vg = pair_group(l, dg);
+    return (dg + vg - 1) / vg;
+}
+
 // The small-stage tests of a node of degree dg at stage l >= 1 run on the staged
 // kernel when its neighbourhood block fits the shared-memory layout (and the
-// node is not one of the warp-per-pair kernel).
+// node is not one of the pair-group kernel).
 __device__ __forceinline__ bool node_staged(const TestParams &tp, int l, int dg)
 {
     return l >= 1 && dg <= tp.node_dmax && !pair_warped(tp, l, dg);
@@ -389,10 +408,10 @@ __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, 
         const ull nc = sat_mul((T + ch - 1) / ch, (ull)dg);
         return nc == KEY_NONE ? KEY_NONE : (nc + NODE_ITEM_CHUNKS - 1) / NODE_ITEM_CHUNKS;
     };
-    // warp-per-pair kernel: the pairs of the larger direct nodes of stages 1-2
+    // pair-group kernel: the pairs of the larger direct nodes of stages 1-2
     auto warp_mode = [&](int dg, ull T) -> bool { return small && T && pair_warped(tp, l, dg); };
     // direct, complement, proposal rows, staged nodes (their first items), the
-    // staged nodes' further items, warp-per-pair ordered pairs
+    // staged nodes' further items, pair groups
     ull v[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull}, mxT = 0;
     bool sat = false;
     for (int u = s0; u < s1; ++u) {
@@ -413,7 +432,7 @@ __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, 
             v[2] = sat_add(v[2], prows(dg, T));           // complement-path pairs keep the plain order
             v[3] += k ? 1ull : 0ull;
             v[4] = sat_add(v[4], k ? k - 1 : 0ull);
-            v[5] += warp_mode(dg, T) ? (ull)dg : 0ull;
+            v[5] += warp_mode(dg, T) ? (ull)pair_groups(l, dg) : 0ull;
         }
     }
     const int ssat = __syncthreads_or(sat);
@@ -445,7 +464,7 @@ __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, 
                 const ull k = Ik[u - s0];
                 ra += k ? 1ull : 0ull;
                 ri = sat_add(ri, k ? k - 1 : 0ull);
-                rw += (!cm[u - s0] && warp_mode(dg, T)) ? (ull)dg : 0ull;
+                rw += (!cm[u - s0] && warp_mode(dg, T)) ? (ull)pair_groups(l, dg) : 0ull;
             }
         }
     }
@@ -564,6 +583,7 @@ size_t scan_ws_bytes(long long n) { return 64 + 0 * n; }
 // than 2^32 tests of one stage); its FP32 flops are tests x F(L), formed at the end
 struct LaneAcc {
     unsigned tests, band, guard;
+    unsigned red, degen;       // decided in FP64 on the spot (pair groups)
 };
 
 // Candidate position x of the ordered pair (u, j) (d candidates) -> node id:
@@ -972,7 +992,7 @@ template <int L, bool PROP>
 __device__ __forceinline__ void lane_dispatch(const GraphDev &g, const TestParams &tp, const float *C32, int ldc,
                                               ull *queue, ull qcap, ull *qlen)
 {
-    LaneAcc acc = {0u, 0u, 0u};
+    LaneAcc acc = {};
     const int p = g.p;
     const long long NP = g.info->n_opairs;
     const int rounds = g.info->lane_rounds;
@@ -993,7 +1013,7 @@ __device__ __forceinline__ void lane_dispatch(const GraphDev &g, const TestParam
             const int u = g.opu[o];                     // owner of ordered pair o
             if (g.tn_off[u + 1] == g.tn_off[u]) continue;   // not a direct node this stage
             if (g.ia_off[u + 1] != g.ia_off[u]) continue;   // its pairs run on the staged kernel
-            if (g.wo_off[u + 1] != g.wo_off[u]) continue;   // ... or on the warp-per-pair kernel
+            if (g.wo_off[u + 1] != g.wo_off[u]) continue;   // ... or on the pair-group kernel
             const int d = g.deg[u] - 1;
             const ull T = g.binom[(long long)d * g.ldb + L];
             const ull r0 = (ull)r * chunk;
@@ -1079,7 +1099,7 @@ __device__ __forceinline__ void node_dispatch(const GraphDev &g, const TestParam
     float *cus = node_smem;                              // NODE_DMAX floats
     short *pos_s = (short *)(node_smem + NODE_DMAX);     // NODE_ROUNDS_MAX x L start positions
     float *B = node_smem + NODE_DMAX + (NODE_ROUNDS_MAX * LP + 1) / 2;   // deg x deg
-    LaneAcc acc = {0u, 0u, 0u};
+    LaneAcc acc = {};
     const int p = g.p;
     const ull na = g.ia_off[p], nitems = na + g.it_off[p];
     int staged = -1;                                     // node whose block is in shared memory
@@ -1170,15 +1190,76 @@ __global__ void __launch_bounds__(NODE_THREADS, HI <= 2 ? 3 : (HI <= 4 ? 3 : (HI
     node_switch<(LO > 1 ? LO : 1), HI, PROP>(l, g, tp, C32, ldc, queue, qcap, qlen);
 }
 
-// ---------------------------------------------------------------- one warp per pair (stages 1-2)
-// At stages 1 and 2 the nodes too large for the staged layout have hundreds of
-// neighbours.  A warp takes one of their ordered pairs (u, v) from the stage
-// counter and walks its sets in lexicographic order, 32 at a time: lane i tests
-// the set of rank base + i (the bordered test of lane_tests_lex, one set), so
-// the rows corr[u, .], corr[v, .] and the prefix member's row are the same for
-// the whole warp and the index arithmetic is shared.  The pair stops at the
-// first block in which a test separates (keys by atomicMin: the lowest rank
-// wins), or when the pair's key shows an earlier separation.
+// ---------------------------------------------------------------- pair groups (stages 1-2)
+// At stages 1 and 2 nearly every test is clearly dependent, and the work of a test
+// splits into a part of (u, S) alone and a part of v.  A group is a number of ordered
+// pairs (u, v_0), (u, v_1), ... of one node; the sets of adj(u) are walked in
+// lexicographic order, a lane per set.  The lane forms once what depends on u and S only
+// -- at stage 2 c = corr(s0, s1), x = 1 - c^2, the row of u eliminated by S, h11, and from
+// them the bound below -- and then tests the set against every pair of the group, with
+// corr(v, s0) and corr(v, s1): about 12 FP32 operations a test.
+//
+// Such a test decides only where the rule of fp32_trust certainly trusts FP32.  With
+// alpha_u^2 = A_u^2 / h11, alpha_v^2 = A_v^2 / h22 and eps = eps_c + 4 m eps32 that rule's
+// bound is at most
+//   |dr| <= 2 eps (alpha_u^2 + alpha_v^2) + 8 eps32,
+// and the coefficients of v on S satisfy
+//   A_v <= 1 + |b0| + |c_v|/x (1 + |c|) <= 2 + (1 + |c|) / sqrt(x) = A_max
+// because c_v^2 / x <= 1 (L = 1: A_v <= 2).  So the test is dependent when
+//   |h12| > sqrt(h11) sqrt(h22) (r_q + g0 + 2 eps alpha_u^2 + 2 eps A_max^2 / h22),
+// g0 = band / sqrt(n-l-3) + 8 eps32 covering the band, which with k1 = sqrt(h11)
+// (r_q + g0 + 2 eps alpha_u^2) and kappa = 2 eps A_max^2 / (r_q + g0) follows from
+//   |h12| > k1 (h22 + kappa) / sqrt(h22),
+// and independent when (h11 <= 1)
+//   |h12| < (ki h22 - 2 eps A_max^2) / sqrt(h22),  ki = sqrt(h11) (r_q - g0 - 2 eps alpha_u^2).
+// The rule's premises (pivots above the guard, eps alpha^2 and kap below 0.05) are kept
+// by h22 >= hmin and by the limits on x and h11; factors 1.05 and 1.0001 cover the
+// rounding.  Every other test (NaN included) goes to a list of its warp, and the warp
+// runs up to 32 of them at a time through lane_tests_lex: the keys, the queue and the
+// decisions are those of the other layouts.
+//
+// A set that contains v itself is not a test of that pair (skipped when listed: its
+// h22 is 0, so it never passes as dependent).  A pair is dropped once a set before the
+// present ones separates it (sep_s), or the other side of the edge has.  At stage 1 (one
+// member: x = 1) a warp takes a group, at stage 2 a CTA.
+//
+// Bound: issue slots and the latency of the u side's gathers.  A sparse graph of 1000 nodes
+// (20000 samples): stage 1 took 765 us and stage 2 (3e8 tests) 3.1 ms with a warp per pair
+// and the general test for every set (about 300 instructions); 0.36 and 0.75 ms here.  One
+// warp per group at stage 2 as well took 2.4 ms (the few groups left at the end walk 1e4
+// sets each), all eight warps on the same sets from the start 0.78 ms but twice the tests
+// where pairs separate early.  64 dense graphs of 50-400 nodes, stages 1 and 2: 4.6 -> 2.4 ms.
+
+__device__ __forceinline__ float rsqrt_fast(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcp_fast(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The last u < p with off[u] <= t (off: p + 1 ascending offsets, off[0] = 0 <= t < off[p]),
+// by the whole warp: 32 probes at a time instead of a chain of binary steps.
+__device__ __forceinline__ int warp_owner(const ull *off, int p, ull t)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = p;                                    // the answer lies in [lo, lo + n)
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, i < n && off[lo + min(i, n - 1)] <= t);
+        const int k = 31 - __clz(m);                      // lane 0 always holds
+        lo += k * step;
+        n = min(step, n - k * step);
+    }
+    return lo;
+}
+
 // Advance the lexicographic position (q0 < q1 < d) by k sets; positions past the
 // last set stop at q0 = d - 1.
 __device__ __forceinline__ void lex2_advance(int &q0, int &q1, int k, int d)
@@ -1190,73 +1271,420 @@ __device__ __forceinline__ void lex2_advance(int &q0, int &q1, int k, int d)
     }
 }
 
+// One ordered pair by a warp, 32 consecutive sets at a time in the order of its
+// candidate list: the pairs of a proposal-ordered stage (each pair has its own order)
+// and of nodes whose rows do not fit the shared memory.
 template <int L, bool PROP>
-__device__ __forceinline__ void pairwarp_dispatch(const GraphDev &g, const TestParams &tp, const float *C32, int ldc,
-                                                  ull *queue, ull qcap, ull *qlen)
+__device__ __noinline__ void pair_by_warp(const GraphDev &g, const TestParams &tp, const float *C32, int ldc,
+                                          int u, int j, ull *queue, ull qcap, ull *qlen, LaneAcc &acc)
 {
-    static_assert(L == 1 || L == 2, "the warp-per-pair kernel runs stages 1 and 2");
     const int lane = threadIdx.x & 31;
-    LaneAcc acc = {0u, 0u, 0u};
-    const int p = g.p;
-    const ull npairs = g.wo_off[p];
-    for (;;) {
-        ull o = 0;
-        if (lane == 0) o = atomicAdd(&g.info->pair_next, 1ull);
-        o = __shfl_sync(0xffffffffu, o, 0);
-        if (o >= npairs) break;
-        const int u = (int)(upper_bound_dev(g.wo_off, (long long)p + 1, o) - 1);
-        const int j = (int)(o - g.wo_off[u]);
-        const int d = g.deg[u] - 1;
+    const int d = g.deg[u] - 1;
+    const ull T = g.binom[(long long)d * g.ldb + L];
+    const int *nb = g.nbr + nidx(g, u);
+    const int v = nb[j];
+    const GlobalSrc src{C32, tp.prow, ldc, nb, C32 + cidx(tp.prow, ldc, u, 0), C32 + cidx(tp.prow, ldc, v, 0), v};
+    const float sqf = sqrtf((float)(n_of(tp, u) - L - 3)), rq = tanhf(tp.qf / sqf);
+    const ull *bp = g.best + pidx(g, min(u, v), max(u, v));
+    const ull side = (ull)(u > v) << 62;
+    int b0 = 0, b1 = 1;                                   // positions of the block's first set (L = 2)
+    for (ull base = 0; base < T; base += 32) {
+        if (*(volatile const ull *)bp < (side | base)) break;   // an earlier set separates
+        const ull rank = base + (ull)lane;
+        int pos[L];
+        if (L == 1) {
+            pos[0] = (int)rank;
+        } else {
+            int q0 = b0, q1 = b1;
+            lex2_advance(q0, q1, lane, d);
+            pos[0] = q0;
+            pos[L - 1] = q1;
+        }
+        bool found = false;
+        if (rank < T)
+            found = lane_tests_lex<L, PROP, GlobalSrc, false, int>(g, tp, src, u, v, j, d, T, rank, rank + 1, queue,
+                                                                   qcap, qlen, acc, sqf, rq, pos);
+        if (__any_sync(0xffffffffu, found)) break;
+        if (L == 2) lex2_advance(b0, b1, 32, d);
+    }
+}
+
+// Lexicographic rank of the listed set (indices into adj(u)) among the sets of pair j.
+template <int L>
+__device__ __forceinline__ ull pair_set_rank(unsigned key, int j, int d, int *pos)
+{
+    if (L == 1) {
+        pos[0] = (int)key - ((int)key > j);
+        return (ull)pos[0];
+    }
+    const int i0 = (int)(key >> 16), i1 = (int)(key & 0xffffu);
+    pos[0] = i0 - (i0 > j);
+    pos[L - 1] = i1 - (i1 > j);
+    const ull q = (ull)pos[0];                            // sets before the row of q, then the place in it
+    return q * (ull)d - q * (q + 1) / 2 + (ull)(pos[L - 1] - pos[0] - 1);
+}
+
+// The test of (u, v) given S = {s0} or {s0, s1} in FP64: the bordered elimination of the
+// FP32 tests, the degeneracy rule and the decision of the warp-per-test evaluation (|r| against
+// r_q = tanh(q / sqrt(n-l-3)) where they differ by more than rq's rounding, else the
+// statistic itself).
+template <int L>
+__device__ __forceinline__ bool pair_test64(const TestParams &tp, const double *C64, int ldc, int u, int v, int s0,
+                                            int s1, float rq, LaneAcc &acc)
+{
+    const double *Cu = C64 + cidx(tp.prow, ldc, u, 0), *Cv = C64 + cidx(tp.prow, ldc, v, 0);
+    const double a0 = Cu[s0], b0 = Cv[s0];
+    double h11 = fma(-a0, a0, 1.0), h22 = fma(-b0, b0, 1.0), h12 = fma(-a0, b0, Cu[v]), x = 1.0;
+    ++acc.tests;
+    ++acc.red;
+    if (L == 2) {
+        const double c = C64[cidx(tp.prow, ldc, s0, 0) + s1];
+        const double wu = fma(-a0, c, Cu[s1]), wv = fma(-b0, c, Cv[s1]);
+        x = fma(-c, c, 1.0);
+        const double rx = rcp_pivot(x), t = wu * rx;
+        h11 = fma(-t, wu, h11);
+        h22 = fma(-wv * rx, wv, h22);
+        h12 = fma(-t, wv, h12);
+    }
+    if (fmin(x, fmin(h11, h22)) < tp.guard) ++acc.guard;
+    else ++acc.band;
+    if (!(x > DEGEN) || !(h11 > DEGEN) || !(h22 > DEGEN)) {
+        ++acc.degen;
+        return true;
+    }
+    const double hh = h11 * h22, t = h12 * h12, q2 = (double)rq * (double)rq * hh;
+    if (t < q2 * (1.0 - 8e-6)) return true;
+    if (t > q2 * (1.0 + 8e-6)) return false;
+    const double r = h12 / sqrt(hh), sq = sqrt((double)(n_of(tp, u) - L - 3));
+    return fabs(r) < 1.0 && sq * fabs(atanh(r)) <= tp.q;
+}
+
+// The first n <= 32 listed tests of the warp, one per lane.  An entry holds the set's
+// indices into adj(u) (x: the lexicographic key i0 << 16 | i1, or i0 at stage 1) and the
+// pair's place in the group (y).  In FP64 at once when all FP64 correlations are there: a
+// pair whose FP32 tests cannot be trusted then ends at its separating set, instead of
+// queueing the tests of all its sets.
+template <int L>
+__device__ __noinline__ void pair_group_listed(const GraphDev &g, const TestParams &tp, const float *C32,
+                                               const double *C64, int ldc, int u, int j0, const uint2 *list, int n,
+                                               unsigned *sep_s, float sqf, float rq, ull *queue, ull qcap, ull *qlen,
+                                               LaneAcc &acc)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane >= n) return;
+    const uint2 e = list[lane];
+    if (*(volatile unsigned *)(sep_s + e.y) < e.x) return;      // an earlier set separates
+    const int d = g.deg[u] - 1, j = j0 + (int)e.y;
+    const int *nb = g.nbr + nidx(g, u);
+    const int v = nb[j];
+    int pos[L];
+    const ull rank = pair_set_rank<L>(e.x, j, d, pos);
+    bool ind;
+    if (!tp.lazy) {
+        ind = pair_test64<L>(tp, C64, ldc, u, v, nb[L == 1 ? e.x : e.x >> 16], nb[L == 1 ? e.x : e.x & 0xffffu], rq, acc);
+        if (ind) atomicMin(g.best + pidx(g, min(u, v), max(u, v)), ((ull)(u > v) << 62) | rank);
+    } else {
         const ull T = g.binom[(long long)d * g.ldb + L];
-        const int *nb = g.nbr + nidx(g, u);
-        const int v = nb[j];
-        const GlobalSrc src{C32, tp.prow, ldc, nb, C32 + cidx(tp.prow, ldc, u, 0), C32 + cidx(tp.prow, ldc, v, 0),
-                            v};
-        const float sqf = sqrtf((float)(n_of(tp, u) - L - 3)), rq = tanhf(tp.qf / sqf);
-        const ull *bp = g.best + pidx(g, min(u, v), max(u, v));
-        const ull side = (ull)(u > v) << 62;
-        int b0 = 0, b1 = 1;                               // positions of the block's first set (L = 2)
-        for (ull base = 0; base < T; base += 32) {
-            if (*(volatile const ull *)bp < (side | base)) break;   // an earlier set separates
-            const ull rank = base + (ull)lane;
+        const GlobalSrc src{C32, tp.prow, ldc, nb, C32 + cidx(tp.prow, ldc, u, 0), C32 + cidx(tp.prow, ldc, v, 0), v};
+        ind = lane_tests_lex<L, false, GlobalSrc, false, int>(g, tp, src, u, v, j, d, T, rank, rank + 1, queue, qcap,
+                                                              qlen, acc, sqf, rq, pos);
+    }
+    if (ind) atomicMin(sep_s + e.y, e.x);
+}
+
+// What the bound needs of (u, S), per lane (see above).
+template <int L>
+struct PairBound {
+    float k1, ki;              // sqrt(h11) (r_q +- (g0 + 2 eps alpha_u^2)); INFINITY and -1: the premises fail
+    float kappa, k2, hmin;     // of A_max
+    // x: 1 - c^2 (L = 1: 1)
+    __device__ __forceinline__ PairBound(const TestParams &tp, float rq, float g0, float x, float c, float h11,
+                                         float Au, bool ok)
+    {
+        const float eps = tp.eps_c + (4.0f * (float)(L + 2)) * EPS32;
+        const float guard = 1.001f * (float)tp.guard + 1e-12f;
+        const float ih = rsqrt_fast(fmaxf(h11, 1e-30f)), sh = h11 * ih, au2 = Au * Au * ih * ih;
+        const float am = L == 1 ? 2.0f : 2.0f + (1.0f + fabsf(c)) * rsqrt_fast(fmaxf(x, 1e-30f));
+        const float m = g0 + 2.1f * eps * au2;
+        ok &= tp.dr_max >= 0.5f && x >= guard && (float)(2 * (L + 2)) * eps <= 0.045f * x && h11 >= guard &&
+              1.05f * eps * au2 <= 0.05f;
+        k1 = ok ? 1.0001f * sh * (rq + m) : INFINITY;
+        ki = ok ? 0.9998f * sh * (rq - m) : -1.0f;
+        k2 = 2.1f * eps * am * am;
+        kappa = k2 * rcp_fast(rq + g0);
+        hmin = fmaxf(guard, 10.0f * k2);
+    }
+    __device__ __forceinline__ bool dependent(float h22, float h12) const
+    {
+        return h22 >= hmin && fabsf(h12) > k1 * (h22 + kappa) * rsqrt_fast(h22);
+    }
+    __device__ __forceinline__ bool independent(float h22, float h12) const
+    {
+        return h22 >= hmin && fabsf(h12) < (ki * h22 - k2) * rsqrt_fast(h22);
+    }
+};
+
+// A step of pair vi with tests that are not certain to be dependent (put; ind: certain to be
+// independent).  The first certain separation is recorded at once -- the tests after it are
+// not needed -- and the other tests before it join the warp's list, which runs as soon as
+// it holds 32.
+template <int L>
+__device__ __forceinline__ void pair_group_put(const GraphDev &g, const TestParams &tp, const float *C32, const double *C64, int ldc,
+                                               int u, int j0, int dg, uint2 *list, int &nlist, bool put, bool ind,
+                                               unsigned key, int vi, unsigned *sep_s, float sqf, float rq,
+                                               ull *queue, ull qcap, ull *qlen, LaneAcc &acc)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned bi = __ballot_sync(0xffffffffu, ind);
+    if (bi) {
+        const int at = __ffs(bi) - 1;
+        if (put && lane >= at) {
+            ++acc.tests;                                  // decided here, or not needed
+            put = false;
+        }
+        if (lane == at) {
+            const int v = g.nbr[nidx(g, u) + j0 + vi];
             int pos[L];
-            if (L == 1) {
-                pos[0] = (int)rank;
-            } else {
-                int q0 = b0, q1 = b1;
-                lex2_advance(q0, q1, lane, d);
-                pos[0] = q0;
-                pos[L - 1] = q1;
-            }
-            bool found = false;
-            if (rank < T)
-                found = lane_tests_lex<L, PROP, GlobalSrc, false, int>(g, tp, src, u, v, j, d, T, rank, rank + 1,
-                                                                       queue, qcap, qlen, acc, sqf, rq, pos);
-            if (__any_sync(0xffffffffu, found)) break;
-            if (L == 2) lex2_advance(b0, b1, 32, d);
+            const ull rank = pair_set_rank<L>(key, j0 + vi, dg - 1, pos);
+            atomicMin(g.best + pidx(g, min(u, v), max(u, v)), ((ull)(u > v) << 62) | rank);
+            atomicMin(sep_s + vi, key);
         }
     }
-    ull tests = acc.tests, band = acc.band, guard = acc.guard;
+    const unsigned bs = __ballot_sync(0xffffffffu, put);
+    if (put) list[nlist + __popc(bs & ((1u << lane) - 1u))] = make_uint2(key, (unsigned)vi);
+    nlist += __popc(bs);
+    __syncwarp();
+    if (nlist >= 32) {
+        pair_group_listed<L>(g, tp, C32, C64, ldc, u, j0, list, 32, sep_s, sqf, rq, queue, qcap, qlen, acc);
+        __syncwarp();
+        nlist -= 32;
+        if (lane < nlist) list[lane] = list[32 + lane];
+        __syncwarp();
+    }
+}
+
+__device__ __forceinline__ void pair_group_flush(const LaneAcc &acc, ull fast, ull fl, DevCounters *ctr)
+{
+    ull tests = (ull)acc.tests + fast, band = acc.band, guard = acc.guard, red = acc.red, degen = acc.degen;
     for (int off = 16; off > 0; off >>= 1) {
         tests += __shfl_xor_sync(0xffffffffu, tests, off);
         band += __shfl_xor_sync(0xffffffffu, band, off);
         guard += __shfl_xor_sync(0xffffffffu, guard, off);
+        red += __shfl_xor_sync(0xffffffffu, red, off);
+        degen += __shfl_xor_sync(0xffffffffu, degen, off);
     }
-    if (lane == 0) {
-        WarpAcc w = {tests, 0, band, guard, 0, tests * flops_direct(L), 0, 0.f};
-        flush_acc(w, g.ctr);
+    if ((threadIdx.x & 31) == 0) {
+        WarpAcc wa = {tests, red, band, guard, degen, (tests - red) * fl, red * fl, 0.f};
+        flush_acc(wa, ctr);
     }
 }
 
+// Stage 1: a warp per group of up to PG1_PAIRS pairs; the group's entries corr(v, s) of a
+// round are loaded together from L2 (each is used once).
 template <bool PROP>
-__global__ void __launch_bounds__(256, 4) ci_pairwarp_kernel(GraphDev g, TestParams tp, const float *C32, int ldc,
-                                                             ull *queue, ull qcap, ull *qlen)
+__device__ __forceinline__ void pairgroup_stage1(const GraphDev &g, const TestParams &tp, const float *C32, const double *C64, int ldc,
+                                                 ull *queue, ull qcap, ull *qlen)
+{
+    __shared__ unsigned sep_all[PG_THREADS / 32][PG1_PAIRS];   // first separating set found of each pair
+    __shared__ uint2 list_all[PG_THREADS / 32][64];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned *sep_s = sep_all[w];
+    uint2 *list = list_all[w];
+    LaneAcc acc = {};
+    unsigned fast_tests = 0;
+    const int p = g.p;
+    const ull nitems = g.wo_off[p];
+    ull nxt = 0;
+    if (lane == 0) nxt = atomicAdd(&g.info->pair_next, 1ull);
+    for (;;) {
+        const ull it = __shfl_sync(0xffffffffu, nxt, 0);
+        if (it >= nitems) break;
+        if (lane == 0) nxt = atomicAdd(&g.info->pair_next, 1ull);     // needed after this group
+        const int u = warp_owner(g.wo_off, p, it);
+        const int dg = g.deg[u], vg = pair_group(1, dg);
+        const int j0 = (int)(it - g.wo_off[u]) * vg, nv = min(vg, dg - j0);
+        if (PROP && stage_prop(g, 1) && g.row_off[u + 1] > g.row_off[u]) {
+            for (int vi = 0; vi < nv; ++vi)
+                pair_by_warp<1, PROP>(g, tp, C32, ldc, u, j0 + vi, queue, qcap, qlen, acc);
+            continue;
+        }
+        const int *nb = g.nbr + nidx(g, u);
+        const float *Cu = C32 + cidx(tp.prow, ldc, u, 0);
+        const float *Cv[PG1_PAIRS];
+        float cuv[PG1_PAIRS];
+        __syncwarp();
+        if (lane < nv) sep_s[lane] = 0xffffffffu;
+#pragma unroll
+        for (int vi = 0; vi < PG1_PAIRS; ++vi) {
+            const int v = nb[j0 + min(vi, nv - 1)];
+            Cv[vi] = C32 + cidx(tp.prow, ldc, v, 0);
+            cuv[vi] = __ldg(Cu + v);
+        }
+        // the keys of the lane's pair, for the separations found from the other side (u > v:
+        // the keys of side u < v come first)
+        const ull *bp = nullptr;
+        if (lane < nv && u > nb[j0 + lane]) bp = g.best + pidx(g, nb[j0 + lane], u);
+        __syncwarp();
+        const float sqf = sqrtf((float)(n_of(tp, u) - 4)), rq = tanhf(tp.qf / sqf);
+        const float g0 = (float)tp.band / sqf + 8.0f * EPS32;
+        bool other = false;
+        int nlist = 0;
+        int s = nb[min(lane, dg - 1)];
+        for (int base = 0; base < dg; base += 32) {
+            const int i = base + lane;
+            const bool valid = i < dg;
+            if (bp && (base & 96) == 0) other = *(volatile const ull *)bp < (1ull << 62);
+            const unsigned alive = __ballot_sync(0xffffffffu, lane < nv && !other &&
+                                                                  sep_s[lane & (PG1_PAIRS - 1)] > (unsigned)base);
+            if (!alive) break;
+            float b[PG1_PAIRS];
+            const float wu = __ldg(Cu + s);
+#pragma unroll
+            for (int vi = 0; vi < PG1_PAIRS; ++vi) b[vi] = (alive >> vi) & 1u ? __ldg(Cv[vi] + s) : 0.f;
+            s = nb[min(i + 32, dg - 1)];                  // the next round's members
+            const float h11 = fmaf(-wu, wu, 1.0f);
+            const PairBound<1> pb(tp, rq, g0, 1.0f, 0.f, h11, 1.0f + fabsf(wu), valid);
+#pragma unroll
+            for (int vi = 0; vi < PG1_PAIRS; ++vi) {
+                if (!((alive >> vi) & 1u)) continue;
+                const float h22 = fmaf(-b[vi], b[vi], 1.0f), h12 = fmaf(-wu, b[vi], cuv[vi]);
+                const bool dep = pb.dependent(h22, h12);
+                fast_tests += dep;
+                const bool put = !dep && valid && i != j0 + vi;
+                if (__any_sync(0xffffffffu, put))
+                    pair_group_put<1>(g, tp, C32, C64, ldc, u, j0, dg, list, nlist, put,
+                                      put && pb.independent(h22, h12), (unsigned)i, vi, sep_s, sqf, rq, queue,
+                                      qcap, qlen, acc);
+            }
+            if (nlist >= 16) {                            // (the rest after the last round)
+                pair_group_listed<1>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
+                __syncwarp();
+                nlist = 0;
+            }
+        }
+        if (nlist) pair_group_listed<1>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
+    }
+    pair_group_flush(acc, fast_tests, flops_direct(1), g.ctr);
+}
+
+// Stage 2: a CTA per group of up to PG_PAIRS pairs, their rows corr[v, adj(u)] in shared
+// memory.  The first PG_FIRST sets, where most of the pairs that separate do, are walked
+// by each warp for its share of the pairs, 32 sets at a time; the further sets of the
+// pairs left are split over the warps.
+template <bool PROP>
+__device__ __forceinline__ void pairgroup_stage2(const GraphDev &g, const TestParams &tp, const float *C32, const double *C64, int ldc,
+                                                 ull *queue, ull qcap, ull *qlen)
+{
+    extern __shared__ __align__(16) float pg_rows[];
+    constexpr int NW = PG_THREADS / 32;
+    __shared__ unsigned sep_s[PG_PAIRS];                 // first separating set found of each pair
+    __shared__ float cuv_s[PG_PAIRS];
+    __shared__ uint2 list_all[NW][64];
+    __shared__ ull item_s;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint2 *list = list_all[w];
+    LaneAcc acc = {};
+    unsigned fast_tests = 0;
+    const int p = g.p;
+    const ull nitems = g.wo_off[p];
+    ull nxt = 0;
+    if (threadIdx.x == 0) nxt = atomicAdd(&g.info->pair_next, 1ull);
+    for (;;) {
+        __syncthreads();                                 // the last group's tests are done with the rows
+        if (threadIdx.x == 0) {
+            item_s = nxt;
+            nxt = atomicAdd(&g.info->pair_next, 1ull);   // needed after this group
+        }
+        __syncthreads();
+        const ull it = item_s;
+        if (it >= nitems) break;
+        const int u = warp_owner(g.wo_off, p, it);
+        const int dg = g.deg[u], vg = pair_group(2, dg);
+        const int j0 = (int)(it - g.wo_off[u]) * vg, nv = min(vg, dg - j0);
+        if ((PROP && stage_prop(g, 2) && g.row_off[u + 1] > g.row_off[u]) || dg > PG_FLOATS) {
+            for (int vi = w; vi < nv; vi += NW)
+                pair_by_warp<2, PROP>(g, tp, C32, ldc, u, j0 + vi, queue, qcap, qlen, acc);
+            continue;
+        }
+        const int *nb = g.nbr + nidx(g, u);
+        const float *Cu = C32 + cidx(tp.prow, ldc, u, 0);
+        if (threadIdx.x < nv) {
+            sep_s[threadIdx.x] = 0xffffffffu;
+            cuv_s[threadIdx.x] = __ldg(Cu + nb[j0 + threadIdx.x]);
+        }
+        for (int vi = w; vi < nv; vi += NW) {
+            const float *Cv = C32 + cidx(tp.prow, ldc, nb[j0 + vi], 0);
+            for (int i = lane; i < dg; i += 32) pg_rows[vi * dg + i] = __ldg(Cv + nb[i]);
+        }
+        __syncthreads();
+        const float sqf = sqrtf((float)(n_of(tp, u) - 5)), rq = tanhf(tp.qf / sqf);
+        const float g0 = (float)tp.band / sqf + 8.0f * EPS32;
+        // the keys of the lane's pair, for the separations found from the other side (u > v:
+        // the keys of side u < v come first)
+        const ull *bp = nullptr;
+        if (lane < nv && u > nb[j0 + lane]) bp = g.best + pidx(g, nb[j0 + lane], u);
+        bool other = false;
+        int nlist = 0;
+        const int share = (nv + NW - 1) / NW;
+        for (int ph = 0; ph < 2; ++ph) {
+            if (ph) __syncthreads();
+            const bool mine = lane < nv && (ph || (lane >= w * share && lane < (w + 1) * share));
+            int q0 = 0, q1 = 1;
+            lex2_advance(q0, q1, ph ? PG_FIRST + w * 32 + lane : lane, dg);
+            for (int rd = 0; ph || rd < PG_FIRST / 32; ++rd) {
+                const bool valid = q0 < dg - 1;
+                const int i0 = valid ? q0 : 0, i1 = valid ? q1 : 1;
+                const unsigned key = (unsigned)i0 << 16 | (unsigned)i1;
+                if (!__shfl_sync(0xffffffffu, (int)valid, 0)) break;      // lane 0 has the first set
+                const unsigned first = __shfl_sync(0xffffffffu, key, 0);
+                if (bp && mine && (rd & 3) == 0) other = *(volatile const ull *)bp < (1ull << 62);
+                const unsigned alive = __ballot_sync(0xffffffffu, mine && !other &&
+                                                                      *(volatile unsigned *)(sep_s + lane) > first);
+                if (!alive) break;
+                // what depends on u and the set
+                const int s0 = nb[i0], s1 = nb[i1];
+                const float c = __ldg(C32 + cidx(tp.prow, ldc, s0, 0) + s1), a0 = __ldg(Cu + s0);
+                const float x = fmaf(-c, c, 1.0f), rx = rcp_fast(fmaxf(x, 1e-30f));
+                const float wu = fmaf(-a0, c, __ldg(Cu + s1));
+                const float h11 = fmaf(-wu * rx, wu, fmaf(-a0, a0, 1.0f));
+                const PairBound<2> pb(tp, rq, g0, x, c, h11, 1.0f + fabsf(a0) + fabsf(wu) * rx * (1.0f + fabsf(c)),
+                                      valid);
+                for (unsigned m = alive; m; m &= m - 1) {
+                    const int vi = __ffs(m) - 1;
+                    const float b0 = pg_rows[vi * dg + i0], b1 = pg_rows[vi * dg + i1];
+                    const float cv = fmaf(-b0, c, b1), t = cv * rx;
+                    const float h22 = fmaf(-cv, t, fmaf(-b0, b0, 1.0f));
+                    const float h12 = fmaf(-t, wu, fmaf(-a0, b0, cuv_s[vi]));
+                    const bool dep = pb.dependent(h22, h12);
+                    fast_tests += dep;
+                    const bool put = !dep && valid && i0 != j0 + vi && i1 != j0 + vi;
+                    if (__any_sync(0xffffffffu, put))
+                        pair_group_put<2>(g, tp, C32, C64, ldc, u, j0, dg, list, nlist, put,
+                                          put && pb.independent(h22, h12), key, vi, sep_s, sqf, rq, queue, qcap,
+                                          qlen, acc);
+                }
+                if (nlist >= 16 || (nlist && (rd & 7) == 7)) {
+                    pair_group_listed<2>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
+                    __syncwarp();
+                    nlist = 0;
+                }
+                lex2_advance(q0, q1, ph ? PG_THREADS : 32, dg);
+            }
+        }
+        if (nlist) pair_group_listed<2>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
+    }
+    pair_group_flush(acc, fast_tests, flops_direct(2), g.ctr);
+}
+
+template <bool PROP>
+__global__ void __launch_bounds__(PG_THREADS, 4) ci_pairgroup_kernel(GraphDev g, TestParams tp, const float *C32,
+                                                                     const double *C64, int ldc, ull *queue, ull qcap, ull *qlen)
 {
     if (stopped(g.info)) return;
     const int l = g.info->l;
     if (tp.precision == 0 || l < 1 || l > PAIRWARP_LMAX || g.wo_off[g.p] == 0) return;
-    if (l == 1) pairwarp_dispatch<1, PROP>(g, tp, C32, ldc, queue, qcap, qlen);
-    else pairwarp_dispatch<2, PROP>(g, tp, C32, ldc, queue, qcap, qlen);
+    if (l == 1) pairgroup_stage1<PROP>(g, tp, C32, C64, ldc, queue, qcap, qlen);
+    else pairgroup_stage2<PROP>(g, tp, C32, C64, ldc, queue, qcap, qlen);
 }
 
 // FP64 pass over the queued tests of the lane kernel (one warp per test).
@@ -3093,13 +3521,16 @@ static int node_blocks_per_sm(size_t smem)
 }
 
 template <int LO, int HI, bool PROP>
-static void lane_launch_p(GraphDev g, TestParams tp, const float *C32, int ldc, ull *queue, ull qcap, ull *qlen,
+static void lane_launch_p(GraphDev g, TestParams tp, const float *C32, const double *C64, int ldc, ull *queue, ull qcap, ull *qlen,
                           cudaStream_t s)
 {
     ci_lane_kernel<LO, HI, PROP><<<num_sms() * tp.lane_blocks, 256, 0, s>>>(g, tp, C32, ldc, queue, qcap, qlen);
     note_launch();
     if (LO <= PAIRWARP_LMAX && tp.pair_warp) {
-        ci_pairwarp_kernel<PROP><<<num_sms() * 4, 256, 0, s>>>(g, tp, C32, ldc, queue, qcap, qlen);
+        cudaFuncSetAttribute(ci_pairgroup_kernel<PROP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(PG_FLOATS * sizeof(float)));
+        ci_pairgroup_kernel<PROP><<<num_sms() * 4, PG_THREADS, PG_FLOATS * sizeof(float), s>>>(g, tp, C32, C64, ldc,
+                                                                                               queue, qcap, qlen);
         note_launch();
     }
     if (HI >= 1 && tp.node_dmax > 0) {
@@ -3112,11 +3543,11 @@ static void lane_launch_p(GraphDev g, TestParams tp, const float *C32, int ldc, 
 }
 
 template <int LO, int HI>
-static void lane_launch(GraphDev g, TestParams tp, const float *C32, int ldc, ull *queue, ull qcap, ull *qlen,
+static void lane_launch(GraphDev g, TestParams tp, const float *C32, const double *C64, int ldc, ull *queue, ull qcap, ull *qlen,
                         bool prop, cudaStream_t s)
 {
-    if (prop) lane_launch_p<LO, HI, true>(g, tp, C32, ldc, queue, qcap, qlen, s);
-    else lane_launch_p<LO, HI, false>(g, tp, C32, ldc, queue, qcap, qlen, s);
+    if (prop) lane_launch_p<LO, HI, true>(g, tp, C32, C64, ldc, queue, qcap, qlen, s);
+    else lane_launch_p<LO, HI, false>(g, tp, C32, C64, ldc, queue, qcap, qlen, s);
 }
 
 cudaError_t launch_ci_lane(GraphDev g, TestParams tp, const float *C32, const double *C64, int ldc,
@@ -3125,12 +3556,12 @@ cudaError_t launch_ci_lane(GraphDev g, TestParams tp, const float *C32, const do
 {
     cudaError_t e = cudaMemsetAsync(qlen, 0, sizeof(ull), s);
     if (e != cudaSuccess) return e;
-    if (range < 0 || range == 0) lane_launch<0, 2>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
-    if (range < 0 || range == 1) lane_launch<3, 4>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
-    if (range < 0 || range == 2) lane_launch<5, 6>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
-    if (range < 0 || range == 3) lane_launch<7, 8>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
-    if (range < 0 || range == 4) lane_launch<9, 10>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
-    if (range < 0 || range == 5) lane_launch<11, 12>(g, tp, C32, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 0) lane_launch<0, 2>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 1) lane_launch<3, 4>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 2) lane_launch<5, 6>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 3) lane_launch<7, 8>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 4) lane_launch<9, 10>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
+    if (range < 0 || range == 5) lane_launch<11, 12>(g, tp, C32, C64, ldc, queue, qcap, qlen, prop, s);
     int ms, per_warp, wpc;
     direct_shape(LANE_LMAX + 2, ms, per_warp, wpc);
     size_t smem = (size_t)wpc * per_warp;
