@@ -2,6 +2,7 @@
 // corr = Xs^T Xs / n (Sec. 4, the matrix corr): FP64 column statistics, FP64
 // and FP32 Gram kernels on the CUDA cores, and the FP64 -> FP32 cast.
 #include "internal.h"
+#include <type_traits>
 #include "device_util.cuh"
 #include <cuda_bf16.h>
 #include <algorithm>
@@ -158,7 +159,9 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
                              double *C, long long ldc, int *err)
 {
     __shared__ double red[CS_WARPS][33];
-    __shared__ double part[2][32];                       // this CTA's sums of the two passes
+    __shared__ float redm[CS_WARPS][33];
+    __shared__ double part[3][32];                       // this CTA's sums of the passes
+    __shared__ float partm[32];                          // its largest |x| (FP32 input)
     cg::cluster_group cl = cg::this_cluster();
     const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int col = blockIdx.x * 32 + tx;
@@ -183,21 +186,36 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
         return s;
     };
     double v = 0.0;
-    if constexpr (sizeof(T) == 4) {
+    float sc = 1.f;                                      // FP32: the power of two that brings the column near 1
+    float am = 0.f;
+    // the warp's sum of sc x (FP32 input), am its largest |x|
+    auto sum32 = [&](auto scaled) -> double {
         float hi = 0.f, lo = 0.f;
         for (long long r = r0; r < n; r += 8 * step) {
             float f[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : 0.f;
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? (float)__ldg(x + (r + u * step) * ld) : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 float e;
+                if constexpr (scaled.value) f[u] = __fmul_rn(sc, f[u]);
+                else am = fmaxf(am, fabsf(f[u]));
                 two_sum_f(hi, f[u], hi, e);
                 lo = __fadd_rn(lo, e);
                 if (u & 1) two_sum_f(hi, lo, hi, lo);
             }
         }
-        v = f2d(hi) + f2d(lo);
+        return f2d(hi) + f2d(lo);
+    };
+    if constexpr (sizeof(T) == 4) {
+        v = sum32(std::false_type{});
+        redm[w][tx] = am;                                // published with the sums (total)
+        __syncthreads();
+        if (w == 1) {
+            float m = 0.f;
+            for (int k = 0; k < CS_WARPS; ++k) m = fmaxf(m, redm[k][tx]);
+            partm[tx] = m;
+        }
     } else {
         double s0 = 0.0, s1 = 0.0;
         for (long long r = r0; r < n; r += 8 * step) {
@@ -212,20 +230,31 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
         }
         v = s0 + s1;
     }
-    const double mu = total(v, 0) / (double)n;
+    double mu = total(v, 0) / (double)n;
     double m2;
     if constexpr (sizeof(T) == 4) {
-        const float mh = (float)mu;
+        // The squares are taken of the column scaled by a power of two (their FP32 products
+        // neither overflow nor underflow whatever the column's units); a column whose plain sum
+        // may have overflowed is summed again scaled.
+        float m = 0.f;
+        for (int k = 0; k < CS_CLUSTER; ++k) m = fmaxf(m, cl.map_shared_rank(&partm[0], k)[tx]);
+        sc = __int_as_float(min(254, max(1, 254 - (__float_as_int(m) >> 23))) << 23);
+        mu *= (double)sc;
+        if (__syncthreads_or(m >= 0x1p90f)) {             // the same in every CTA of the cluster
+            const double ms = total(sum32(std::true_type{}), 2) / (double)n;
+            if (m >= 0x1p90f) mu = ms;
+        }
+        const float mr = (float)(mu / (double)sc), mh = __fmul_rn(sc, mr);
         double Q = 0.0;
         for (long long r = r0; r < n; r += 8 * step) {
             float f[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? __ldg(x + (r + u * step) * ld) : mh;
+            for (int u = 0; u < 8; ++u) f[u] = ok && r + u * step < n ? (float)__ldg(x + (r + u * step) * ld) : mr;
             float hi = 0.f, lo = 0.f, sm = 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {                // (f - mh)^2 exactly, a missing row adds 0
                 float sd, e, ee;
-                two_sum_f(f[u], -mh, sd, e);
+                two_sum_f(__fmul_rn(sc, f[u]), -mh, sd, e);
                 const float pp = __fmul_rn(sd, sd), pe = __fmaf_rn(sd, sd, -pp);
                 sm = __fadd_rn(sm, __fmaf_rn(e, e, __fmaf_rn(__fmul_rn(2.f, sd), e, pe)));
                 two_sum_f(hi, pp, hi, ee);
@@ -251,9 +280,9 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
         m2 = total(q0 + q1, 1);
     }
     if (cl.block_rank() == 0 && w == 0 && ok) {
-        const double var = m2 / (double)n;
-        mean[col] = mu;
-        rsd[col] = var > 0.0 ? 1.0 / sqrt(var) : 0.0;    // constant column -> zero column
+        const double var = m2 / (double)n, us = (double)sc;
+        mean[col] = mu / us;
+        rsd[col] = var > 0.0 ? us / sqrt(var) : 0.0;     // constant column -> zero column
     }
     cl.sync();                                           // no CTA leaves while another reads its sums
 }

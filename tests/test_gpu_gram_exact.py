@@ -92,3 +92,18 @@ def test_non_finite_columns(fp):                                         # noqa:
 def test_repeatable(fp):                                                 # noqa: F811
     X = np.random.default_rng(5).standard_normal((5000, 200)).astype(np.float32)
     assert np.array_equal(_run(fp, X), _run(fp, X))      # integer accumulation: any order, the same bits
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_fixed_point_limits(fp, dtype):                                  # noqa: F811
+    """FP32 input: columns on both sides of the limits of the 32-bit fixed point (|mean| against
+    8 sqrt(n) sd, 2^s a normal FP32 number), next to each other in a group of 8 columns."""
+    rng = np.random.default_rng(17)
+    n, p = 500, 40
+    X = rng.standard_normal((n, p)) @ (np.eye(p) + 0.3 * rng.standard_normal((p, p)))
+    sd = X.std(0)
+    X += np.sqrt(n) * sd * np.where(np.arange(p) < 16, 2.0 ** (np.arange(p) % 16 - 8), 0.0)
+    X[:, 16:24] += np.sqrt(n) * sd[16:24] * np.array([3.9, 4.1, 7.9, 8.1, -3.9, -4.1, -7.9, -8.1])
+    X[:, 24:32] *= 10.0 ** np.array([-32, -28, -24, -20, 20, 25, 30, 34])
+    X = X.astype(dtype)
+    np.testing.assert_allclose(_run(fp, X), _want(X), rtol=0, atol=TOL)
