@@ -867,7 +867,7 @@ static pc_status ensure_c32tc(pc_handle *h)
 // them (the reversed order) or they cost no more than the split-precision product with its
 // planes and the FP64 entries formed on demand: problems of p <= NL_PMAX, and batches of
 // instances of p <= EXACT_BATCH_PMAX, whose products fill the chip side by side
-// (64 instances of 50-400 variables and 2000-20000 samples: 6.3 ms for 3.1 with the
+// (64 instances of 50-400 variables and 2000-20000 samples: 4.5 ms for 3.1 with the
 // split-precision product, and in return the search takes 8-9 ms for 19-66, its FP64 tests
 // being decided on the spot instead of queued, their entries formed and re-read).
 static bool exact_corr(const pc_handle *h)
