@@ -180,8 +180,8 @@ __device__ void tail_body(GraphDev g, TestParams tp, int cap, int mode, const in
                           bool fused)
 {
     LevelInfo *I = g.info;
-    __shared__ long long part[1024];
-    __shared__ int smax[1024];
+    __shared__ long long part[32];
+    __shared__ int smax[32];
     __shared__ int sh_l, sh_go, sh_need, sh_removed;
     const int p = g.p, t = threadIdx.x;
     if (mode == 0 && t == 0) I->body_runs++;
@@ -193,42 +193,53 @@ __device__ void tail_body(GraphDev g, TestParams tp, int cap, int mode, const in
         return;
     }
     if (t == 0) sh_need = 0;
-    const int nth = blockDim.x;                          // 32..1024, a multiple of 32
-    const int per = (p + nth - 1) / nth;
-    const int s0 = min(p, t * per), s1 = min(p, s0 + per);
+    // a run of nodes per warp, its lanes on neighbouring nodes (coalesced; the sums of a run
+    // first, then its prefixes; with a run of nodes per thread the kernel took 49 us at 15000 nodes, 37 so)
+    const int nw = blockDim.x >> 5, w = t >> 5, lane = t & 31;      // 32..1024 threads
+    const int per = ((p + nw - 1) / nw + 31) / 32 * 32;
+    const int s0 = min(p, w * per), s1 = min(p, s0 + per);
     long long sum = 0;
     int mx = 0;
-    for (int i = s0; i < s1; ++i) {
+#pragma unroll 8
+    for (int i = s0 + lane; i < s1; i += 32) {
         const int dg = __ldcg(g.deg + i);
         sum += dg;
         mx = max(mx, dg);
     }
-    part[t] = sum;
-    smax[t] = mx;
-    __syncthreads();
-    for (int off = 1; off < nth; off <<= 1) {
-        long long v = (t >= off) ? part[t - off] : 0;
-        int m2 = (t >= off) ? smax[t - off] : 0;
-        __syncthreads();
-        part[t] += v;
-        smax[t] = max(smax[t], m2);
-        __syncthreads();
+    for (int off = 16; off > 0; off >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     }
-    long long run = part[t] - sum;
-    for (int i0 = s0; i0 < s1; i0 += 8) {              // batches of independent loads, then the stores
-        int dv[8];
+    if (lane == 0) {
+        part[w] = sum;
+        smax[w] = mx;
+    }
+    __syncthreads();
+    long long run = 0;
+    for (int k = 0; k < w; ++k) run += part[k];
+    for (int i0 = s0; i0 < s1; i0 += 128) {              // batches of independent loads
+        int dv[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) dv[k] = i0 + k < s1 ? __ldcg(g.deg + i0 + k) : 0;
+        for (int k = 0; k < 4; ++k) dv[k] = i0 + 32 * k + lane < s1 ? __ldcg(g.deg + i0 + 32 * k + lane) : 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (i0 + k < s1) {
-                g.ooff[i0 + k] = run;
-                run += dv[k];
+        for (int k = 0; k < 4; ++k) {
+            int incl = dv[k];                            // 32 degrees: below 2^31
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
             }
+            if (i0 + 32 * k + lane < s1) g.ooff[i0 + 32 * k + lane] = run + incl - dv[k];
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
     }
     if (t == 0) {
-        const long long tot = part[nth - 1];
-        const int lstar = smax[nth - 1] - 1;              // -1 when no edge is left
+        long long tot = 0;
+        int lstar = 0;
+        for (int k = 0; k < nw; ++k) {
+            tot += part[k];
+            lstar = max(lstar, smax[k]);
+        }
+        --lstar;                                         // -1 when no edge is left
         g.ooff[p] = tot;
         I->n_opairs = tot;
         sh_removed = I->edges != (unsigned long long)tot;   // the commit deleted edges
@@ -306,7 +317,7 @@ __global__ void __launch_bounds__(1024) tail_kernel(GraphDev g, TestParams tp, i
 __device__ __forceinline__ ull sat_mul(ull a, ull b)
 {
     if (a == 0 || b == 0) return 0;
-    if (a == KEY_NONE || b == KEY_NONE || a > KEY_NONE / b) return KEY_NONE;
+    if (a == KEY_NONE || b == KEY_NONE || __umul64hi(a, b)) return KEY_NONE;
     return a * b;
 }
 
@@ -370,74 +381,97 @@ __device__ __forceinline__ void block_scan_sat(const ull (&v)[NV], ull (&ex)[NV]
 
 // Work of stage l per node u: every ordered pair (u, v) has C(d, l) tests,
 // d = |adj(u)| - 1, all on the direct path or all on the complement path.
-// One CTA scans the per-node totals into tn_off / cn_off and gates the stage:
+// The first CTA scans the per-node totals into tn_off / cn_off and gates the stage:
 // budget and saturation (PC_ERR_BUDGET), or direct tests at an l larger than
 // the direct kernel's shared-memory layout (the host runs that stage).  In the
 // stages of the small-stage kernel it also lays out its rank-major rounds.
-constexpr int HEAD_PER_MAX = MAXP_BATCH / 1024;           // nodes per thread at most
+// The other CTAs write the owner node of every ordered pair (the small-stage kernel's work
+// items; the commit), a warp per node.
+// A thread takes one node of each block of nodes, so that loads and stores are coalesced, and
+// the scan carries over the blocks.  Bound by latency: at 15000 nodes 145 us with a run of 15
+// nodes per thread (32 sectors a store), 85 here; at 1000 nodes 21 us (100 with every pair
+// alive, the owners written by the same CTA), 15 here.
 __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, double budget, int mmax_direct,
                                           const StageConds &conds)
 {
     LevelInfo *I = g.info;
+    const int p = g.p, t = threadIdx.x, nth = blockDim.x;
+    if (blockIdx.x > 0) {
+        if (stopped(I)) return;
+        const int nw = (int)(gridDim.x - 1) * (nth >> 5);
+        for (int u = (int)(blockIdx.x - 1) * (nth >> 5) + (t >> 5); u < p; u += nw) {
+            const long long b = g.ooff[u];
+            const int dg = g.deg[u];
+            for (int jj = t & 31; jj < dg; jj += 32) g.opu[b + jj] = u;
+        }
+        return;
+    }
     if (stopped(I)) {
         if (conds.use && threadIdx.x == 0) set_stage_conds(conds, I, LANE_RANGES, 0, 0, 0, 0);
         return;
     }
     __shared__ ull sh[6 * 32];                           // scratch of block_scan_sat<6>
-    const int p = g.p, l = I->l, t = threadIdx.x;
-    const int per = (p + (int)blockDim.x - 1) / (int)blockDim.x;   // <= HEAD_PER_MAX
-    const int s0 = min(p, t * per), s1 = min(p, s0 + per);
-    // tests per pair of each of this thread's nodes; 0 for complement-path nodes' direct count
-    ull Tn[HEAD_PER_MAX];
-    bool cm[HEAD_PER_MAX];
-    // each node's staged work items and degree, formed once (64-bit divisions)
-    ull Ik[HEAD_PER_MAX];
-    int Dg[HEAD_PER_MAX];
+    const int l = I->l;
+    const bool small = tp.lane_stages && tp.precision != 0 && l <= LANE_LMAX;
+    // what node u has at this stage: T tests per pair (0: none), complement path or direct,
+    // the staged kernel's work items (consecutive ranges of NODE_ITEM_CHUNKS chunks of its
+    // rank-major chunk space, chunk r of every pair before r+1), pair groups
+    struct Node {
+        int dg;
+        ull T, items, groups;
+        bool comp;
+    };
+    auto node = [&](int u) -> Node {
+        Node k = {0, 0ull, 0ull, 0ull, false};
+        if (u >= p) return k;
+        const int dg = g.deg[u], d = dg - 1;
+        k.dg = dg;
+        k.T = (dg > 0 && d >= l && dof_ok(tp, u, l)) ? g.binom[(long long)d * g.ldb + l] : 0ull;
+        if (!k.T) return k;
+        k.comp = comp_eligible(d, l, tp) && g.prec_m[u] > 0;
+        if (k.comp || !small) return k;
+        if (node_staged(tp, l, dg)) {
+            const ull ch = node_chunk(tp, k.T, dg);
+            const ull r = (k.T >> 32) == 0 ? (ull)(((unsigned)k.T - 1u) / (unsigned)ch) + 1ull : (k.T + ch - 1) / ch;
+            const ull nc = sat_mul(r, (ull)dg);
+            k.items = nc == KEY_NONE ? KEY_NONE : (nc + NODE_ITEM_CHUNKS - 1) / NODE_ITEM_CHUNKS;
+        } else if (pair_warped(tp, l, dg)) {
+            k.groups = (ull)pair_groups(l, dg);
+        }
+        return k;
+    };
     // proposal rows: a direct-path node whose pairs have at least two sets to order
     // gets deg*(deg-1) score rows (pair j, candidate position x); the complement path
     // (dropped sets of at most KC_MAX members, reverse-lexicographic) keeps the plain order
-    auto prows = [&](int dg, ull T) -> ull {
-        return (g.row_off && l >= 1 && l <= tp.learned_lmax && T >= 2) ? (ull)dg * (ull)(dg - 1) : 0ull;
+    auto prows = [&](const Node &k) -> ull {
+        return (g.row_off && l >= 1 && l <= tp.learned_lmax && k.T >= 2 && !k.comp) ? (ull)k.dg * (ull)(k.dg - 1) : 0ull;
     };
-    const bool small = tp.lane_stages && tp.precision != 0 && l <= LANE_LMAX;
-    // staged kernel work items of a node: consecutive ranges of NODE_ITEM_CHUNKS
-    // chunks of its rank-major chunk space (chunk r of every pair before r+1)
-    auto items = [&](int dg, ull T) -> ull {
-        if (!small || !T || !node_staged(tp, l, dg)) return 0ull;
-        const ull ch = node_chunk(tp, T, dg);
-        const ull nc = sat_mul((T + ch - 1) / ch, (ull)dg);
-        return nc == KEY_NONE ? KEY_NONE : (nc + NODE_ITEM_CHUNKS - 1) / NODE_ITEM_CHUNKS;
-    };
-    // pair-group kernel: the pairs of the larger direct nodes of stages 1-2
-    auto warp_mode = [&](int dg, ull T) -> bool { return small && T && pair_warped(tp, l, dg); };
-    // direct, complement, proposal rows, staged nodes (their first items), the
-    // staged nodes' further items, pair groups
-    ull v[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull}, mxT = 0;
+    // totals before this block of nodes: direct, complement, proposal rows, staged nodes
+    // (their first items), the staged nodes' further items, pair groups
+    ull tot[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull}, mxT = 0;
     bool sat = false;
-    for (int u = s0; u < s1; ++u) {
-        const int dg = g.deg[u], d = dg - 1;
-        const ull T = (dg > 0 && d >= l && dof_ok(tp, u, l)) ? g.binom[(long long)d * g.ldb + l] : 0ull;
-        const ull tot = sat_mul(T, (ull)dg);
-        sat |= tot == KEY_NONE;
-        const bool comp = T && comp_eligible(d, l, tp) && g.prec_m[u] > 0;
-        Tn[u - s0] = T;
-        cm[u - s0] = comp;
-        Dg[u - s0] = dg;
-        const ull k = comp ? 0ull : items(dg, T);
-        Ik[u - s0] = k;
-        if (comp) v[1] = sat_add(v[1], tot);
-        else {
-            v[0] = sat_add(v[0], tot);
-            if (!k && !warp_mode(dg, T)) mxT = T > mxT ? T : mxT;   // the lane kernel's pairs only
-            v[2] = sat_add(v[2], prows(dg, T));           // complement-path pairs keep the plain order
-            v[3] += k ? 1ull : 0ull;
-            v[4] = sat_add(v[4], k ? k - 1 : 0ull);
-            v[5] += warp_mode(dg, T) ? (ull)pair_groups(l, dg) : 0ull;
+    for (int u0 = 0; u0 < p; u0 += nth) {
+        const int u = u0 + t;
+        const Node k = node(u);
+        const ull all = sat_mul(k.T, (ull)k.dg);
+        sat |= all == KEY_NONE;
+        const ull v[6] = {k.comp ? 0ull : all, k.comp ? all : 0ull, prows(k), k.items ? 1ull : 0ull,
+                          k.items ? k.items - 1 : 0ull, k.groups};
+        if (!k.comp && !k.items && !k.groups) mxT = k.T > mxT ? k.T : mxT;   // the lane kernel's pairs only
+        ull ex[6], bt[6];
+        block_scan_sat<6>(v, ex, bt, sh);
+        if (u < p) {
+            g.tn_off[u] = sat_add(tot[0], ex[0]);
+            g.cn_off[u] = sat_add(tot[1], ex[1]);
+            if (g.row_off) g.row_off[u] = sat_add(tot[2], ex[2]);
+            g.ia_off[u] = sat_add(tot[3], ex[3]);
+            g.it_off[u] = sat_add(tot[4], ex[4]);
+            g.wo_off[u] = sat_add(tot[5], ex[5]);
         }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) tot[i] = sat_add(tot[i], bt[i]);
     }
     const int ssat = __syncthreads_or(sat);
-    ull ex[6], tot[6];
-    block_scan_sat<6>(v, ex, tot, sh);
     // else: plain order this stage (too many rows, or too few tests for the order to matter)
     // score rows are one per candidate; the order pays off only when a pair has
     // many more sets than candidates (l >= 2 and large neighbourhoods)
@@ -446,43 +480,8 @@ __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, 
                           tests_all >= tp.learned_ratio * (double)tot[2];
     const ull rows_total = tot[2];
     if (t == 0 && g.scored) g.scored[l] = rows_fit && rows_total > 0;
-    {
-        ull rd = ex[0], rc = ex[1], rr = ex[2], ra = ex[3], ri = ex[4], rw = ex[5];
-        for (int u = s0; u < s1; ++u) {
-            const int dg = Dg[u - s0];
-            const ull T = Tn[u - s0], tt = sat_mul(T, (ull)dg);
-            g.tn_off[u] = rd;
-            g.cn_off[u] = rc;
-            g.ia_off[u] = ra;
-            g.it_off[u] = ri;
-            g.wo_off[u] = rw;
-            if (g.row_off) g.row_off[u] = rows_fit ? rr : 0ull;
-            if (cm[u - s0]) rc = sat_add(rc, tt);
-            else {
-                rd = sat_add(rd, tt);
-                rr = sat_add(rr, prows(dg, T));
-                const ull k = Ik[u - s0];
-                ra += k ? 1ull : 0ull;
-                ri = sat_add(ri, k ? k - 1 : 0ull);
-                rw += (!cm[u - s0] && warp_mode(dg, T)) ? (ull)pair_groups(l, dg) : 0ull;
-            }
-        }
-    }
-    // owner node of every ordered pair (the small-stage kernel's work items; the commit):
-    // a warp takes 32 consecutive nodes, each lane loading one node's offset and degree
-    // (one round of loads instead of one per node), then writes the nodes' runs in turn
-    // with consecutive entries per lane group (coalesced stores)
-    for (int u0 = (t >> 5) * 32; u0 < p; u0 += (int)blockDim.x) {
-        const int ul = u0 + (t & 31);
-        const long long bl = ul < p ? g.ooff[ul] : 0;
-        const int dl = ul < p ? g.deg[ul] : 0;
-        const int nk = min(32, p - u0);
-        for (int k = 0; k < nk; ++k) {
-            const long long b = __shfl_sync(0xffffffffu, bl, k);
-            const int dg = __shfl_sync(0xffffffffu, dl, k);
-            for (int jj = t & 31; jj < dg; jj += 32) g.opu[b + jj] = u0 + k;
-        }
-    }
+    if (g.row_off && !rows_fit)
+        for (int u = t; u < p; u += nth) g.row_off[u] = 0ull;
     int rounds = 0;
     if (small && tot[0] > 0) {
         // rank-major rounds of the lane kernel: at most tp.lane_rounds chunks of
@@ -494,29 +493,23 @@ __device__ __noinline__ void head_body(const GraphDev &g, const TestParams &tp, 
         if ((t & 31) == 0) sh[t >> 5] = mxT;
         __syncthreads();
         ull maxT = 0;
-        for (int i = 0; i < 32; ++i) maxT = sh[i] > maxT && i < ((int)blockDim.x >> 5) ? sh[i] : maxT;
+        for (int i = 0; i < nth >> 5; ++i) maxT = sh[i] > maxT ? sh[i] : maxT;
         __syncthreads();
         const ull chunk = (ull)tp.lane_chunk;
         rounds = (int)(maxT == 0 ? 0 : min((ull)tp.lane_rounds, (maxT + chunk - 1) / chunk));
         const ull skip = (ull)rounds * chunk;
-        ull v2[1] = {0ull};
-        for (int u = s0; u < s1; ++u) {
-            const ull T = Tn[u - s0];
-            const int dg = Dg[u - s0];
-            if (!cm[u - s0] && T > skip && !Ik[u - s0] && !warp_mode(dg, T))
-                v2[0] = sat_add(v2[0], sat_mul(T - skip, (ull)dg));
-        }
-        ull ex2[1], tot2[1];
-        block_scan_sat<1>(v2, ex2, tot2, sh);
-        ull rr2 = ex2[0];
-        for (int u = s0; u < s1; ++u) {
-            const ull T = Tn[u - s0];
-            const int dg = Dg[u - s0];
-            g.rn_off[u] = rr2;
-            if (!cm[u - s0] && T > skip && !Ik[u - s0] && !warp_mode(dg, T))
-                rr2 = sat_add(rr2, sat_mul(T - skip, (ull)dg));
-        }
-        if (t == 0) g.rn_off[p] = tot2[0];
+        ull rest = 0;                                    // rn_off is read only when some pair has a remainder
+        if (maxT > skip)
+            for (int u0 = 0; u0 < p; u0 += nth) {
+                const int u = u0 + t;
+                const Node k = node(u);
+                const ull v[1] = {!k.comp && !k.items && !k.groups && k.T > skip ? sat_mul(k.T - skip, (ull)k.dg) : 0ull};
+                ull ex[1], bt[1];
+                block_scan_sat<1>(v, ex, bt, sh);
+                if (u < p) g.rn_off[u] = sat_add(rest, ex[0]);
+                rest = sat_add(rest, bt[0]);
+            }
+        if (t == 0) g.rn_off[p] = rest;
     }
     __syncthreads();
     if (t == 0) {
@@ -3448,7 +3441,9 @@ cudaError_t launch_tail(GraphDev g, TestParams tp, int cap, int mode, const int 
 
 cudaError_t launch_head(GraphDev g, TestParams tp, double budget, int mmax_direct, StageConds sc, cudaStream_t s)
 {
-    head_kernel<<<1, stage_threads(g.p), 0, s>>>(g, tp, budget, mmax_direct, sc); note_launch();
+    const int threads = stage_threads(g.p);
+    const int owners = std::min(128, (g.p * 32 + threads - 1) / threads);      // CTAs of the owner nodes
+    head_kernel<<<1 + owners, threads, 0, s>>>(g, tp, budget, mmax_direct, sc); note_launch();
     return cudaGetLastError();
 }
 
