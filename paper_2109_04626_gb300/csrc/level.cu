@@ -1771,10 +1771,13 @@ __device__ __forceinline__ void release_byte(unsigned char *flags, long long e)
 }
 
 // One warp per queued test: its node set (as the FP64 pass builds it), then each
-// missing pair (a < b) of it is claimed and listed -- for the first queued test of
-// each tested pair only: a later one runs only if that test does not separate the
+// missing pair (a < b) of it is claimed and listed -- in a long queue for the first queued
+// test of each tested pair only: a later one runs only if that test does not separate the
 // pair, and then forms its entries on demand (dense problems queue many tests per
-// pair, most of which an earlier set decides).
+// pair, most of which an earlier set decides).  A queue of up to COLLECT_ALL tests lists them
+// all: the entries of a test on demand are a serial chain, 20000 samples each (stage 2 of the
+// 1000-node sparse graph, about 800 tests in all: the FP64 pass 315 us with the first tests only, 23 so).
+constexpr ull COLLECT_ALL = 4096;
 __global__ void __launch_bounds__(256) c64_collect_kernel(GraphDev g, TestParams tp, const ull *queue,
                                                           const ull *qlen, ull qcap)
 {
@@ -1799,7 +1802,7 @@ __global__ void __launch_bounds__(256) c64_collect_kernel(GraphDev g, TestParams
         if (*(volatile ull *)(g.best + ep) < key) continue;   // no FP64 test follows
         int first = 0;
         if (lane == 0) first = claim_byte(tp.pair_seen, ep);
-        if (!__shfl_sync(0xffffffffu, first, 0)) continue;    // not the pair's first queued test
+        if (!__shfl_sync(0xffffffffu, first, 0) && nq > COLLECT_ALL) continue;   // not the pair's first queued test
         if (lane == 0) {
             unrank_lex(rank, d, l, g.binom, g.ldb, pos);
             for (int i = 0; i < l; ++i) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
