@@ -190,7 +190,7 @@ __device__ __forceinline__ int fp32_trust(const TestParams &tp, int m, float sqf
     if (dr > tp.dr_max) return 2;
     // |z - q| >= sqf |a - rq| / (1 - min(a, rq)^2) (mean-value theorem on atanh)
     const float gap = fabsf(a - rq), mn = fminf(a, rq);
-    if (gap <= dr || sqf * gap < (float)tp.band * (1.0f - mn * mn)) return 1;
+    if (gap <= dr || sqf * gap < tp.band_f * (1.0f - mn * mn)) return 1;
     return 0;
 }
 

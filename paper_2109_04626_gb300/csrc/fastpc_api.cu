@@ -299,6 +299,8 @@ static TestParams make_tp(const pc_handle *h)
     tp.rq_tab = h->rq_tab;
     tp.band = h->band;
     tp.guard = h->guard;
+    tp.guard_f = (float)h->guard;
+    tp.band_f = (float)h->band;
     tp.eps_c = h->used_tc && !h->c32_rounded ? 1.0e-6f : 1.2e-7f;
     tp.dr_max = 1.0f;            // skeleton: only the decision is returned (no bound on r itself)
     tp.lane_chunk = h->lane_chunk;

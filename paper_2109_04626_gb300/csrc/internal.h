@@ -180,6 +180,7 @@ struct TestParams {
     const double *rq_tab;   // stage l -> tanh(q / sqrt(n - l - 3)) (one problem's n), formed on the host
     double band;        // |z - q| band for FP64 re-decision
     double guard;       // pivot guard
+    float guard_f, band_f;   // both as FP32 (a conversion per test would run on the FP64 pipe)
     float eps_c;        // bound on |C32 - corr| (FP32 GEMM or cast: 2^-23; BF16x3 tensor cores: 1e-6)
     float dr_max;       // largest FP32 error bound on r trusted without FP64: 5e-6 where r is
                         // returned (raw tests); no limit where only the decision is (skeleton)

@@ -555,19 +555,71 @@ __global__ void __launch_bounds__(1024) head_kernel(GraphDev g, TestParams tp, d
     head_body(g, tp, budget, mmax_direct, conds);
 }
 
+// The last u < p with off[u] <= t (off: p + 1 ascending offsets, off[0] = 0 <= t < off[p]),
+// by the whole warp: 32 probes at a time instead of a chain of binary steps.
+__device__ __forceinline__ int warp_owner(const ull *off, int p, ull t)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = p;                                    // the answer lies in [lo, lo + n)
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, i < n && off[lo + min(i, n - 1)] <= t);
+        const int k = 31 - __clz(m);                      // lane 0 always holds
+        lo += k * step;
+        n = min(step, n - k * step);
+    }
+    return lo;
+}
+
 // test index t of the stage -> (u, j, rank): node by the per-node offsets,
 // then j = (t - off[u]) / C(d,l) and rank = (t - off[u]) mod C(d,l)
+// WARP: by the whole warp, t the same in all lanes
+template <bool WARP>
 __device__ __forceinline__ void locate_test(const GraphDev &g, const ull *noff, int l, ull t, int &u,
                                             int &j, int &d, ull &rank)
 {
-    const int p = g.p;
-    u = (int)(upper_bound_dev(noff, (long long)p + 1, t) - 1);
+    if (WARP) u = warp_owner(noff, g.p, t);
+    else u = (int)(upper_bound_dev(noff, (long long)g.p + 1, t) - 1);
     d = g.deg[u] - 1;
     const ull T = g.binom[(long long)d * g.ldb + l];
     const ull w = t - noff[u];
     const ull jj = w / T;
     j = (int)jj;
     rank = w - jj * T;
+}
+
+// unrank_lex by the whole warp, pos in its shared memory: the lanes probe 32 places of a
+// member at once, one round trip to the table instead of a chain of about log2(d) (or of a
+// walk over the places; a stage-13 test of 16 candidates spent most of its time there).
+__device__ __forceinline__ void warp_unrank_lex(ull rank, int d, int l, const ull *binom, int ldb, int *pos)
+{
+    const int lane = threadIdx.x & 31;
+    int x = 0;
+    for (int i = 0; i < l; ++i) {
+        const int r1 = l - i;
+        // C(d - x, r1) sets are left; those whose next place is below y number
+        // C(d - x, r1) - C(d - y, r1): the last y with at most `rank` of them
+        ull target = 0, at = 0, first = 0;
+        int lo = x;
+        for (int y0 = x;; y0 += 32) {
+            const int y = y0 + lane;
+            const ull c = y <= d - r1 ? __ldg(binom + (long long)(d - y) * ldb + r1) : 0ull;
+            if (y0 == x) {
+                first = __shfl_sync(0xffffffffu, c, 0);
+                target = first - rank;
+            }
+            const int k = __popc(__ballot_sync(0xffffffffu, y <= d - r1 && c >= target));
+            if (k > 0) {
+                lo = y0 + k - 1;
+                at = __shfl_sync(0xffffffffu, c, k - 1);
+            }
+            if (k < 32) break;
+        }
+        if (lane == 0) pos[i] = lo;
+        rank -= first - at;
+        x = lo + 1;
+    }
+    __syncwarp();
 }
 
 size_t scan_ws_bytes(long long n) { return 64 + 0 * n; }
@@ -639,16 +691,17 @@ __global__ void __launch_bounds__(256) ci_direct_kernel(GraphDev g, TestParams t
     for (ull t = gw; t < total; t += nw) {
         int u, j, d;
         ull rank;
-        locate_test(g, g.tn_off, l, t, u, j, d, rank);
+        locate_test<true>(g, g.tn_off, l, t, u, j, d, rank);
         const int v = g.nbr[nidx(g, u) + j];
         const int side = u > v;
         const int a = min(u, v), b = max(u, v);
         const ull key = ((ull)side << 62) | rank;
         ull *bp = g.best + pidx(g, a, b);
         if (*(volatile ull *)bp < key) continue;   // an earlier set already separates
+        warp_unrank_lex(rank, d, l, g.binom, g.ldb, pos);
+        for (int i = lane; i < l; i += 32) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
+        __syncwarp();
         if (lane == 0) {
-            unrank_lex(rank, d, l, g.binom, g.ldb, pos);
-            for (int i = 0; i < l; ++i) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
             if (prop) sort_small(nd, l);        // the set is tested in ascending-id order
             nd[l] = u;
             nd[l + 1] = v;
@@ -697,7 +750,7 @@ __device__ __forceinline__ bool lane_decide(const TestParams &tp, float sqf, flo
     bad |= !(h11 > 1e-12f) || !(h22 > 1e-12f);
     ++acc.tests;
     bool queue_it = false, ind = false;
-    if (bad || pmin < (float)tp.guard) {
+    if (bad || pmin < tp.guard_f) {
         queue_it = true;
         ++acc.guard;
     } else {
@@ -1237,22 +1290,6 @@ __device__ __forceinline__ float rcp_fast(float x)
     return y;
 }
 
-// The last u < p with off[u] <= t (off: p + 1 ascending offsets, off[0] = 0 <= t < off[p]),
-// by the whole warp: 32 probes at a time instead of a chain of binary steps.
-__device__ __forceinline__ int warp_owner(const ull *off, int p, ull t)
-{
-    const int lane = threadIdx.x & 31;
-    int lo = 0, n = p;                                    // the answer lies in [lo, lo + n)
-    while (n > 1) {
-        const int step = (n + 31) / 32, i = lane * step;
-        const unsigned m = __ballot_sync(0xffffffffu, i < n && off[lo + min(i, n - 1)] <= t);
-        const int k = 31 - __clz(m);                      // lane 0 always holds
-        lo += k * step;
-        n = min(step, n - k * step);
-    }
-    return lo;
-}
-
 // Advance the lexicographic position (q0 < q1 < d) by k sets; positions past the
 // last set stop at q0 = d - 1.
 __device__ __forceinline__ void lex2_advance(int &q0, int &q1, int k, int d)
@@ -1711,15 +1748,16 @@ __global__ void __launch_bounds__(256) ci_redecide_kernel(GraphDev g, TestParams
         const ull t = queue[qi];
         int u, j, d;
         ull rank;
-        locate_test(g, g.tn_off, l, t, u, j, d, rank);
+        locate_test<true>(g, g.tn_off, l, t, u, j, d, rank);
         const int v = g.nbr[nidx(g, u) + j];
         const int side = u > v;
         const ull key = ((ull)side << 62) | rank;
         ull *bp = g.best + pidx(g, min(u, v), max(u, v));
         if (*(volatile ull *)bp < key) continue;
+        warp_unrank_lex(rank, d, l, g.binom, g.ldb, pos);
+        for (int i = lane; i < l; i += 32) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
+        __syncwarp();
         if (lane == 0) {
-            unrank_lex(rank, d, l, g.binom, g.ldb, pos);
-            for (int i = 0; i < l; ++i) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
             if (prop) sort_small(nd, l);
             nd[l] = u;
             nd[l + 1] = v;
@@ -1795,7 +1833,7 @@ __global__ void __launch_bounds__(256) c64_collect_kernel(GraphDev g, TestParams
         const ull t = queue[qi];
         int u, j, d;
         ull rank;
-        locate_test(g, g.tn_off, l, t, u, j, d, rank);
+        locate_test<true>(g, g.tn_off, l, t, u, j, d, rank);
         const int v = g.nbr[nidx(g, u) + j];
         const ull key = ((ull)(u > v) << 62) | rank;
         const long long ep = pidx(g, min(u, v), max(u, v));
@@ -1803,9 +1841,9 @@ __global__ void __launch_bounds__(256) c64_collect_kernel(GraphDev g, TestParams
         int first = 0;
         if (lane == 0) first = claim_byte(tp.pair_seen, ep);
         if (!__shfl_sync(0xffffffffu, first, 0) && nq > COLLECT_ALL) continue;   // not the pair's first queued test
+        warp_unrank_lex(rank, d, l, g.binom, g.ldb, pos);
+        for (int i = lane; i < l; i += 32) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
         if (lane == 0) {
-            unrank_lex(rank, d, l, g.binom, g.ldb, pos);
-            for (int i = 0; i < l; ++i) nd[i] = cand_node(g, prop, u, j, d, pos[i]);
             nd[l] = u;
             nd[l + 1] = v;
         }
@@ -1838,7 +1876,7 @@ __global__ void __launch_bounds__(256) c64_fill_kernel(GraphDev g, TestParams tp
         const long long na = n_of(tp, ab.x), nh = na >> 1;
         const double2 *xa2 = reinterpret_cast<const double2 *>(xa), *xb2 = reinterpret_cast<const double2 *>(xb);
         double acc0 = 0.0, acc1 = 0.0;
-#pragma unroll 4
+#pragma unroll 10
         for (long long t = threadIdx.x; t < nh; t += blockDim.x) {
             const double2 a2 = __ldg(xa2 + t), b2 = __ldg(xb2 + t);
             acc0 = fma(a2.x, b2.x, acc0);
@@ -2048,7 +2086,7 @@ __device__ __noinline__ void complement_body(const GraphDev &g, const TestParams
     for (ull t = (ull)threadIdx.x * ncta + cta; t < total; t += nthr) {
         int u, j, d;
         ull rank;
-        locate_test(g, noff, l, t, u, j, d, rank);
+        locate_test<false>(g, noff, l, t, u, j, d, rank);
         const ull T = g.binom[(long long)d * g.ldb + l];
         const int v = g.nbr[nidx(g, u) + j];
         const int k = d - l;
