@@ -61,8 +61,8 @@ CLASS_KERNELS = {
     "prec": "prec_update_kernel (neighbourhood precision blocks, FP64)",
     "stage_a": "stage_a sweep inverse (FP64)",
     "corr": "pc_corr: column statistics, standardisation, correlation GEMM",
-    "stage_loop": "stage_loop_kernel (one cooperative kernel over the complement-only stages: head, FP32-first "
-                  "complement tests, commit, degrees, tail, FP64 precision downdates, grid barriers between)",
+    "stage_loop": "node_loop_kernel (one cooperative kernel over the whole search of a small problem, a CTA per "
+                  "node: closed-form stage, FP32-first tests, commit, FP64 precision downdates)",
 }
 
 

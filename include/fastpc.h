@@ -85,7 +85,8 @@ void pc_destroy(pc_handle *h);
  *   "precision"   0 = FP64 everywhere; 1 = FP32 SIMT correlation GEMM + FP32 tests
  *                 with FP64 re-decision; 2 = split-precision BF16x3 tensor-core
  *                 correlation GEMM + FP32 tests with FP64 re-decision (default).
- *                 0, and 2 in the reversed order or with p <= 128, form all FP64
+ *                 0, and 2 in the reversed order, with p <= 128 or in a batched
+ *                 handle with instances of p <= 512, form all FP64
  *                 correlations by exact integer products on the tensor cores;
  *                 2 then rounds them to FP32 for the search
  *   "band"        FP64 re-decision band on |z - q| (default 1e-3)
@@ -252,13 +253,11 @@ pc_status pc_corr_block(pc_handle *h, int32_t i, const void *X, int32_t dtype, i
 /* pc_corr_blocks -- pc_corr_block for every instance of a batched handle in one
  * call: X[i], dtype[i], ld[i] (host arrays of k entries) as pc_corr_block's
  * arguments for instance i.  The instances' standardisation and correlation
- * GEMMs are independent (disjoint planes, disjoint diagonal blocks of corr),
+ * products are independent (disjoint planes, disjoint diagonal blocks of corr),
  * so they run concurrently on up to 8 internal streams of the handle, each with
  * its own staging and split-K workspaces, forked from and joined back into the
  * handle's stream: the call is ordered on that stream like one pc_corr_block
- * per instance, and gives the same results.  With "precision" 0 (FP64 Gram,
- * one shared workspace) the instances run one after the other on the handle's
- * stream.  Timing class "corr" covers the whole fork and join; "corr_gemm" is
+ * per instance, and gives the same results.  Timing class "corr" covers the whole fork and join; "corr_gemm" is
  * not recorded.  PC_ERR_STATE on a handle from pc_create, PC_ERR_ARG (nothing
  * issued) on a null array or a bad entry.  Not in the paper: it runs one
  * problem at a time. */

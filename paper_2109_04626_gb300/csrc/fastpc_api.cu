@@ -68,7 +68,7 @@ struct pc_handle {
     int comp_fp32 = 1;                // complement tests in FP32 first (FP32 modes)
     int stage_loop = 1;               // p <= NL_PMAX: the search in one kernel (node_loop.cu)
     int coop = -1;                    // device supports cooperative launches (-1: not asked yet)
-    int pair_warp = 1;                // stages 1-2: warp-per-pair kernel for the larger nodes
+    int pair_warp = 1;                // stages 1-2: pair groups for the larger nodes
     int pair_warp_dmin = fpc::PAIRWARP_DMIN;
     // path-restricted pools (option "path_pool"): component labels of the graph
     // without each node, the largest pool
