@@ -3002,11 +3002,12 @@ __device__ __forceinline__ bool lt_factor64(St &M, const Get &C, int l_rt, doubl
     return above_floor(h11) && above_floor(h22);
 }
 
-// sq |atanh r| to about 1e-9 of its value (it is returned as FP32).  atanh r = atanh c +
+// sq |atanh r| to about 2e-9 of its value (it is returned as FP32).  atanh r = atanh c +
 // atanh((r - c) / (1 - r c)) with c = tanh(0.34 k), k the nearest by FP32, leaves an
-// argument below 0.17, whose odd Taylor series to the 17th power runs in FP32 beyond its
-// first term (below 1 % of it): 9 FP64 instructions for every lane.  (The library function
-// takes about 60, and one lane of a warp with |r| > 0.17 is enough to pay them: the batch
+// argument below 0.171 for |r| up to 0.99999, whose odd Taylor series to the 17th power runs in FP32
+// beyond its first term (below 1 % of it): 9 FP64 instructions for every lane.  Nearer to 1 the
+// table has no entry: the library function, and infinity from 1 on.  (It
+// takes about 60, and one lane of a warp with |r| > 0.17 would be enough to pay them: the batch
 // of 1 M tests above ran at 271 us with it there, at 187 without.)
 constexpr int FISHER_K = 19;
 __constant__ double c_fisher[FISHER_K] = {0.0, 0.32747739480870536, 0.5915193954318165, 0.7698665359089004,
@@ -3018,8 +3019,9 @@ __constant__ double c_fisher[FISHER_K] = {0.0, 0.32747739480870536, 0.5915193954
 __device__ __forceinline__ double lt_fisher(double r, double sq)
 {
     const double a = fabs(r);
-    const int k = __float2int_rn(atanhf(fminf(round_f32(a), 0.99999f)) * (1.0f / 0.34f));
-    if (k >= FISHER_K) return a < 1.0 ? sq * atanh(a) : INFINITY;
+    const float af = round_f32(a);                       // a NaN: infinity
+    if (af > 0.99999f) return a < 1.0 ? sq * atanh(a) : INFINITY;
+    const int k = __float2int_rn(atanhf(af) * (1.0f / 0.34f));   // at most 18
     const double c = c_fisher[k];
     const double y = (a - c) * rcp_pivot(fma(-a, c, 1.0));
     const float g = round_f32(y), x = g * g;
