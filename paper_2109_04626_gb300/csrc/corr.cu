@@ -150,7 +150,7 @@ __device__ __forceinline__ void dev_split(float x, float mh, float ml, float &sd
 // distributed shared memory, in a fixed order, between the two passes (the second mostly
 // hits L2).  A lane owns a column.  FP32 input in double-single sums (col_sum_f32_kernel,
 // col_m2_f32_kernel below), FP64 input in FP64.  It also clears what the exact product adds
-// into: C above the diagonal, and its error flag.
+// into: C above the diagonal, and its error word.
 constexpr int CS_CLUSTER = 8, CS_WARPS = 8;
 
 template <typename T>
@@ -170,7 +170,7 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
     const T *x = X + (ok ? col : 0);
     for (int a = blockIdx.x * CS_CLUSTER + (int)cl.block_rank(); a < p; a += gridDim.x * CS_CLUSTER)
         for (int b = a + 1 + threadIdx.x; b < p; b += blockDim.x) C[(long long)a * ldc + b] = 0.0;
-    if (err && blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
+    if (blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
     // the warps' values -> the cluster's total, the same in every CTA
     auto total = [&](double v, int pass) -> double {
         red[w][tx] = v;

@@ -94,7 +94,8 @@ struct pc_handle {
     double *C64 = nullptr, *Pbuf = nullptr, *work = nullptr;
     float *C32 = nullptr, *tc_ws = nullptr;
     size_t tc_ws_bytes = 0;
-    int *tc_err = nullptr;
+    int *tc_err = nullptr;           // error words of the correlation product: one per instance of a batch
+    int nerr = 1;
     int *singular = nullptr;
     void *Xstage = nullptr;
     size_t Xstage_bytes = 0;
@@ -116,15 +117,16 @@ struct pc_handle {
     ull *binom = nullptr;
     double *rq_tab = nullptr;         // per stage l: tanh(q / sqrt(n - l - 3)), the |r| threshold
     long long opair_cap = 0;
-    // the search's scalars, counters and the GEMM's error flag lie together on the device,
-    // with one pinned mirror: one copy brings them all
+    // the search's scalars, counters and the correlation product's error words lie together
+    // on the device, with one pinned mirror: one copy brings them all
     struct HostView {
         LevelInfo info;
         DevCounters ctr;
-        int tc_err;
         int orient[2];               // pc_orient's rounds and error (pinned side only)
+        int tc_err[2];               // nerr words
     };
     HostView *view_d = nullptr, *view_h = nullptr;
+    size_t view_bytes() const { return offsetof(HostView, tc_err) + std::max(2, nerr) * sizeof(int); }
     LevelInfo *info_h = nullptr;     // into view_h
     DevCounters *ctr_h = nullptr;
     unsigned long long *nl_xch = nullptr;   // exchange words of the one-kernel search
@@ -332,15 +334,18 @@ static TestParams make_tp(const pc_handle *h)
 }
 
 // ---------------------------------------------------------------- create / destroy
-// pmax: largest problem size (binomial table), batch: block-diagonal batch
-// layout (no precision blocks, conventional order only)
 // bytes of the gradient (padded to 8), the loss (double) and the error flag (with padding)
 static size_t mlp_block_bytes() { return ((size_t)fpc::mlp_nparam() * sizeof(float) + 7) / 8 * 8 + 16; }
 
+// pmax: largest problem size (binomial table), blocks: instances of a block-diagonal batch
+// layout (no precision blocks, conventional order only); 0: one problem
+
 static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_level, int32_t pmax,
-                             long long pool_cap, bool batch, size_t packed, pc_handle **out)
+                             long long pool_cap, int blocks, size_t packed, pc_handle **out)
 {
+    const bool batch = blocks > 0;
     pc_handle *h = new pc_handle();
+    h->nerr = std::max(1, blocks);
     h->n = n;
     h->p = p;
     h->alpha = alpha;
@@ -387,11 +392,12 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
     A(dalloc(h, &g.prec_mem, (size_t)p * fpc::PREC_MAX * sizeof(int)));
     A(dalloc(h, &g.prec_pos, pp * sizeof(short)));
     A(dalloc(h, &g.prec_need, (size_t)p * sizeof(int)));
-    A(dalloc(h, &h->view_d, sizeof(pc_handle::HostView)));
+    A(dalloc(h, &h->view_d, h->view_bytes()));
+    A(cudaMemsetAsync(h->view_d, 0, e == cudaSuccess ? h->view_bytes() : 0, 0));   // before the copies below return
     if (e == cudaSuccess) {
         g.info = &h->view_d->info;
         g.ctr = &h->view_d->ctr;
-        h->tc_err = &h->view_d->tc_err;
+        h->tc_err = h->view_d->tc_err;
     }
     if (p <= fpc::NL_PMAX && !batch) A(dalloc(h, &h->nl_xch, fpc::node_loop_xch_bytes(p)));
     A(dalloc(h, &h->mean, (size_t)p * sizeof(double)));
@@ -413,7 +419,7 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
     }
     A(dalloc(h, &h->wpack, fpc::mlp_pack_bytes()));
     A(dalloc(h, &h->work, (size_t)(2 * p + 16) * sizeof(double)));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&h->view_h, sizeof(pc_handle::HostView));
+    if (e == cudaSuccess) e = cudaMallocHost((void **)&h->view_h, h->view_bytes());
     if (e == cudaSuccess) {
         h->info_h = &h->view_h->info;
         h->ctr_h = &h->view_h->ctr;
@@ -468,7 +474,7 @@ extern "C" pc_status pc_create(int64_t n, int32_t p, double alpha, int32_t max_l
     *out = nullptr;
     if (n < 4 || n > (1ll << 21) || p < 2 || p > fpc::MAXP || !(alpha > 0.0 && alpha < 1.0))
         return PC_ERR_ARG;
-    return create_impl(n, p, alpha, max_level, p, std::max<long long>(1 << 20, 16ll * p * p), false, 0, out);
+    return create_impl(n, p, alpha, max_level, p, std::max<long long>(1 << 20, 16ll * p * p), 0, 0, out);
 }
 
 // One handle over k independent problems laid out block-diagonally: instance i
@@ -496,7 +502,7 @@ extern "C" pc_status pc_create_batch(int32_t k, const int64_t *n, const int32_t 
     for (int i = 0; i < k; ++i) packed += (size_t)p[i] * p[i];
     pc_handle *h = nullptr;
     if (pc_status r = create_impl(nmax, (int32_t)ptot, alpha, max_level, pmax, std::max<long long>(1 << 20, pool),
-                                  true, packed, &h))
+                                  k, packed, &h))
         return r;
     h->nblk = k;
     h->order = 0;
@@ -797,15 +803,23 @@ static pc_status materialize_c64(pc_handle *h)
     return PC_OK;
 }
 
-// a bounded wait inside the tensor-core GEMM expired (device-side error word)
+// a bounded wait inside the tensor-core product of some instance expired: its device-side
+// error word, as the pinned mirror holds it.  A word is cleared only with its own instance's
+// data, so that giving another instance again hides nothing.
+static pc_status tc_status(pc_handle *h)
+{
+    if (!h->used_tc) return PC_OK;
+    for (int i = 0; i < h->nerr; ++i)
+        if (h->view_h->tc_err[i])
+            return fail(h, (pc_status)h->view_h->tc_err[i], "tensor-core correlation product: a bounded wait expired");
+    return PC_OK;
+}
 static pc_status check_tc(pc_handle *h)
 {
     if (!h->used_tc) return PC_OK;
-    int e = 0;
-    CK(cudaMemcpyAsync(&e, h->tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->view_h->tc_err, h->tc_err, h->nerr * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (e) return fail(h, (pc_status)e, "tensor-core correlation GEMM: a bounded wait expired");
-    return PC_OK;
+    return tc_status(h);
 }
 
 // The pair list of the FP64 entries formed in parallel before a small stage's FP64
@@ -885,7 +899,7 @@ static bool exact_corr(const pc_handle *h)
 // batched handle (its columns are rows [o, o+p) of the planes, its block of
 // corr the diagonal block there).
 // lane: run on a side stream with its own workspaces (pc_corr_blocks, which has
-// allocated the handle's planes and flags and cleared the GEMM's error flag first)
+// allocated the handle's planes and flags and cleared the error words first)
 static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t ld, int blk, CorrLane *lane = nullptr)
 {
     cudaStream_t s = lane ? lane->s : h->stream;
@@ -898,6 +912,7 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
     const int o = blk < 0 ? 0 : h->boff[blk];
     const int p = blk < 0 ? h->p : h->boff[blk + 1] - o;
     const long long n = blk < 0 ? h->n : h->bn[blk];
+    int *err = h->tc_err + std::max(0, blk);               // this instance's
     if (!X || (dtype != PC_F32 && dtype != PC_F64) || ld < p)
         return fail(h, PC_ERR_ARG, "pc_corr: bad X, dtype or ld");
     const size_t esz = dtype == PC_F64 ? 8 : 4;
@@ -940,13 +955,10 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
         double *C64b = blk < 0 ? h->C64 : h->C64 + h->pbase[blk];
         float *C32x = blk < 0 ? h->C32 : h->C32 + h->pbase[blk];
         const int ldx = blk < 0 ? h->ldc : p;
-        // a batch's instances share the error flag: cleared with the first of them
-        if (blk == 0 && !lane) CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
-        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, blk < 0 ? h->tc_err : nullptr,
-                                 s));
+        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, err, s));   // clears err
         {
             Timed tg(h, lane ? -1 : 7);
-            CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, C32x, ldx, h->tc_err, s));
+            CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, C32x, ldx, err, s));
         }
         h->used_tc = true;
         h->c32_rounded = true;
@@ -1028,10 +1040,10 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
             CK(dalloc(h, &tc_ws, need));
             tc_ws_bytes = need;
         }
-        if (blk <= 0 && !lane) CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
+        if (!lane) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
         Timed tg(h, lane ? -1 : 7);
         CK(fpc::launch_corr_bf16x3(h->Xhi + po, h->Xlo + po, n, h->ldk, p, C32b, ldb, tc_ws, tc_ws_bytes,
-                                   h->tc_err, s));
+                                   err, s));
         tc = true;
     }
     if (blk < 0) {
@@ -1086,7 +1098,7 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
     cudaStream_t s = h->stream;
     Timed tm(h, 0);
     // what the instances share, on the handle's stream before the fork: the
-    // standardised planes, the FP64-validity flags, the GEMM's error flag
+    // standardised planes, the FP64-validity flags, the error words
     if (!exact) {
         if (pc_status r = alloc_planes(h, s)) return r;
         if (!h->c64_valid) {
@@ -1095,7 +1107,7 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
             if (pc_status r = alloc_c64_list(h)) return r;
         }
     }
-    CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(h->tc_err, 0, h->nerr * sizeof(int), s));
     const int nl = std::min(k, 8);
     while ((int)h->lanes.size() < nl) {
         CorrLane cl;
@@ -1175,14 +1187,12 @@ extern "C" pc_status pc_corr_get(pc_handle *h, float *C32, double *C64)
 }
 
 // ---------------------------------------------------------------- skeleton
-// scalars, counters and the GEMM's error flag in one copy
+// scalars, counters and the product's error words in one copy
 static pc_status read_info(pc_handle *h)
 {
-    CK(cudaMemcpyAsync(h->view_h, h->view_d, sizeof(pc_handle::HostView), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->view_h, h->view_d, h->view_bytes(), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (h->used_tc && h->view_h->tc_err)
-        return fail(h, (pc_status)h->view_h->tc_err, "tensor-core correlation GEMM: a bounded wait expired");
-    return PC_OK;
+    return tc_status(h);
 }
 
 static int level_cap(const pc_handle *h)

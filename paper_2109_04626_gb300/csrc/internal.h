@@ -223,7 +223,7 @@ struct TestParams {
 void note_launch();
 
 // ---- correlation (corr.cu)
-// without a workspace; also clears C above the diagonal and err (nullptr: the caller has) for launch_gram_exact
+// without a workspace; also clears C above the diagonal and err for launch_gram_exact
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
                              double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s);
 cudaError_t launch_col_stats_split(const void *X, int dtype, long long n, int p, long long ld,

@@ -1,0 +1,98 @@
+"""Error words of the device on the library's host side (no GPU needed): fastpc_api.cu compiled for
+the CPU against a fake of the CUDA runtime and of the launchers (fake_cuda.cpp), whose device
+memory holds anything and whose products report expired waits on demand.  An error
+reaches the call that returns what it spoilt, whatever the order of the calls, and goes with
+the data that it belongs to."""
+import importlib.util
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+PKG = os.path.join(ROOT, "paper_2109_04626_gb300")
+TIMEOUT = 7
+
+
+@pytest.fixture(scope="module")
+def fp(tmp_path_factory):
+    cuda = "/usr/local/cuda/include"
+    if not shutil.which("g++") or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        pytest.skip("g++ or the CUDA headers are missing")
+    d = tmp_path_factory.mktemp("host")
+    flags = ["g++", "-std=c++17", "-O1", "-fPIC", "-I", cuda, "-I", os.path.join(PKG, "csrc"),
+             "-I", os.path.join(ROOT, "include")]
+    objs = []
+    for src in (os.path.join(PKG, "csrc", "fastpc_api.cu"), os.path.join(ROOT, "tests", "fake_cuda.cpp")):
+        objs.append(str(d / (os.path.basename(src) + ".o")))
+        subprocess.run(flags + ["-x", "c++", "-c", src, "-o", objs[-1]], check=True, timeout=300)
+    # what no test here reaches: a function that ends the process
+    names = [ln.split() for o in objs for ln in
+             subprocess.run(["nm", o], check=True, capture_output=True, text=True).stdout.splitlines()]
+    missing = {f[-1] for f in names if f[-2] == "U"} - {f[-1] for f in names if f[-2] != "U"}
+    stubs = sorted(m for m in missing if m.startswith(("_ZN3fpc", "cuda")))
+    (d / "stubs.c").write_text("#include <stdlib.h>\n" + "".join(f"void {m}(void) {{ abort(); }}\n" for m in stubs))
+    lib = str(d / "libhost.so")
+    subprocess.run(["gcc", "-fPIC", "-c", str(d / "stubs.c"), "-o", str(d / "stubs.o")], check=True, timeout=60)
+    subprocess.run(["g++", "-shared", "-o", lib] + objs + [str(d / "stubs.o")], check=True, timeout=60)
+    spec = importlib.util.spec_from_file_location("fastpc_host", os.path.join(PKG, "fastpc.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.LIB_PATH = lib
+    mod.fail = lambda exact=0, split=0: mod.load().fake_fail(exact, split)
+    yield mod
+    mod.fail()
+
+
+X = [np.zeros((40, p)) for p in (6, 9, 5)]
+LARGE = [np.zeros((40, p)) for p in (520, 530)]          # instances above the exact product's size in a batch
+
+
+def _batch(fp, Xs, **opts):
+    return fp.PCBatch([x.shape[0] for x in Xs], [x.shape[1] for x in Xs], 0.01, -1, **opts)
+
+
+@pytest.mark.parametrize("Xs", [X, LARGE])
+@pytest.mark.parametrize("precision", [0, 2])
+def test_instances_in_any_order(fp, Xs, precision):
+    """The words start clean: no instance has to come first."""
+    with _batch(fp, Xs, precision=precision) as pb:
+        for i in reversed(range(len(Xs))):
+            pb.corr_block(i, Xs[i])
+        C32, C64 = pb.corr_get()
+        assert np.isfinite(C64).all() and np.isfinite(C32).all()
+
+
+@pytest.mark.parametrize("Xs", [X, LARGE])
+@pytest.mark.parametrize("first", [0, 1])
+def test_error_of_one_instance(fp, Xs, first):
+    """An instance's expired wait is reported until that instance is given again, and by no other order."""
+    with _batch(fp, Xs) as pb:
+        order = [1, 0, 2][:len(Xs)]
+        fp.fail(1, 1)
+        for i in (order if first else order[::-1]):
+            pb.corr_block(i, Xs[i])
+        fp.fail()
+        bad = (order if first else order[::-1])[0]
+        for _ in range(2):
+            with pytest.raises(fp.PCError) as e:
+                pb.corr_get()
+            assert e.value.status == TIMEOUT
+            other = 0 if bad else 1
+            pb.corr_block(other, Xs[other])               # a good instance again changes nothing
+        pb.corr_block(bad, Xs[bad])
+        pb.corr_get()
+
+
+@pytest.mark.parametrize("Xs", [X, LARGE])
+def test_error_in_one_call_for_all(fp, Xs):
+    with _batch(fp, Xs) as pb:
+        fp.fail(2, 2)
+        pb.corr_blocks(Xs)
+        with pytest.raises(fp.PCError) as e:
+            pb.corr_get()
+        assert e.value.status == TIMEOUT
+        pb.corr_blocks(Xs)
+        pb.corr_get()
