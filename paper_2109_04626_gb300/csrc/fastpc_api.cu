@@ -2139,11 +2139,12 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     CK(cudaMemsetAsync(h->g.ctr, 0, sizeof(DevCounters), s));
     CK(fpc::launch_ci_list(ij, S, l, b, C32, h->C64, h->ldc, h->p, tp, r_out, indep_out, z_out,
                            h->g.ctr, h->g.blk_lo, h->g.blk_hi, s));
-    CK(cudaMemcpyAsync(h->ctr_h, h->g.ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(h->view_h, h->view_d, h->view_bytes(), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (h->ctr_h->status)
         return fail(h, (pc_status)h->ctr_h->status,
                     "pc_ci_batch: node id out of range, u == v, or nodes of different instances");
+    if (pc_status r = tc_status(h)) return r;            // r of a product that did not finish
     std::memset(&h->last, 0, sizeof(h->last));
     h->last.tests_executed = h->ctr_h->tests_executed;
     h->last.tests_redecided = h->ctr_h->redecided;
@@ -2199,7 +2200,7 @@ extern "C" pc_status pc_mlp_features(pc_handle *h, const int32_t *quads, int64_t
     CK(cudaMemcpyAsync(&e, h->mlp_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     if (e) return fail(h, PC_ERR_ARG, "pc_mlp_features: node id out of range or repeated in a quadruple");
-    return PC_OK;
+    return check_tc(h);                                  // features of a product that did not finish
 }
 
 // forward (and, with h1/h2, the activations a backward pass needs)

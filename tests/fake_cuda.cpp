@@ -148,6 +148,11 @@ cudaError_t launch_ci_list(const int *, const int *, int, long long, const float
     if (r) r[0] = tp.precision == 0 ? C64[1] : C32[1];
     return cudaSuccess;
 }
+cudaError_t launch_mlp_features(const int *, long long, const float *, int, const long long *, int, long long,
+                                const long long *, double, float *, int *, cudaStream_t)
+{
+    return cudaSuccess;
+}
 cudaError_t launch_expand_adj(GraphDev g, uint8_t *out, cudaStream_t)
 {
     memset(out, 1, (size_t)g.p * g.p);

@@ -96,3 +96,31 @@ def test_error_in_one_call_for_all(fp, Xs):
         assert e.value.status == TIMEOUT
         pb.corr_blocks(Xs)
         pb.corr_get()
+
+
+def _raw(fp, h, l):
+    """One raw test; its r."""
+    ij, S, r = np.zeros(2, np.int32), np.zeros(max(l, 1), np.int32), np.zeros(1)
+    fp._check(h, fp.load().pc_ci_batch(h, ij.ctypes.data, S.ctypes.data, l, 1, r.ctypes.data, None, None))
+    return r[0]
+
+
+def _features(fp, h, l):
+    q, f = np.zeros(4, np.int32), np.zeros(16, np.float32)
+    fp._check(h, fp.load().pc_mlp_features(h, q.ctypes.data, 1, f.ctypes.data))
+
+
+@pytest.mark.parametrize("call", [_raw, _features])
+@pytest.mark.parametrize("p, opts", [(20, {}), (20, dict(order=0)), (150, dict(order=0)), (150, {}), (20, dict(precision=0))])
+def test_values_of_a_failed_product_are_refused(fp, call, p, opts):
+    with fp.PC(40, p, 0.01, **opts) as pc:
+        fp.fail(1, 1)
+        pc.corr(np.zeros((40, p)))
+        fp.fail()
+        for l in (4, 0):
+            with pytest.raises(fp.PCError) as e:
+                call(fp, pc.h, l)
+            assert e.value.status == TIMEOUT
+        pc.corr(np.zeros((40, p)))
+        for l in (0, 4):
+            call(fp, pc.h, l)
