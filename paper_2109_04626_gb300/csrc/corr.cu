@@ -150,13 +150,14 @@ __device__ __forceinline__ void dev_split(float x, float mh, float ml, float &sd
 // distributed shared memory, in a fixed order, between the two passes (the second mostly
 // hits L2).  A lane owns a column.  FP32 input in double-single sums (col_sum_f32_kernel,
 // col_m2_f32_kernel below), FP64 input in FP64.  It also clears what the exact product adds
-// into: C above the diagonal, and its error word.
+// into: C above the diagonal, and its error word.  With nmrs also what launch_standardize
+// reads (the float splits of mean and 1/sd, and -mean/sd), and the word behind err cleared.
 constexpr int CS_CLUSTER = 8, CS_WARPS = 8;
 
 template <typename T>
 __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WARPS)
     col_stats_cluster_kernel(const T *__restrict__ X, long long n, int p, long long ld, double *mean, double *rsd,
-                             double *C, long long ldc, int *err)
+                             double *C, long long ldc, int *err, float4 *split, double *nmrs)
 {
     __shared__ double red[CS_WARPS][33];
     __shared__ float redm[CS_WARPS][33];
@@ -170,7 +171,10 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
     const T *x = X + (ok ? col : 0);
     for (int a = blockIdx.x * CS_CLUSTER + (int)cl.block_rank(); a < p; a += gridDim.x * CS_CLUSTER)
         for (int b = a + 1 + threadIdx.x; b < p; b += blockDim.x) C[(long long)a * ldc + b] = 0.0;
-    if (blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) *err = 0;
+    if (blockIdx.x == 0 && cl.block_rank() == 0 && threadIdx.x == 0) {
+        err[0] = 0;
+        if (nmrs) err[1] = 0;
+    }
     // the warps' values -> the cluster's total, the same in every CTA
     auto total = [&](double v, int pass) -> double {
         red[w][tx] = v;
@@ -281,8 +285,14 @@ __global__ void __cluster_dims__(1, CS_CLUSTER, 1) __launch_bounds__(32 * CS_WAR
     }
     if (cl.block_rank() == 0 && w == 0 && ok) {
         const double var = m2 / (double)n, us = (double)sc;
-        mean[col] = mu / us;
-        rsd[col] = var > 0.0 ? us / sqrt(var) : 0.0;     // constant column -> zero column
+        const double m = mu / us, rs = var > 0.0 ? us / sqrt(var) : 0.0;   // constant column -> zero column
+        mean[col] = m;
+        rsd[col] = rs;
+        if (nmrs) {                                      // as col_sum_f32_kernel and col_m2_f32_kernel leave them
+            const float mh = (float)m, rh = (float)rs;
+            split[col] = make_float4(mh, (float)(m - (double)mh), rh, (float)(rs - (double)rh));
+            nmrs[col] = -(m * rs);
+        }
     }
     cl.sync();                                           // no CTA leaves while another reads its sums
 }
@@ -821,15 +831,18 @@ cudaError_t launch_cast_block(const double *C64, float *C32, int ldc, int o, int
 }
 
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
-                             double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s)
+                             double *mean, double *rsd, double *C, long long ldc, int *err, double *ws, cudaStream_t s)
 {
     const dim3 g((p + 31) / 32, CS_CLUSTER);
+    const StatsLayout L = stats_layout_f32(n, p);
+    float4 *split = ws ? (float4 *)((char *)ws + L.split_off) : nullptr;
+    double *nmrs = ws ? (double *)((char *)ws + L.nmrs_off) : nullptr;
     if (dtype == 1)
         col_stats_cluster_kernel<double><<<g, 32 * CS_WARPS, 0, s>>>((const double *)X, n, p, ld, mean, rsd, C,
-                                                                        ldc, err);
+                                                                        ldc, err, split, nmrs);
     else
         col_stats_cluster_kernel<float><<<g, 32 * CS_WARPS, 0, s>>>((const float *)X, n, p, ld, mean, rsd, C,
-                                                                       ldc, err);
+                                                                       ldc, err, split, nmrs);
     note_launch();
     return cudaGetLastError();
 }

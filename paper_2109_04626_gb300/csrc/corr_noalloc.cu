@@ -73,7 +73,7 @@ extern "C" pc_status pc_corr_noalloc(const void *X, int32_t dtype, int64_t n, in
     cudaStream_t s = (cudaStream_t)stream;
     // column statistics into the file-scope scratch (every call overwrites
     // entries 0..p-1 of both halves; nothing accumulates across calls)
-    if (launch_col_stats(X, dtype, n, p, ld, stats, stats + NOALLOC_MAXP, C_out, ldc, err, s) != cudaSuccess)
+    if (launch_col_stats(X, dtype, n, p, ld, stats, stats + NOALLOC_MAXP, C_out, ldc, err, nullptr, s) != cudaSuccess)
         return PC_ERR_CUDA;
     // FP64 correlations by exact integer products on the tensor cores, accumulated in C_out
     // itself (gram_exact.cu): no workspace

@@ -94,24 +94,22 @@ struct pc_handle {
     double *C64 = nullptr, *Pbuf = nullptr, *work = nullptr;
     float *C32 = nullptr, *tc_ws = nullptr;
     size_t tc_ws_bytes = 0;
-    int *tc_err = nullptr;           // error words of the correlation product: one per instance of a batch
-    int nerr = 1;
+    // error words of the correlation product: one per instance of a batch; one problem: of
+    // the matrix the search uses, and of the split-precision product beside it
+    int *tc_err = nullptr;
+    int nerr = 2;
     int *singular = nullptr;
     void *Xstage = nullptr;
     size_t Xstage_bytes = 0;
     bool have_corr = false;
     bool used_tc = false;
     bool c32_rounded = false;        // C32 is the FP32 rounding of full FP64 correlations
-    // pc_ci_batch returns r from the split-precision product: beside a rounded C32 it is
-    // formed on demand, from a copy of X
-    void *Xkeep = nullptr;
-    size_t Xkeep_bytes = 0;
-    const void *keep_x = nullptr;    // Xkeep, or the staging buffer of a host X
-    int keep_dtype = 0;
-    long long keep_ld = 0;
-    unsigned char *c32tc_ws = nullptr;
-    float *C32tc = nullptr;          // into c32tc_ws
-    bool c32tc_valid = false;
+    // pc_ci_batch returns r from the split-precision product, formed beside a rounded C32
+    unsigned char *split_ws = nullptr;
+    float *C32s = nullptr;           // into split_ws
+    // its column statistics are there, the caller's data have been read, the product is there
+    cudaEvent_t split_stats = nullptr, split_read = nullptr, split_done = nullptr;
+    bool split_pending = false;      // the handle's stream has not waited for split_done
     // graph state
     GraphDev g{};
     ull *binom = nullptr;
@@ -126,7 +124,7 @@ struct pc_handle {
         int tc_err[2];               // nerr words
     };
     HostView *view_d = nullptr, *view_h = nullptr;
-    size_t view_bytes() const { return offsetof(HostView, tc_err) + std::max(2, nerr) * sizeof(int); }
+    size_t view_bytes() const { return offsetof(HostView, tc_err) + nerr * sizeof(int); }
     LevelInfo *info_h = nullptr;     // into view_h
     DevCounters *ctr_h = nullptr;
     unsigned long long *nl_xch = nullptr;   // exchange words of the one-kernel search
@@ -144,7 +142,7 @@ struct pc_handle {
     // captured stage loop (CUDA graph with a conditional WHILE node)
     int use_graph = 1;
     cudaStream_t cap_stream = nullptr;
-    cudaStream_t br_stream = nullptr;      // captures the bodies of conditional nodes
+    cudaStream_t br_stream = nullptr;      // captures the bodies of conditional nodes; runs the split product
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     cudaGraphConditionalHandle hcond = 0;
@@ -345,7 +343,7 @@ static pc_status create_impl(int64_t n, int32_t p, double alpha, int32_t max_lev
 {
     const bool batch = blocks > 0;
     pc_handle *h = new pc_handle();
-    h->nerr = std::max(1, blocks);
+    h->nerr = std::max(2, blocks);
     h->n = n;
     h->p = p;
     h->alpha = alpha;
@@ -573,6 +571,7 @@ extern "C" void pc_destroy(pc_handle *h)
     if (!h) return;
     for (auto &cl : h->lanes)
         if (cl.s) cudaStreamSynchronize(cl.s);
+    if (h->split_ws) cudaStreamSynchronize(h->br_stream);
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
     if (h->view_h) cudaFreeHost(h->view_h);
@@ -590,6 +589,8 @@ extern "C" void pc_destroy(pc_handle *h)
     for (auto &cl : h->lanes)
         if (cl.s) cudaStreamDestroy(cl.s);
     for (auto e : h->lane_ev) cudaEventDestroy(e);
+    for (auto e : {h->split_stats, h->split_read, h->split_done})
+        if (e) cudaEventDestroy(e);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->br_stream) cudaStreamDestroy(h->br_stream);
     delete h;
@@ -806,10 +807,11 @@ static pc_status materialize_c64(pc_handle *h)
 // a bounded wait inside the tensor-core product of some instance expired: its device-side
 // error word, as the pinned mirror holds it.  A word is cleared only with its own instance's
 // data, so that giving another instance again hides nothing.
-static pc_status tc_status(pc_handle *h)
+// split: of the split-precision product beside a rounded C32 as well.
+static pc_status tc_status(pc_handle *h, bool split = false)
 {
     if (!h->used_tc) return PC_OK;
-    for (int i = 0; i < h->nerr; ++i)
+    for (int i = 0; i < (h->nblk ? h->nblk : 1 + split); ++i)
         if (h->view_h->tc_err[i])
             return fail(h, (pc_status)h->view_h->tc_err[i], "tensor-core correlation product: a bounded wait expired");
     return PC_OK;
@@ -851,30 +853,74 @@ static pc_status alloc_planes(pc_handle *h, cudaStream_t s)
     return PC_OK;
 }
 
-// The split-precision product beside a rounded C32, once per pc_corr, for the raw tests.
-// Its planes, workspaces and matrix are one allocation, made at the first such call.
-static pc_status ensure_c32tc(pc_handle *h)
+// The split-precision product beside a rounded C32, for the raw tests' r: from the exact
+// product's column statistics on a side stream, beside that product (both leave most of the
+// SMs idle at the sizes where a search takes less than a millisecond).  pc_corr joins the last
+// read of the caller's data; the product itself, which outlasts the exact one by 10-40 us at
+// p = 20-100 (joined there, p = 55, n = 5000: the search 179 -> 197 us, so 177), is joined where it
+// is read or written again (split_join), and under a capture at once.  Its planes, statistics, workspace and
+// matrix are one allocation, made at the first pc_corr.
+struct SplitBuffers {
+    size_t plane, c32, sws, tws;
+    uint16_t *hi, *lo;
+    float *C32;
+    double *stats;                   // what launch_standardize reads beside mean and rsd
+    float *ws;
+};
+static pc_status split_join(pc_handle *h)
 {
-    if (h->c32tc_valid) return PC_OK;
-    cudaStream_t s = h->stream;
-    const int p = h->p;
-    const size_t plane = (size_t)p * h->ldk * sizeof(uint16_t);
-    const size_t c32 = ((size_t)p * h->ldc * sizeof(float) + 255) / 256 * 256;
-    const size_t sws = (fpc::col_stats_ws_bytes(h->n, p) + 255) / 256 * 256;
-    const size_t tws = fpc::corr_bf16x3_ws_bytes(h->n, p);
-    if (!h->c32tc_ws) {
-        CK(dalloc(h, &h->c32tc_ws, 2 * plane + c32 + sws + tws));
-        CK(cudaMemsetAsync(h->c32tc_ws, 0, 2 * plane, s));    // the padding samples stay zero
-        h->C32tc = (float *)(h->c32tc_ws + 2 * plane);
+    if (!h->split_pending) return PC_OK;
+    cudaStreamCaptureStatus cap;
+    CK(cudaStreamIsCapturing(h->stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+        CK(cudaStreamWaitEvent(h->stream, h->split_done, 0));
+    } else {                                             // a product before the capture: no part of it
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaEventSynchronize(h->split_done);
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        CK(e);
     }
-    uint16_t *hi = (uint16_t *)h->c32tc_ws, *lo = (uint16_t *)(h->c32tc_ws + plane);
-    double *st = (double *)(h->c32tc_ws + 2 * plane + c32);
-    float *ws = (float *)(h->c32tc_ws + 2 * plane + c32 + sws);
-    CK(fpc::launch_col_stats_split(h->keep_x, h->keep_dtype, h->n, p, h->keep_ld, h->mean, h->rsd, st, s));
-    CK(fpc::launch_standardize(h->keep_x, h->keep_dtype, h->n, p, h->keep_ld, h->mean, h->rsd, st, nullptr, nullptr,
-                               hi, lo, h->ldk, s));
-    CK(fpc::launch_corr_bf16x3(hi, lo, h->n, h->ldk, p, h->C32tc, h->ldc, ws, tws, h->tc_err, s));
-    h->c32tc_valid = true;
+    h->split_pending = false;
+    return PC_OK;
+}
+static pc_status split_buffers(pc_handle *h, SplitBuffers &b)
+{
+    if (pc_status r = split_join(h)) return r;           // of the data before
+    auto pad = [](size_t x) { return (x + 255) / 256 * 256; };
+    b.plane = (size_t)h->p * h->ldk * sizeof(uint16_t);
+    b.c32 = pad((size_t)h->p * h->ldc * sizeof(float));
+    b.sws = pad(fpc::col_stats_ws_bytes(h->n, h->p));
+    b.tws = fpc::corr_bf16x3_ws_bytes(h->n, h->p);
+    for (auto e : {&h->split_stats, &h->split_read, &h->split_done})
+        if (!*e) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    if (!h->split_ws) {
+        CK(dalloc(h, &h->split_ws, 2 * b.plane + b.c32 + b.sws + b.tws));
+        CK(cudaMemsetAsync(h->split_ws, 0, 2 * b.plane, h->stream));   // the padding samples stay zero
+        h->C32s = (float *)(h->split_ws + 2 * b.plane);
+    }
+    b.hi = (uint16_t *)h->split_ws;
+    b.lo = (uint16_t *)(h->split_ws + b.plane);
+    b.C32 = h->C32s;
+    b.stats = (double *)(h->split_ws + 2 * b.plane + b.c32);
+    b.ws = (float *)(h->split_ws + 2 * b.plane + b.c32 + b.sws);
+    return PC_OK;
+}
+// after the statistics (event split_stats on the handle's stream)
+static pc_status split_product(pc_handle *h, const SplitBuffers &b, const void *X, int dtype, long long ld)
+{
+    cudaStream_t side = h->br_stream;
+    CK(cudaStreamWaitEvent(side, h->split_stats, 0));
+    CK(fpc::launch_standardize(X, dtype, h->n, h->p, ld, h->mean, h->rsd, b.stats, nullptr, nullptr, b.hi, b.lo, h->ldk,
+                               side));
+    CK(cudaEventRecord(h->split_read, side));
+    CK(cudaStreamWaitEvent(h->stream, h->split_read, 0));
+    CK(fpc::launch_corr_bf16x3(b.hi, b.lo, h->n, h->ldk, h->p, b.C32, h->ldc, b.ws, b.tws, h->tc_err + 1, side));
+    CK(cudaEventRecord(h->split_done, side));
+    cudaStreamCaptureStatus cap;
+    CK(cudaStreamIsCapturing(h->stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone) h->split_pending = true;
+    else CK(cudaStreamWaitEvent(h->stream, h->split_done, 0));
     return PC_OK;
 }
 
@@ -931,35 +977,21 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
     }
     if (exact_corr(h)) {
         Timed tm(h, lane ? -1 : 0);
-        if (h->precision == 2 && blk < 0) {
-            h->keep_dtype = dtype;
-            h->keep_x = Xd;
-            h->keep_ld = ld;
-            if (Xd == X) {
-                const size_t bytes = (size_t)n * p * esz;
-                if (bytes > h->Xkeep_bytes) {
-                    dfree(h, h->Xkeep);
-                    h->Xkeep = nullptr;
-                    h->Xkeep_bytes = 0;
-                    CK(dalloc(h, &h->Xkeep, bytes));
-                    h->Xkeep_bytes = bytes;
-                }
-                h->keep_x = h->Xkeep;
-                h->keep_ld = p;
-                if (ld == p) CK(cudaMemcpyAsync(h->Xkeep, X, bytes, cudaMemcpyDeviceToDevice, s));
-                else CK(cudaMemcpy2DAsync(h->Xkeep, (size_t)p * esz, X, (size_t)ld * esz, (size_t)p * esz, n,
-                                          cudaMemcpyDeviceToDevice, s));
-            }
-        }
-        h->c32tc_valid = false;
+        const bool split = h->precision == 2 && blk < 0;
+        SplitBuffers sb{};
+        if (split)
+            if (pc_status r = split_buffers(h, sb)) return r;
         double *C64b = blk < 0 ? h->C64 : h->C64 + h->pbase[blk];
         float *C32x = blk < 0 ? h->C32 : h->C32 + h->pbase[blk];
         const int ldx = blk < 0 ? h->ldc : p;
-        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, err, s));   // clears err
+        CK(fpc::launch_col_stats(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, err, sb.stats, s));   // clears err
+        if (split) CK(cudaEventRecord(h->split_stats, s));
         {
             Timed tg(h, lane ? -1 : 7);
             CK(fpc::launch_gram_exact(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, C64b, ldx, C32x, ldx, err, s));
         }
+        if (split)
+            if (pc_status r = split_product(h, sb, Xd, dtype, ld)) return r;
         h->used_tc = true;
         h->c32_rounded = true;
         h->have_corr = true;
@@ -2125,15 +2157,17 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     cudaStream_t s = h->stream;
     // r itself is returned: from the split-precision product, as at every size
     const float *C32 = h->C32;
+    bool split = false;
     TestParams tp = make_tp(h);
     tp.dr_max = 5e-6f;
     if (h->c32_rounded && h->precision == 2) {
         tp.eps_c = 1.0e-6f;
         if (h->nblk) {
-            tp.precision = 0;                            // a batch keeps no X for that product: all in FP64
+            tp.precision = 0;                            // a batch has no such product: all in FP64
         } else if (fpc::ci_list_uses_fp32(l, tp)) {
-            if (pc_status r = ensure_c32tc(h)) return r;
-            C32 = h->C32tc;
+            split = true;
+            C32 = h->C32s;
+            if (pc_status r = split_join(h)) return r;
         }
     }
     CK(cudaMemsetAsync(h->g.ctr, 0, sizeof(DevCounters), s));
@@ -2144,7 +2178,7 @@ extern "C" pc_status pc_ci_batch(pc_handle *h, const int32_t *ij, const int32_t 
     if (h->ctr_h->status)
         return fail(h, (pc_status)h->ctr_h->status,
                     "pc_ci_batch: node id out of range, u == v, or nodes of different instances");
-    if (pc_status r = tc_status(h)) return r;            // r of a product that did not finish
+    if (pc_status r = tc_status(h, split)) return r;     // r of a product that did not finish
     std::memset(&h->last, 0, sizeof(h->last));
     h->last.tests_executed = h->ctr_h->tests_executed;
     h->last.tests_redecided = h->ctr_h->redecided;

@@ -223,9 +223,10 @@ struct TestParams {
 void note_launch();
 
 // ---- correlation (corr.cu)
-// without a workspace; also clears C above the diagonal and err for launch_gram_exact
+// without a workspace; also clears C above the diagonal and err for launch_gram_exact;
+// ws (col_stats_ws_bytes; nullptr: not wanted) receives what launch_standardize reads, then err[1] is cleared too
 cudaError_t launch_col_stats(const void *X, int dtype, long long n, int p, long long ld,
-                             double *mean, double *rsd, double *C, long long ldc, int *err, cudaStream_t s);
+                             double *mean, double *rsd, double *C, long long ldc, int *err, double *ws, cudaStream_t s);
 cudaError_t launch_col_stats_split(const void *X, int dtype, long long n, int p, long long ld,
                                    double *mean, double *rsd, double *ws, cudaStream_t s);
 size_t col_stats_ws_bytes(long long n, int p);

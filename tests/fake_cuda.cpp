@@ -13,9 +13,11 @@ static std::map<char *, size_t> g_mem;
 static char g_dummy[64];
 // calls of a product until its wait expires (0: none does)
 static int g_fail_exact, g_fail_split;
+static int g_split;                                      // split-precision products run
 
 extern "C" {
 void fake_fail(int exact, int split) { g_fail_exact = exact, g_fail_split = split; }
+int fake_split() { return g_split; }
 void fake_device(void *p, long long bytes) { g_mem[(char *)p] = (size_t)bytes; }
 int pc_corr_noalloc(void *, int, long long, int, long long, void *, long long, void *) { return 1; }
 
@@ -61,6 +63,10 @@ cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return mem
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)g_dummy, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *c)
+{
+    return *c = cudaStreamCaptureStatusNone, cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = (cudaEvent_t)g_dummy, cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)g_dummy, cudaSuccess; }
@@ -85,9 +91,10 @@ bool tc_gemm_available() { return true; }
 bool ci_list_uses_fp32(int l, const TestParams &tp) { return tp.precision != 0 && l <= 2; }
 
 cudaError_t launch_col_stats(const void *, int, long long, int, long long, double *, double *, double *, long long,
-                             int *err, cudaStream_t)
+                             int *err, double *ws, cudaStream_t)
 {
-    if (err) *err = 0;
+    err[0] = 0;
+    if (ws) err[1] = 0;
     return cudaSuccess;
 }
 cudaError_t launch_gram_exact(const void *, int, long long, int p, long long, const double *, const double *, double *C,
@@ -114,6 +121,7 @@ cudaError_t launch_standardize(const void *, int, long long, int, long long, con
 cudaError_t launch_corr_bf16x3(const uint16_t *, const uint16_t *, long long, long long, int p, float *C32, int ldc,
                                float *, size_t, int *err, cudaStream_t)
 {
+    ++g_split;
     if (g_fail_split && --g_fail_split == 0) *err = 7;
     for (int a = 0; a < p; ++a)
         for (int b = 0; b < p; ++b) C32[(size_t)a * ldc + b] = a == b ? 1.f : 0.5f;

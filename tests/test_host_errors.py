@@ -124,3 +124,29 @@ def test_values_of_a_failed_product_are_refused(fp, call, p, opts):
         pc.corr(np.zeros((40, p)))
         for l in (0, 4):
             call(fp, pc.h, l)
+
+
+def test_raw_tests_need_no_work_put_off(fp):
+    """Everything a raw test reads is formed by pc_corr: the caller's data are not needed later."""
+    with fp.PC(40, 20, 0.01) as pc:
+        for _ in range(2):
+            before = fp.load().fake_split()
+            pc.corr(np.zeros((40, 20)))
+            assert fp.load().fake_split() == before + 1
+            assert _raw(fp, pc.h, 0) == 0.5 and _raw(fp, pc.h, 0) == 0.5
+            assert fp.load().fake_split() == before + 1
+
+
+def test_error_of_the_split_product_alone(fp):
+    """It spoils the raw tests that read it, not the search, and goes with the next data."""
+    with fp.PC(40, 20, 0.01) as pc:
+        fp.fail(0, 1)
+        pc.corr(np.zeros((40, 20)))
+        fp.fail()
+        with pytest.raises(fp.PCError) as e:
+            _raw(fp, pc.h, 0)
+        assert e.value.status == TIMEOUT
+        pc.corr_get()
+        pc.skeleton()
+        pc.corr(np.zeros((40, 20)))
+        _raw(fp, pc.h, 0)
