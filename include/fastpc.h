@@ -187,8 +187,8 @@ pc_status pc_corr_get(pc_handle *h, float *C32, double *C64);
  * sqrt(n-l-3)|atanh r_uv.S| <= Phi^{-1}(1-alpha/2) (Eq. 1, Sec. 2.2.2), r from
  * the Schur complement of Sec. 4.  Writes the skeleton into adj_out (p x p,
  * 0/1, symmetric, host or device; may be NULL) and the counters into stats
- * (host; may be NULL).  Sepsets stay in the handle (pc_sepsets_*).
- * Requires a prior pc_corr.  Synchronises. */
+ * (host; may be NULL); a call that returns an error writes neither.  Sepsets
+ * stay in the handle (pc_sepsets_*).  Requires a prior pc_corr.  Synchronises. */
 pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats);
 
 /* pc_skeleton_many -- the skeleton searches of `count` independent problems

@@ -1457,6 +1457,17 @@ static pc_status ensure_graph(pc_handle *h)
     return PC_OK;
 }
 
+// The skeleton into the caller's device matrix, behind the search and before the host has seen
+// its result: written only if the device finds what the host will take for success, so that a
+// failed call leaves the matrix as it was.
+static pc_status expand_early(pc_handle *h)
+{
+    if (!h->adj_early) return PC_OK;
+    Timed t(h, 5);
+    CK(fpc::launch_expand_adj(h->g, h->adj_early, h->g.info, h->tc_err, h->used_tc ? (h->nblk ? h->nblk : 1) : 0, h->stream));
+    return PC_OK;
+}
+
 static pc_status clear_halt(pc_handle *h)
 {
     // need_host and halt are adjacent ints after 'done'
@@ -1522,11 +1533,9 @@ static pc_status skeleton_enqueue(pc_handle *h)
         if (e != cudaErrorCooperativeLaunchTooLarge) {
             CK(e);
             CK(cudaEventRecord(h->ev1, s));
-            if (h->adj_early) {
-                Timed t(h, 5);
-                CK(fpc::launch_expand_adj(g, h->adj_early, s));
-            }
             h->loop_ran = true;
+            if (!h->learned)
+                if (pc_status r = expand_early(h)) return r;
             return PC_OK;
         }
         cudaGetLastError();                            // not resident: the loop below runs it all
@@ -1646,21 +1655,17 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
             more = true;
         }
     }
-    if (!h->loop_ran || more) {
-        CK(cudaEventRecord(h->ev1, s));
-        if (h->adj_early) {
-            Timed t(h, 5);
-            CK(fpc::launch_expand_adj(g, h->adj_early, s));
-        }
-    }
+    if (!h->loop_ran || more) CK(cudaEventRecord(h->ev1, s));
     if (h->learned && h->learned_lmax >= 1) {
         // largest stage run: the first one in the reversed order, the last one conventionally
         Timed tm(h, h->timing ? 6 : -1);
         const int lmax = h->order == 1 ? h->info_h->first_level : h->info_h->l - 1;
         CK(fpc::launch_reverify(g, tp, h->C32, h->C64, h->ldc, lmax, s));
     }
-    if (!h->loop_ran || more || h->learned)
+    if (!h->loop_ran || more || h->learned) {
+        if (pc_status r = expand_early(h)) return r;
         if (pc_status r = read_info(h)) return r;
+    }
     if (!h->info_h->done) return fail(h, PC_ERR_INTERNAL, "stage loop did not finish");
     const DevCounters &c = *h->ctr_h;
     const LevelInfo &I = *h->info_h;
@@ -1989,7 +1994,7 @@ static pc_status copy_adj(pc_handle *h, uint8_t *adj_out)
     cudaStream_t s = h->stream;
     Timed t(h, 5);
     if (is_device_ptr(adj_out)) {
-        CK(fpc::launch_expand_adj(h->g, adj_out, s));
+        CK(fpc::launch_expand_adj(h->g, adj_out, nullptr, nullptr, 0, s));
     } else {
         if (h->adj_stage_bytes < bytes) {
             dfree(h, h->adj_stage);
@@ -1997,7 +2002,7 @@ static pc_status copy_adj(pc_handle *h, uint8_t *adj_out)
             CK(dalloc(h, &h->adj_stage, bytes));
             h->adj_stage_bytes = bytes;
         }
-        CK(fpc::launch_expand_adj(h->g, h->adj_stage, s));
+        CK(fpc::launch_expand_adj(h->g, h->adj_stage, nullptr, nullptr, 0, s));
         CK(cudaMemcpyAsync(adj_out, h->adj_stage, bytes, cudaMemcpyDeviceToHost, s));
     }
     CK(cudaStreamSynchronize(s));

@@ -3428,10 +3428,19 @@ cudaError_t launch_pp_commit(GraphDev g, cudaStream_t s)
 // division (p * p <= MAXP_BATCH^2 < 2^32), one 16-bit field of the row, one 16-byte store.
 // Bound by the stores: 15000 nodes (a batch, 225 MB) 43 us, 372 us with a 64-bit division per
 // entry.
-__global__ void __launch_bounds__(256) expand_adj_kernel(const uint32_t *adj, int p, int W, uint8_t *out)
+// gate (or nullptr): written only behind a search that succeeded, as the host will find it --
+// the search's scalars and counters, and the correlation product's error words.
+__global__ void __launch_bounds__(256) expand_adj_kernel(const uint32_t *adj, int p, int W, uint8_t *out,
+                                                         const LevelInfo *gate, const DevCounters *ctr, const int *err,
+                                                         int nerr)
 {
     const uint32_t total = (uint32_t)p * (uint32_t)p, step = gridDim.x * blockDim.x * 16u;
     const bool wide = ((uintptr_t)out & 15) == 0;
+    if (gate) {
+        bool bad = !gate->done || gate->error || gate->pool_overflow || ctr->status;
+        for (int i = threadIdx.x; i < nerr; i += blockDim.x) bad |= err[i] != 0;
+        if (__syncthreads_or(bad)) return;
+    }
     for (unsigned long long q0 = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) * 16; q0 < total; q0 += step) {
         const uint32_t q = (uint32_t)q0;
         uint32_t u = q / (uint32_t)p, v = q - u * (uint32_t)p;
@@ -3465,9 +3474,12 @@ __global__ void __launch_bounds__(256) expand_adj_kernel(const uint32_t *adj, in
 }
 static_assert((unsigned long long)MAXP_BATCH * MAXP_BATCH <= 0xffffffffull, "expand_adj_kernel counts entries in 32 bits");
 
-cudaError_t launch_expand_adj(GraphDev g, uint8_t *out, cudaStream_t s)
+cudaError_t launch_expand_adj(GraphDev g, uint8_t *out, const LevelInfo *gate, const int *err, int nerr, cudaStream_t s)
 {
-    expand_adj_kernel<<<num_sms() * 8, 256, 0, s>>>(g.adj, g.p, g.W, out);
+    // a CTA writes 4096 entries per turn
+    const long long need = ((long long)g.p * g.p + 4095) / 4096;
+    expand_adj_kernel<<<(unsigned)std::min<long long>(num_sms() * 8, need), 256, 0, s>>>(g.adj, g.p, g.W, out, gate, g.ctr,
+                                                                                        err, nerr);
     note_launch();
     return cudaGetLastError();
 }

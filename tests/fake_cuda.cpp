@@ -161,9 +161,11 @@ cudaError_t launch_mlp_features(const int *, long long, const float *, int, cons
 {
     return cudaSuccess;
 }
-cudaError_t launch_expand_adj(GraphDev g, uint8_t *out, cudaStream_t)
+cudaError_t launch_expand_adj(GraphDev g, uint8_t *out, const LevelInfo *gate, const int *err, int nerr, cudaStream_t)
 {
-    memset(out, 1, (size_t)g.p * g.p);
+    bool bad = gate && (!gate->done || gate->error || gate->pool_overflow || g.ctr->status);
+    for (int i = 0; gate && i < nerr; ++i) bad |= err[i] != 0;
+    if (!bad) memset(out, 1, (size_t)g.p * g.p);
     return cudaSuccess;
 }
 

@@ -3,6 +3,7 @@ the CPU against a fake of the CUDA runtime and of the launchers (fake_cuda.cpp),
 memory holds anything and whose products report expired waits on demand.  An error
 reaches the call that returns what it spoilt, whatever the order of the calls, and goes with
 the data that it belongs to."""
+import ctypes
 import importlib.util
 import os
 import shutil
@@ -150,3 +151,19 @@ def test_error_of_the_split_product_alone(fp):
         pc.skeleton()
         pc.corr(np.zeros((40, 20)))
         _raw(fp, pc.h, 0)
+
+
+def test_device_skeleton_of_a_failed_product(fp):
+    """The skeleton of an unfinished matrix does not reach a device output."""
+    out = np.full((20, 20), 9, np.uint8)
+    fp.load().fake_device(ctypes.c_void_p(out.ctypes.data), ctypes.c_longlong(out.size))
+    with fp.PC(40, 20, 0.01) as pc:
+        fp.fail(1, 0)
+        pc.corr(np.zeros((40, 20)))
+        with pytest.raises(fp.PCError) as e:
+            pc.skeleton(out)
+        assert e.value.status == TIMEOUT
+        assert (out == 9).all()
+        pc.corr(np.zeros((40, 20)))
+        pc.skeleton(out)
+        assert (out == 1).all()
