@@ -291,7 +291,10 @@ pc_status pc_sepsets_get(pc_handle *h, int32_t *pairs, int32_t *level, int32_t *
  * batched handle: the block-diagonal p x p matrix of all instances).
  * rounds_out (host, may be NULL): rule rounds that oriented an edge.
  * PC_ERR_STATE before pc_skeleton, PC_ERR_ARG for a NULL codes_out.  Runs on
- * the handle's stream as one cooperative kernel; synchronises once. */
+ * the handle's stream as one cooperative kernel, synchronising once; a graph whose
+ * work between two of its barriers could outlast their bound of 2 s (the largest
+ * degree above about 1000), and a device without cooperative launches, take a
+ * launch per phase and a synchronisation per round of the rules. */
 pc_status pc_orient(pc_handle *h, int8_t *codes_out, int32_t *rounds_out);
 
 /* pc_ci_batch -- b raw CI tests on the current correlation matrix (the index

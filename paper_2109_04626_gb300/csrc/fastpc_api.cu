@@ -136,6 +136,7 @@ struct pc_handle {
     int8_t *or_codes = nullptr;
     bool have_skel = false;
     long long skel_edges = 0;        // of that skeleton
+    int skel_dmax = 0;               // at least its largest degree
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     pc_stats last{};
     std::vector<void *> allocs;
@@ -1687,6 +1688,7 @@ static pc_status skeleton_complete(pc_handle *h, pc_stats *st, bool *overflow)
     st->complement_tests = c.complement_tests;
     st->edges_removed = c.edges_removed;
     st->edges_kept = I.edges / 2;
+    h->skel_dmax = I.lstar + 1;
     unsigned int bits = c.max_dz_bits;
     float mdz;
     std::memcpy(&mdz, &bits, sizeof(mdz));
@@ -1937,6 +1939,7 @@ static pc_status skeleton_pathpool_once(pc_handle *h, pc_stats *st, bool *overfl
     st->tests_redecided = 0;
     st->edges_removed = c.edges_removed;
     st->edges_kept = (uint64_t)p * (p - 1) / 2 - c.edges_removed;
+    h->skel_dmax = p - 1;
     st->levels_run = levels;
     st->first_level = first;
     st->stage_a_ran = stage_a_ran;
@@ -2137,7 +2140,8 @@ extern "C" pc_status pc_orient(pc_handle *h, int8_t *codes_out, int32_t *rounds_
     }
     // each round that changes something adds a mark; there are at most 32 W p marks
     int *ctl = nullptr, *res = h->view_h->orient;
-    CK(fpc::launch_orient(h->g, h->skel_edges, h->or_ws, (long long)words * 32, dst, &ctl, s));
+    const int dmax = (int)std::min<long long>(h->skel_dmax, h->skel_edges);
+    CK(fpc::launch_orient(h->g, h->skel_edges, dmax, h->or_ws, (long long)words * 32, dst, &ctl, s));
     CK(cudaMemcpyAsync(res, ctl + 3, sizeof(h->view_h->orient), cudaMemcpyDeviceToHost, s));
     if (dst != codes_out) CK(cudaMemcpyAsync(codes_out, dst, pp, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

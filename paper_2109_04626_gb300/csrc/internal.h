@@ -293,7 +293,7 @@ int lane_range_of(int l);
 cudaError_t launch_prec_update(GraphDev g, TestParams tp, const double *C64, int ldc, cudaStream_t s);
 // ---- orientation, Algorithm 1 Phase II, in one cooperative kernel (orient.cu)
 size_t orient_ws_bytes(const GraphDev &g);
-cudaError_t launch_orient(GraphDev g, long long edges, void *ws, long long max_rounds, int8_t *out, int **ctl,
+cudaError_t launch_orient(GraphDev g, long long edges, int dmax, void *ws, long long max_rounds, int8_t *out, int **ctl,
                           cudaStream_t s);
 // degrees of the frozen graph, then (last CTA) the stage tail of mode 0 in the same kernel
 cudaError_t launch_degrees_tail(GraphDev g, TestParams tp, int cap, cudaGraphConditionalHandle hc, int use_cond,

@@ -188,6 +188,90 @@ __device__ __forceinline__ uint32_t codes4(uint32_t A, uint32_t H, uint32_t T)
     return c4;
 }
 
+// The phases, over the nodes of the whole grid (a warp or a CTA each).
+constexpr int OR_DEG_WARP = 64;          // nodes of larger degree: their triples by the whole CTA
+struct Marks {
+    uint32_t *ah, *at, *add;
+};
+__device__ __forceinline__ int grid_warp() { return (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); }
+__device__ __forceinline__ int grid_warps() { return (int)((gridDim.x * blockDim.x) >> 5); }
+
+__device__ __forceinline__ void phase_triples_warp(const GraphDev &g, const Marks &m)
+{
+    for (int k = grid_warp(); k < g.p; k += grid_warps()) {
+        int lo, hi, w0, w1;
+        inst_words(g, k, lo, hi, w0, w1);
+        int *nb = g.nbr + nidx(g, k);
+        const int dg = warp_neighbours(g, k, w0, w1, nb);
+        if ((threadIdx.x & 31) == 0) g.deg[k] = dg;
+        if (dg <= OR_DEG_WARP) colliders_of(g, m.ah, m.at, k, nb, dg, threadIdx.x & 31, 32);
+    }
+}
+__device__ __forceinline__ void phase_triples_cta(const GraphDev &g, const Marks &m)
+{
+    for (int k = blockIdx.x; k < g.p; k += gridDim.x) {
+        const int dg = __ldcg(g.deg + k);
+        if (dg > OR_DEG_WARP) colliders_of(g, m.ah, m.at, k, g.nbr + nidx(g, k), dg, threadIdx.x, blockDim.x);
+    }
+}
+// the orientations that the marks imply, into each node's row of add; did this thread find one?
+__device__ __forceinline__ bool phase_find(const GraphDev &g, const Marks &m)
+{
+    const int lane = threadIdx.x & 31, W = g.W;
+    const GlobalRows A{g.adj, W}, H{m.ah, W}, T{m.at, W};
+    bool any = false;
+    for (int a = grid_warp(); a < g.p; a += grid_warps()) {
+        int lo, hi, w0, w1;
+        inst_words(g, a, lo, hi, w0, w1);
+        const long long row = (long long)a * W;
+        for (int w = w0 + lane; w <= w1; w += 32) m.add[row + w] = 0u;
+        __syncwarp();
+        const int dg = __ldcg(g.deg + a);
+        const int *nb = g.nbr + nidx(g, a);
+        for (int x = lane; x < dg; x += 32) {
+            const int b = nb[x], w = b >> 5;
+            const uint32_t bit = 1u << (b & 31);
+            if ((m.ah[row + w] | m.at[row + w]) & bit) continue;
+            if (!rule_orients(A, H, T, a, b, w0, w1)) continue;
+            atomicOr(m.add + row + w, bit);
+            any = true;
+        }
+    }
+    return any;
+}
+__device__ __forceinline__ void phase_apply(const GraphDev &g, const Marks &m)
+{
+    const int lane = threadIdx.x & 31, W = g.W;
+    for (int a = grid_warp(); a < g.p; a += grid_warps()) {
+        int lo, hi, w0, w1;
+        inst_words(g, a, lo, hi, w0, w1);
+        const long long row = (long long)a * W;
+        for (int w = w0 + lane; w <= w1; w += 32) m.ah[row + w] |= __ldcg(m.add + row + w);
+        const int dg = __ldcg(g.deg + a);
+        const int *nb = g.nbr + nidx(g, a);
+        for (int x = lane; x < dg; x += 32) {
+            const int b = nb[x];
+            if ((__ldcg(m.add + (long long)b * W + (a >> 5)) >> (a & 31)) & 1u)
+                atomicOr(m.at + row + (b >> 5), 1u << (b & 31));
+        }
+    }
+}
+__device__ __forceinline__ void phase_codes(const GraphDev &g, const Marks &m, int8_t *out, int vec)
+{
+    const int p = g.p;
+    for (int a = grid_warp(); a < p; a += grid_warps()) {
+        const long long row = (long long)a * g.W;
+        int8_t *o = out + (long long)a * p;
+        for (int b0 = (threadIdx.x & 31) * 4; b0 < p; b0 += 128) {
+            const int w = b0 >> 5, sh = b0 & 31;
+            const uint32_t c4 = codes4(g.adj[row + w] >> sh, m.ah[row + w] >> sh, m.at[row + w] >> sh);
+            if (vec) *(uint32_t *)(o + b0) = c4;
+            else
+                for (int q = 0; q < 4 && b0 + q < p; ++q) o[b0 + q] = (int8_t)(c4 >> (8 * q));
+        }
+    }
+}
+
 // Phase II in one cooperative launch: colliders, the rounds of R1-R4, the codes.  A round
 // is two phases with a barrier after each: every node's warp finds the orientations
 // a -> b of its undirected edges (a lane each) from the marks as they stand, into its own
@@ -198,83 +282,46 @@ __device__ __forceinline__ uint32_t codes4(uint32_t A, uint32_t H, uint32_t T)
 // p = 500, 2 rounds 156 -> 63 (a round was two copies, a fill, a launch and a host round
 // trip, about 35 us, and an edge a whole warp's turn).
 // ctl: [0] barrier count, [1], [2] changed flags of even and odd rounds, [3] rounds, [4] error.
-constexpr int OR_DEG_WARP = 64;          // nodes of larger degree: their triples by the whole CTA
-__global__ void __launch_bounds__(256) orient_kernel(GraphDev g, uint32_t *ah, uint32_t *at, uint32_t *add, int *ctl,
-                                                     long long max_rounds, int8_t *out, int vec)
+__global__ void __launch_bounds__(256) orient_kernel(GraphDev g, Marks m, int *ctl, long long max_rounds, int8_t *out,
+                                                     int vec)
 {
-    const int lane = threadIdx.x & 31, W = g.W, p = g.p;
-    const int nwg = (int)((gridDim.x * blockDim.x) >> 5), gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const GlobalRows A{g.adj, W}, H{ah, W}, T{at, W};
     unsigned target = 0;
-    bool ok = true;
-    // colliders
-    for (int k = gw; k < p; k += nwg) {
-        int lo, hi, w0, w1;
-        inst_words(g, k, lo, hi, w0, w1);
-        int *nb = g.nbr + nidx(g, k);
-        const int dg = warp_neighbours(g, k, w0, w1, nb);
-        if (lane == 0) g.deg[k] = dg;
-        if (dg <= OR_DEG_WARP) colliders_of(g, ah, at, k, nb, dg, lane, 32);
-    }
-    ok = grid_wait((unsigned *)ctl, target);
-    for (int k = blockIdx.x; ok && k < p; k += gridDim.x) {
-        const int dg = __ldcg(g.deg + k);
-        if (dg > OR_DEG_WARP) colliders_of(g, ah, at, k, g.nbr + nidx(g, k), dg, threadIdx.x, blockDim.x);
-    }
+    phase_triples_warp(g, m);
+    bool ok = grid_wait((unsigned *)ctl, target);
+    if (ok) phase_triples_cta(g, m);
     ok = ok && grid_wait((unsigned *)ctl, target);
     int rounds = 0;
     for (long long r = 0; ok && r <= max_rounds; ++r) {
-        bool any = false;
-        for (int a = gw; a < p; a += nwg) {
-            int lo, hi, w0, w1;
-            inst_words(g, a, lo, hi, w0, w1);
-            const long long row = (long long)a * W;
-            for (int w = w0 + lane; w <= w1; w += 32) add[row + w] = 0u;
-            __syncwarp();
-            const int dg = __ldcg(g.deg + a);
-            const int *nb = g.nbr + nidx(g, a);
-            for (int x = lane; x < dg; x += 32) {
-                const int b = nb[x], w = b >> 5;
-                const uint32_t bit = 1u << (b & 31);
-                if ((ah[row + w] | at[row + w]) & bit) continue;
-                if (!rule_orients(A, H, T, a, b, w0, w1)) continue;
-                atomicOr(add + row + w, bit);
-                any = true;
-            }
-        }
-        if (any) *(volatile int *)(ctl + 1 + (r & 1)) = 1;
+        if (phase_find(g, m)) *(volatile int *)(ctl + 1 + (r & 1)) = 1;
         if (!(ok = grid_wait((unsigned *)ctl, target))) break;
         if (!*(volatile int *)(ctl + 1 + (r & 1))) break;      // the same in every CTA
         ++rounds;
         if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile int *)(ctl + 1 + ((r + 1) & 1)) = 0;
-        for (int a = gw; a < p; a += nwg) {
-            int lo, hi, w0, w1;
-            inst_words(g, a, lo, hi, w0, w1);
-            const long long row = (long long)a * W;
-            for (int w = w0 + lane; w <= w1; w += 32) ah[row + w] |= __ldcg(add + row + w);
-            const int dg = __ldcg(g.deg + a);
-            const int *nb = g.nbr + nidx(g, a);
-            for (int x = lane; x < dg; x += 32) {
-                const int b = nb[x];
-                if ((__ldcg(add + (long long)b * W + (a >> 5)) >> (a & 31)) & 1u)
-                    atomicOr(at + row + (b >> 5), 1u << (b & 31));
-            }
-        }
+        phase_apply(g, m);
         ok = grid_wait((unsigned *)ctl, target);
     }
-    for (int a = gw; a < p; a += nwg) {
-        const long long row = (long long)a * W;
-        int8_t *o = out + (long long)a * p;
-        for (int b0 = lane * 4; b0 < p; b0 += 128) {
-            const int w = b0 >> 5, sh = b0 & 31;
-            const uint32_t c4 = codes4(g.adj[row + w] >> sh, ah[row + w] >> sh, at[row + w] >> sh);
-            if (vec) *(uint32_t *)(o + b0) = c4;
-            else
-                for (int q = 0; q < 4 && b0 + q < p; ++q) o[b0 + q] = (int8_t)(c4 >> (8 * q));
-        }
-    }
+    phase_codes(g, m, out, vec);
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl[3] = rounds;
     if (!ok && threadIdx.x == 0) ctl[4] = 7;             // PC_ERR_TIMEOUT
+}
+
+// One phase a launch, for graphs whose work between two barriers could outlast the barriers'
+// bound, or where the cooperative launch is not to be had.
+enum { PH_TRIPLES_WARP, PH_TRIPLES_CTA, PH_FIND, PH_APPLY, PH_CODES };
+__global__ void __launch_bounds__(256) orient_phase_kernel(GraphDev g, Marks m, int *ctl, int phase, int rounds,
+                                                           int8_t *out, int vec)
+{
+    switch (phase) {
+    case PH_TRIPLES_WARP: phase_triples_warp(g, m); break;
+    case PH_TRIPLES_CTA: phase_triples_cta(g, m); break;
+    case PH_FIND:
+        if (phase_find(g, m)) ctl[1] = 1;
+        break;
+    case PH_APPLY: phase_apply(g, m); break;
+    default:
+        phase_codes(g, m, out, vec);
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl[3] = rounds;
+    }
 }
 
 // The same for p <= OR_ONE_P in one CTA: the three bitsets in shared memory, the rounds'
@@ -382,46 +429,72 @@ __global__ void __launch_bounds__(OR_ONE_THREADS) orient_one_kernel(GraphDev g, 
 }
 static_assert(OR_ONE_P * (OR_ONE_P - 1) <= 32 * OR_ONE_THREADS, "a thread's pairs fit the word of found orientations");
 
-int sm_count()
+// Word steps (each up to 8 loads) of a lane between two barriers: its nodes' edges in turns of
+// 32, at most `dmax` candidates of W words for each (rule_orients).
+long long lane_steps(int p, int dmax, int W, int warps)
 {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
+    return (long long)((p + warps - 1) / warps) * ((dmax + 31) / 32) * (dmax + 2) * W;
 }
+// 2^20 of them at 700 clocks (L2) are 0.4 s of the barriers' 2; the triples of such nodes are
+// fewer.  A sparse graph has some thousands; 1000 nodes of degree 999 are at the limit.
+constexpr long long OR_STEPS_MAX = 1ll << 20;
 
 }  // namespace
 
 size_t orient_ws_bytes(const GraphDev &g) { return (3 * (size_t)g.p * g.W) * sizeof(uint32_t) + 8 * sizeof(int); }
 
-// edges: of the skeleton; ws: orient_ws_bytes; ctl receives where the rounds ([3]) and the error ([4]) are
-cudaError_t launch_orient(GraphDev g, long long edges, void *ws, long long max_rounds, int8_t *out, int **ctl,
+// edges, dmax: of the skeleton (dmax: at least its largest degree); ws: orient_ws_bytes; ctl receives where
+// the rounds ([3]) and the error ([4]) are
+cudaError_t launch_orient(GraphDev g, long long edges, int dmax, void *ws, long long max_rounds, int8_t *out, int **ctl,
                           cudaStream_t s)
 {
     const size_t words = (size_t)g.p * g.W;
-    uint32_t *ah = (uint32_t *)ws, *at = ah + words, *add = at + words;
-    int *c = (int *)(add + words);
+    Marks m{(uint32_t *)ws, (uint32_t *)ws + words, (uint32_t *)ws + 2 * words};
+    int *c = (int *)(m.add + words);
     *ctl = c;
     const bool one = g.p <= OR_ONE_P && !g.prow && edges <= 8ll * g.p;
-    cudaError_t e = one ? cudaMemsetAsync(c, 0, 8 * sizeof(int), s) : cudaMemsetAsync(ah, 0, orient_ws_bytes(g), s);
+    cudaError_t e = one ? cudaMemsetAsync(c, 0, 8 * sizeof(int), s) : cudaMemsetAsync(ws, 0, orient_ws_bytes(g), s);
     if (e != cudaSuccess) return e;
-    const int vec = g.p % 4 == 0 && ((uintptr_t)out & 3) == 0;
+    int vec = g.p % 4 == 0 && ((uintptr_t)out & 3) == 0;
     if (one) {
         orient_one_kernel<<<1, OR_ONE_THREADS, 0, s>>>(g, c, (int)max_rounds, out); note_launch();
         return cudaGetLastError();
     }
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, orient_kernel, 256, 0);
+    int dev = 0, sms = 0, coop = 0, per_sm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, orient_kernel, 256, 0);
     if (e != cudaSuccess) return e;
-    const int blocks = std::max(1, std::min((g.p + 7) / 8, sm_count() * std::max(1, per_sm)));
-    void *args[] = {&g, &ah, &at, &add, &c, &max_rounds, &out, (void *)&vec};
-    e = cudaLaunchCooperativeKernel((const void *)orient_kernel, dim3(blocks), dim3(256), args, 0, s);
-    note_launch();
-    return e;
+    const int blocks = std::max(1, std::min((g.p + 7) / 8, sms * std::max(1, per_sm)));
+    const int wi = std::min(g.W, (g.ldb + 61) / 32);     // words of the largest instance (ldb - 1 nodes, any first bit)
+    if (coop && lane_steps(g.p, dmax, wi, blocks * 8) <= OR_STEPS_MAX) {
+        void *args[] = {&g, &m, &c, &max_rounds, &out, &vec};
+        e = cudaLaunchCooperativeKernel((const void *)orient_kernel, dim3(blocks), dim3(256), args, 0, s);
+        if (e != cudaErrorCooperativeLaunchTooLarge) {
+            note_launch();
+            return e;
+        }
+        cudaGetLastError();                              // not resident: phase by phase
+    }
+    auto phase = [&](int k, int rounds) -> cudaError_t {
+        orient_phase_kernel<<<(g.p + 7) / 8, 256, 0, s>>>(g, m, c, k, rounds, out, vec); note_launch();
+        return cudaGetLastError();
+    };
+    e = phase(PH_TRIPLES_WARP, 0);
+    if (e == cudaSuccess) e = phase(PH_TRIPLES_CTA, 0);
+    int rounds = 0;
+    for (long long r = 0; e == cudaSuccess && r <= max_rounds; ++r) {
+        int changed = 0;
+        e = cudaMemsetAsync(c + 1, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = phase(PH_FIND, 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&changed, c + 1, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess || !changed) break;
+        ++rounds;
+        e = phase(PH_APPLY, 0);
+    }
+    return e == cudaSuccess ? phase(PH_CODES, rounds) : e;
 }
 
 }  // namespace fpc
