@@ -153,7 +153,8 @@ void pc_destroy(pc_handle *h);
  *                 direct tests of more than 12 conditioning members, a stage
  *                 the proposal may score, more FP64 re-decisions than its queue
  *                 holds, or a stage above the budget (default; skipped on a
- *                 device without cooperative launches).  0 = the captured loop
+ *                 device without cooperative launches, and above 2^17 samples
+ *                 with FP64 entries formed on demand).  0 = the captured loop
  *                 throughout.  The results are the same either way.
  *   "comp_fp32"   1 = complement tests (reversed order) in FP32 first from the
  *                 FP64 precision blocks, decided there when a first-order

@@ -1514,7 +1514,7 @@ static pc_status skeleton_enqueue(pc_handle *h)
     // problems of p <= NL_PMAX: the whole search in one kernel, a CTA per node; the captured
     // loop (or the host loop) goes on from the first stage it does not take
     h->loop_ran = false;
-    bool loop = h->stage_loop && p <= fpc::NL_PMAX && !h->nblk;
+    bool loop = h->stage_loop && p <= fpc::NL_PMAX && !h->nblk && (h->c64_full || n <= fpc::NL_LAZY_NMAX);
     if (loop && h->coop < 0) {
         int dev = 0, v = 0;
         CK(cudaGetDevice(&dev));

@@ -119,6 +119,10 @@ __host__ __device__ inline int stage_branch(int kind, int comp, int score, int h
 constexpr int STAGE_FIXED_KERNELS = 3;
 // the search of a small problem in one cooperative kernel, a CTA per node (node_loop.cu)
 constexpr int NL_PMAX = 128;            // largest p it takes
+// Most samples with FP64 correlations formed on demand: a warp forms an entry in about 6 clocks a
+// sample (a chain of loads), up to about 1000 entries between two of the kernel's waits (p^2/2 over
+// 8 warps): 0.8e9 of their 4e9 clocks at 2^17 samples; at 2^21, the most a handle takes, 13e9.
+constexpr long long NL_LAZY_NMAX = 1ll << 17;
 
 // Everything the stage kernels need, by value.
 struct GraphDev {
