@@ -522,7 +522,8 @@ def run_ours(args):
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": DRAM_BYTES_PER_LAUNCH.get((w["name"], dom)),
                 "kernel": dom, "kernels": CLASS_KERNELS.get(dom, dom),
-                "work": "algorithmic flops F(l) = l^3/3 + 2l^2 + 6l + 10 per executed test (direct), "
+                "work": "algorithmic flops F(l) = l^3/3 + 2l^2 + 6l + 10 per executed test (direct; 8 or 15 for "
+                        "a test of l = 1 or 2 that the pair groups' bound decides), "
                         "k^3/3 + 2k^2 + 6k + 20 (complement)" if dom in ("ci_direct", "ci_complement") else
                         ("precision-block flops (|R|^3/3 + 2|T||R|(|R|+|T|) per downdate, m^3 per build) + "
                          "complement-test flops of the step" if dom == "stage_loop" else

@@ -1462,16 +1462,14 @@ template <int L>
 __device__ __forceinline__ void pair_group_put(const GraphDev &g, const TestParams &tp, const float *C32, const double *C64, int ldc,
                                                int u, int j0, int dg, uint2 *list, int &nlist, bool put, bool ind,
                                                unsigned key, int vi, unsigned *sep_s, float sqf, float rq,
-                                               ull *queue, ull qcap, ull *qlen, LaneAcc &acc)
+                                               ull *queue, ull qcap, ull *qlen, LaneAcc &acc, unsigned &fast)
 {
     const int lane = threadIdx.x & 31;
     const unsigned bi = __ballot_sync(0xffffffffu, ind);
     if (bi) {
         const int at = __ffs(bi) - 1;
-        if (put && lane >= at) {
-            ++acc.tests;                                  // decided here, or not needed
-            put = false;
-        }
+        fast += ind;                                      // decided here
+        if (lane >= at) put = false;                      // ... or not needed
         if (lane == at) {
             const int v = g.nbr[nidx(g, u) + j0 + vi];
             int pos[L];
@@ -1493,18 +1491,23 @@ __device__ __forceinline__ void pair_group_put(const GraphDev &g, const TestPara
     }
 }
 
-__device__ __forceinline__ void pair_group_flush(const LaneAcc &acc, ull fast, ull fl, DevCounters *ctr)
+// FP32 operations of a test that the bound decides, its own part of them (h22, h12 and the comparison)
+__host__ __device__ constexpr ull pair_flops(int l) { return l == 1 ? 8 : 15; }
+
+__device__ __forceinline__ void pair_group_flush(const LaneAcc &acc, ull fast, int l, DevCounters *ctr)
 {
-    ull tests = (ull)acc.tests + fast, band = acc.band, guard = acc.guard, red = acc.red, degen = acc.degen;
+    ull tests = acc.tests, band = acc.band, guard = acc.guard, red = acc.red, degen = acc.degen;
     for (int off = 16; off > 0; off >>= 1) {
         tests += __shfl_xor_sync(0xffffffffu, tests, off);
         band += __shfl_xor_sync(0xffffffffu, band, off);
         guard += __shfl_xor_sync(0xffffffffu, guard, off);
         red += __shfl_xor_sync(0xffffffffu, red, off);
         degen += __shfl_xor_sync(0xffffffffu, degen, off);
+        fast += __shfl_xor_sync(0xffffffffu, fast, off);
     }
     if ((threadIdx.x & 31) == 0) {
-        WarpAcc wa = {tests, red, band, guard, degen, (tests - red) * fl, red * fl, 0.f};
+        const ull fl = flops_direct(l);
+        WarpAcc wa = {tests + fast, red, band, guard, degen, (tests - red) * fl + fast * pair_flops(l), red * fl, 0.f};
         flush_acc(wa, ctr);
     }
 }
@@ -1584,7 +1587,7 @@ __device__ __forceinline__ void pairgroup_stage1(const GraphDev &g, const TestPa
                 if (__any_sync(0xffffffffu, put))
                     pair_group_put<1>(g, tp, C32, C64, ldc, u, j0, dg, list, nlist, put,
                                       put && pb.independent(h22, h12), (unsigned)i, vi, sep_s, sqf, rq, queue,
-                                      qcap, qlen, acc);
+                                      qcap, qlen, acc, fast_tests);
             }
             if (nlist >= 16) {                            // (the rest after the last round)
                 pair_group_listed<1>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
@@ -1594,7 +1597,7 @@ __device__ __forceinline__ void pairgroup_stage1(const GraphDev &g, const TestPa
         }
         if (nlist) pair_group_listed<1>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
     }
-    pair_group_flush(acc, fast_tests, flops_direct(1), g.ctr);
+    pair_group_flush(acc, fast_tests, 1, g.ctr);
 }
 
 // Stage 2: a CTA per group of up to PG_PAIRS pairs, their rows corr[v, adj(u)] in shared
@@ -1691,7 +1694,7 @@ __device__ __forceinline__ void pairgroup_stage2(const GraphDev &g, const TestPa
                     if (__any_sync(0xffffffffu, put))
                         pair_group_put<2>(g, tp, C32, C64, ldc, u, j0, dg, list, nlist, put,
                                           put && pb.independent(h22, h12), key, vi, sep_s, sqf, rq, queue, qcap,
-                                          qlen, acc);
+                                          qlen, acc, fast_tests);
                 }
                 if (nlist >= 16 || (nlist && (rd & 7) == 7)) {
                     pair_group_listed<2>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
@@ -1703,7 +1706,7 @@ __device__ __forceinline__ void pairgroup_stage2(const GraphDev &g, const TestPa
         }
         if (nlist) pair_group_listed<2>(g, tp, C32, C64, ldc, u, j0, list, nlist, sep_s, sqf, rq, queue, qcap, qlen, acc);
     }
-    pair_group_flush(acc, fast_tests, flops_direct(2), g.ctr);
+    pair_group_flush(acc, fast_tests, 2, g.ctr);
 }
 
 template <bool PROP>

@@ -240,6 +240,7 @@ __device__ __noinline__ void nl_direct_stage(NlShared &S, const TestParams &tp, 
     const int dg = S.deg[u], d = dg - 1;
     const uint32_t total = S.T[u] * (uint32_t)dg;
     const float sqf = sqrtf((float)(tp.n - L - 3)), rq = tanhf(tp.qf / sqf);
+    unsigned run = 0;
     for (uint32_t t = threadIdx.x; t < total; t += NL_THREADS) {
         const uint32_t rank = t / (uint32_t)dg;
         const int j = (int)(t - rank * (uint32_t)dg);
@@ -248,7 +249,7 @@ __device__ __noinline__ void nl_direct_stage(NlShared &S, const TestParams &tp, 
         nl_unrank<L>(S, rank, d, s);
 #pragma unroll
         for (int i = 0; i < L; ++i) s[i] = S.nbr[s[i] + (s[i] >= j)];
-        ++acc.tests;
+        ++run;
         const int r = nl_direct<L>(C, ld, u, S.nbr[j], s, tp, sqf, rq);
         if (r == 1) {
             nl_found(S, j, rank);
@@ -259,7 +260,8 @@ __device__ __noinline__ void nl_direct_stage(NlShared &S, const TestParams &tp, 
             if (q < NL_QCAP) S.queue[q] = t;
         }
     }
-    acc.fl32 += (ull)((total + NL_THREADS - 1 - threadIdx.x) / NL_THREADS) * flops_direct(L);
+    acc.tests += run;
+    acc.fl32 += (ull)run * flops_direct(L);
 }
 
 // FP64 evaluation of the tests of the queue (all: of every test of the stage), a warp each.
@@ -471,6 +473,7 @@ __device__ __noinline__ void nl_comp_stage(NlShared &S, const TestParams &tp, co
     const uint32_t T = S.T[u], total = T * (uint32_t)dg;
     const double rq = tp.rq_tab[l];
     const float sqf = sqrtf((float)(tp.n - l - 3)), rqf = (float)rq;
+    unsigned run = 0;
     for (uint32_t t = threadIdx.x; t < total; t += NL_THREADS) {
         const uint32_t rank = t / (uint32_t)dg;
         const int j = (int)(t - rank * (uint32_t)dg);
@@ -480,7 +483,7 @@ __device__ __noinline__ void nl_comp_stage(NlShared &S, const TestParams &tp, co
 #pragma unroll
         for (int i = 0; i < K; ++i) sr[i] = S.nslot[sr[i] + (sr[i] >= j)];
         const int sv = S.nslot[j];
-        ++acc.comp;
+        ++run;
         bool ind = false;
         if (f32) {
             const int r = nl_comp_fp32<K>(Pf, sr, su, sv, tp, sqf, rqf, ind);
@@ -495,8 +498,8 @@ __device__ __noinline__ void nl_comp_stage(NlShared &S, const TestParams &tp, co
         }
         if (ind) nl_found(S, j, rank);
     }
-    acc.flc += (ull)((total + NL_THREADS - 1 - threadIdx.x) / NL_THREADS) *
-               ((ull)(K * K * K) / 3 + 2ull * K * K + 6ull * K + 20);
+    acc.comp += run;
+    acc.flc += (ull)run * ((ull)(K * K * K) / 3 + 2ull * K * K + 6ull * K + 20);
 }
 
 // ---------------------------------------------------------------- block work
@@ -1135,6 +1138,7 @@ __global__ void __launch_bounds__(NL_THREADS, 1) node_loop_kernel(GraphDev g, Te
             break;
         }
         const int dg = S.deg[u], d = dg - 1;
+        const NlAcc before = acc;
         uint32_t mark = 0;
         if (S.T[u] > 0) {
             const bool elig = blocks && comp_eligible(d, l, tp);
@@ -1185,6 +1189,7 @@ __global__ void __launch_bounds__(NL_THREADS, 1) node_loop_kernel(GraphDev g, Te
         publish(seq <= 2u, mark);
         if (gather(seq <= 2u)) {
             handover = !timeout;
+            acc = before;                                // the other driver runs, and counts, the whole stage
             break;
         }
         apply(l, true);
