@@ -3005,10 +3005,10 @@ __device__ __forceinline__ bool lt_factor64(St &M, const Get &C, int l_rt, doubl
     return above_floor(h11) && above_floor(h22);
 }
 
-// sq |atanh r| to about 2e-9 of its value (it is returned as FP32).  atanh r = atanh c +
+// sq |atanh r| to about 5e-11 of its value (it is returned as FP32).  atanh r = atanh c +
 // atanh((r - c) / (1 - r c)) with c = tanh(0.34 k), k the nearest by FP32, leaves an
 // argument below 0.171 for |r| up to 0.99999, whose odd Taylor series to the 17th power runs in FP32
-// beyond its first term (below 1 % of it): 9 FP64 instructions for every lane.  Nearer to 1 the
+// beyond its first two terms (below 2e-4 of it): 11 FP64 instructions for every lane.  Nearer to 1 the
 // table has no entry: the library function, and infinity from 1 on.  (It
 // takes about 60, and one lane of a warp with |r| > 0.17 would be enough to pay them: the batch
 // of 1 M tests above ran at 271 us with it there, at 187 without.)
@@ -3027,7 +3027,8 @@ __device__ __forceinline__ double lt_fisher(double r, double sq)
     const int k = __float2int_rn(atanhf(af) * (1.0f / 0.34f));   // at most 18
     const double c = c_fisher[k];
     const double y = (a - c) * rcp_pivot(fma(-a, c, 1.0));
-    const float g = round_f32(y), x = g * g;
+    const double y2 = y * y;
+    const float x = round_f32(y2);
     float s = 1.0f / 17.0f;
     s = fmaf(s, x, 1.0f / 15.0f);
     s = fmaf(s, x, 1.0f / 13.0f);
@@ -3035,8 +3036,7 @@ __device__ __forceinline__ double lt_fisher(double r, double sq)
     s = fmaf(s, x, 1.0f / 9.0f);
     s = fmaf(s, x, 1.0f / 7.0f);
     s = fmaf(s, x, 1.0f / 5.0f);
-    s = fmaf(s, x, 1.0f / 3.0f);
-    return sq * (fma(y, f2d(s * x), y) + 0.34 * f2d((float)k));
+    return sq * (fma(y, fma(y2, 1.0 / 3.0, f2d(s * (x * x))), y) + 0.34 * f2d((float)k));
 }
 
 // f32: FP32 first under the trust rule (warp_test); else FP64 throughout, `skip32` telling

@@ -5,7 +5,7 @@ batched handles.
 
 The reference is the definition on the r the call returns: z = sqrt(n-l-3) atanh|r| in
 extended precision, infinite from |r| = 1 on.  Tolerances: an FP64-decided z is that value
-rounded to FP32 (6e-8) with a function error below 1e-8; an FP32-decided one (its r is an FP32 number) a
+rounded to FP32 (6e-8) with a function error below 1e-10; an FP32-decided one (its r is an FP32 number) a
 few FP32 roundings."""
 import numpy as np
 import pytest
