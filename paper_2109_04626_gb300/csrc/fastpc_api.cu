@@ -1972,8 +1972,11 @@ extern "C" pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats
     pc_status r;
     // a device output is expanded right behind the search, before its one wait
     const bool early = adj_out && !h->path_pool && is_device_ptr(adj_out);
-    if (h->path_pool) {
+    // (the exact product leaves NaN where it did not finish, which ends a search at once; the
+    // split-precision product leaves anything)
+    if (h->path_pool || !h->c32_rounded)
         if (pc_status c = check_tc(h)) return c;
+    if (h->path_pool) {
         r = skeleton_pathpool(h, &st);
     } else {
         h->adj_early = early ? adj_out : nullptr;
