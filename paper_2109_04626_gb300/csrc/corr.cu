@@ -1,6 +1,6 @@
 // corr.cu -- column standardisation and the correlation matrix
 // corr = Xs^T Xs / n (Sec. 4, the matrix corr): FP64 column statistics, FP64
-// and FP32 Gram kernels on the CUDA cores, and the FP64 -> FP32 cast.
+// and FP32 Gram kernels on the CUDA cores.
 #include "internal.h"
 #include <type_traits>
 #include "device_util.cuh"
@@ -790,14 +790,7 @@ cudaError_t launch_c64_lazy_init(double *C64, int ldc, unsigned char *valid, int
     return cudaGetLastError();
 }
 
-__global__ void cast_kernel(const double *C64, float *C32, int p, int ldc)
-{
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long tot = (long long)p * ldc;
-    if (i < tot) C32[i] = (float)C64[i];
-}
-
-// Batched problems: the same two steps on the diagonal block [o, o+pb) of a
+// Batched problems: the same on the diagonal block [o, o+pb) of a
 // matrix whose validity flags have row stride P.
 __global__ void c64_lazy_init_block_kernel(double *C64, int ldc, unsigned char *valid, int P, int o, int pb)
 {
@@ -810,30 +803,12 @@ __global__ void c64_lazy_init_block_kernel(double *C64, int ldc, unsigned char *
     }
 }
 
-__global__ void cast_block_kernel(const double *C64, float *C32, int ldc, int o, int pb)
-{
-    const long long tot = (long long)pb * pb;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long e = (long long)(o + (int)(i / pb)) * ldc + o + (int)(i % pb);
-        C32[e] = (float)C64[e];
-    }
-}
-
 cudaError_t launch_c64_lazy_init_block(double *C64, int ldc, unsigned char *valid, int P, int o, int pb,
                                        cudaStream_t s)
 {
     long long tot = (long long)pb * pb;
     c64_lazy_init_block_kernel<<<(unsigned)std::min<long long>((tot + 255) / 256, 8192), 256, 0, s>>>(
         C64, ldc, valid, P, o, pb);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cast_block(const double *C64, float *C32, int ldc, int o, int pb, cudaStream_t s)
-{
-    long long tot = (long long)pb * pb;
-    cast_block_kernel<<<(unsigned)std::min<long long>((tot + 255) / 256, 8192), 256, 0, s>>>(C64, C32, ldc, o, pb);
     note_launch();
     return cudaGetLastError();
 }
@@ -950,13 +925,6 @@ cudaError_t launch_syrk_f32(const float *Xs, long long n, long long ldk, int p, 
 {
     int nt = (p + 63) / 64;
     syrk_kernel<float, float><<<nt * (nt + 1) / 2, 256, 0, s>>>(Xs, n, ldk, p, C32, ldc); note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cast_c(const double *C64, float *C32, int p, int ldc, cudaStream_t s)
-{
-    long long tot = (long long)p * ldc;
-    cast_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C64, C32, p, ldc); note_launch();
     return cudaGetLastError();
 }
 

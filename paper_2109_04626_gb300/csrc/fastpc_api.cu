@@ -935,8 +935,9 @@ static pc_status split_product(pc_handle *h, const SplitBuffers &b, const void *
 // being decided on the spot instead of queued, their entries formed and re-read).
 static bool exact_corr(const pc_handle *h)
 {
+    if (h->precision == 0) return true;
     if (!fpc::tc_gemm_available() || h->precision == 1) return false;
-    if (h->precision == 0 || h->order == 1) return true;
+    if (h->order == 1) return true;
     int pm = h->nblk ? 0 : h->p;
     for (int i = 0; i < h->nblk; ++i) pm = std::max(pm, h->boff[i + 1] - h->boff[i]);
     return pm <= (h->nblk ? fpc::EXACT_BATCH_PMAX : fpc::NL_PMAX);
@@ -1024,23 +1025,18 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
                                want_bf16 ? h->Xhi + po : nullptr, want_bf16 ? h->Xlo + po : nullptr, h->ldk,
                                s));
     // FP64 correlations: all of them when a stage needs whole blocks (reversed
-    // order: closed-form stage, precision blocks) or the tests run in FP64;
-    // otherwise per entry on demand when a test is re-decided in FP64
+    // order: closed-form stage, precision blocks); otherwise per entry on demand
+    // when a test is re-decided in FP64
     h->c64_full = false;
     if (blk >= 0) {
-        if (h->precision == 0) {
-            if (pc_status r = syrk64_block(h, o, n, p, blk)) return r;
-        } else {
-            if (!h->c64_valid) {
-                // whole 32-bit words: the claims of c64_collect CAS the word of a flag
-                CK(dalloc(h, &h->c64_valid, (h->pair_elems + 7) / 4 * 4));
-                CK(cudaMemsetAsync(h->c64_valid, 0, (h->pair_elems + 7) / 4 * 4, s));
-                if (pc_status r = alloc_c64_list(h)) return r;
-            }
-            CK(fpc::launch_c64_lazy_init_block(h->C64 + h->pbase[blk], p, h->c64_valid + h->pbase[blk], p, 0, p,
-                                               s));
+        if (!h->c64_valid) {
+            // whole 32-bit words: the claims of c64_collect CAS the word of a flag
+            CK(dalloc(h, &h->c64_valid, (h->pair_elems + 7) / 4 * 4));
+            CK(cudaMemsetAsync(h->c64_valid, 0, (h->pair_elems + 7) / 4 * 4, s));
+            if (pc_status r = alloc_c64_list(h)) return r;
         }
-    } else if (h->precision == 0 || h->order == 1) {
+        CK(fpc::launch_c64_lazy_init_block(h->C64 + h->pbase[blk], p, h->c64_valid + h->pbase[blk], p, 0, p, s));
+    } else if (h->order == 1) {
         if (pc_status r = materialize_c64(h)) return r;
     } else {
         if (!h->c64_valid) {
@@ -1054,10 +1050,7 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
     float *C32b = blk < 0 ? h->C32 : h->C32 + h->pbase[blk];
     const int ldb = blk < 0 ? h->ldc : p;
     bool tc = false;
-    if (h->precision == 0) {
-        if (blk >= 0) CK(fpc::launch_cast_block(h->C64 + h->pbase[blk], h->C32 + h->pbase[blk], p, 0, p, s));
-        else CK(fpc::launch_cast_c(h->C64, h->C32, p, h->ldc, s));
-    } else if (h->precision == 1 || !want_bf16) {
+    if (!want_bf16) {
         if (h->precision == 2) {
             // tensor-core path not available on this device: FP32 operands on the CUDA cores
             CK(fpc::launch_standardize(Xd, dtype, n, p, ld, h->mean + o, h->rsd + o, stats_ws, nullptr, h->Xs32 + po,
@@ -1090,8 +1083,6 @@ static pc_status corr_impl(pc_handle *h, const void *X, int32_t dtype, int64_t l
         bool all = true;
         for (char d : h->bdone) all = all && d;
         h->have_corr = all;
-        // FP64 tests read whole blocks: every block was formed in full above
-        h->c64_full = all && h->precision == 0;
     }
     h->have_skel = false;
     return PC_OK;
@@ -1122,12 +1113,6 @@ extern "C" pc_status pc_corr_blocks(pc_handle *h, const void *const *X, const in
         if (!X[i] || (dtype[i] != PC_F32 && dtype[i] != PC_F64) || ld[i] < h->boff[i + 1] - h->boff[i])
             return fail(h, PC_ERR_ARG, "pc_corr_blocks: bad X, dtype or ld of instance " + std::to_string(i));
     const bool exact = exact_corr(h);
-    if (h->precision == 0 && !exact) {
-        // the FP64 Gram shares one split-K workspace: one instance after the other
-        for (int i = 0; i < k; ++i)
-            if (pc_status r = corr_impl(h, X[i], dtype[i], ld[i], i)) return r;
-        return PC_OK;
-    }
     cudaStream_t s = h->stream;
     Timed tm(h, 0);
     // what the instances share, on the handle's stream before the fork: the

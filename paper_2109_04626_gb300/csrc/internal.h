@@ -252,10 +252,8 @@ cudaError_t launch_gram_exact(const void *X, int dtype, long long n, int p, long
 cudaError_t launch_syrk_f32(const float *Xs, long long n, long long ldk, int p, float *C32,
                             int ldc, cudaStream_t s);
 cudaError_t launch_c64_lazy_init(double *C64, int ldc, unsigned char *valid, int p, cudaStream_t s);
-cudaError_t launch_cast_c(const double *C64, float *C32, int p, int ldc, cudaStream_t s);
 cudaError_t launch_c64_lazy_init_block(double *C64, int ldc, unsigned char *valid, int P, int o, int pb,
                                        cudaStream_t s);
-cudaError_t launch_cast_block(const double *C64, float *C32, int ldc, int o, int pb, cudaStream_t s);
 bool tc_gemm_available();
 cudaError_t launch_corr_bf16x3(const uint16_t *Xhi, const uint16_t *Xlo, long long n, long long ldk,
                                int p, float *C32, int ldc, float *ws, size_t ws_bytes, int *err,
