@@ -36,8 +36,9 @@ def fp(tmp_path_factory):
     stubs = sorted(m for m in missing if m.startswith(("_ZN3fpc", "cuda")))
     (d / "stubs.c").write_text("".join(f"int {m}(void) {{ return 999; }}\n" for m in stubs))
     lib = str(d / "libhost.so")
+    # (-Bsymbolic: its own fakes, also beside a CUDA runtime that the process has loaded)
     subprocess.run(["gcc", "-fPIC", "-c", str(d / "stubs.c"), "-o", str(d / "stubs.o")], check=True, timeout=60)
-    subprocess.run(["g++", "-shared", "-o", lib] + objs + [str(d / "stubs.o")], check=True, timeout=60)
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", lib] + objs + [str(d / "stubs.o")], check=True, timeout=60)
     spec = importlib.util.spec_from_file_location("fastpc_host", os.path.join(PKG, "fastpc.py"))
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
