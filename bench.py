@@ -60,7 +60,7 @@ CLASS_KERNELS = {
     "ci_complement": "ci_complement_kernel (FP64, from neighbourhood precision blocks)",
     "prec": "prec_update_kernel (neighbourhood precision blocks, FP64)",
     "stage_a": "stage_a sweep inverse (FP64)",
-    "corr": "pc_corr: column statistics, standardisation, correlation GEMM",
+    "corr": "pc_corr: column statistics, then the exact integer products or standardisation and BF16x3 GEMM",
     "stage_loop": "node_loop_kernel (one cooperative kernel over the whole search of a small problem, a CTA per "
                   "node: closed-form stage, FP32-first tests, commit, FP64 precision downdates)",
 }
@@ -535,31 +535,35 @@ def run_ours(args):
                 "largest_class": max(cls, key=lambda c: tim[c][0])}
 
     # the correlation step against the tensor roofline: useful flops n p (p+1) of the
-    # symmetric product (the BF16x3 split issues three products per useful one); the
-    # GEMM kernels alone (class corr_gemm) and the whole pc_corr (statistics,
-    # standardisation, GEMM, reduce)
+    # symmetric product (the BF16x3 split issues three products per useful one, the exact
+    # FP64 product 49); the GEMM kernels alone (class corr_gemm) and the whole pc_corr
+    # (statistics, standardisation, GEMM, reduce)
+    exact = mixed_prec == 0 or (mixed_prec == 2 and (fp.pc_get_opt(pc.h, "order") == 1 or p <= 128))
+    products = 49 if exact else 3 if mixed_prec == 2 else 1
     roofline_gemm = roofline_corr = None
     bf16, hbm, src = measured_peaks()
     gemm_flops = n * p * (p + 1)
     if tim["corr_gemm"][0] > 0:
         ach = gemm_flops / (tim["corr_gemm"][0] * 1e-3) / 1e12
-        roofline_gemm = {"bound": "tensor", "kernel": "corr_bf16x3_kernel (tcgen05, TMA) + corr_tc_reduce_kernel"
+        roofline_gemm = {"bound": "tensor", "kernel": "gram_exact_kernel (tcgen05) + gram_finish_kernel" if exact else
+                         "corr_bf16x3_kernel (tcgen05, TMA) + corr_tc_reduce_kernel"
                          if mixed_prec == 2 else "Gram kernel (CUDA cores)",
                          "achieved": ach, "peak": bf16, "unit": "TFLOP/s", "frac": ach / bf16,
-                         "issued_tflops": 3 * ach if mixed_prec == 2 else ach,
+                         "issued_tflops": products * ach,
                          "useful_flops_per_launch": gemm_flops, "ms_per_step": tim["corr_gemm"][0],
                          "launch_groups": tim["corr_gemm"][1],
                          "peak_source": f"bf16 dense burst, {src}"}
     if tim["corr"][0] > 0:
         ach = gemm_flops / (tim["corr"][0] * 1e-3) / 1e12
-        roofline_corr = {"bound": "tensor", "kernel": "pc_corr (column statistics, standardisation, "
-                         "BF16x3 tcgen05 GEMM, Kahan FP32 split-K reduce)" if mixed_prec == 2 else "pc_corr",
+        roofline_corr = {"bound": "tensor", "kernel": "pc_corr (column statistics, exact integer products)" if exact else
+                         "pc_corr (column statistics, standardisation, BF16x3 tcgen05 GEMM, Kahan FP32 split-K "
+                         "reduce)" if mixed_prec == 2 else "pc_corr",
                          "achieved": ach, "peak": bf16, "unit": "TFLOP/s", "frac": ach / bf16,
-                         "issued_tflops": 3 * ach if mixed_prec == 2 else ach, "ms_per_step": tim["corr"][0],
+                         "issued_tflops": products * ach, "ms_per_step": tim["corr"][0],
                          "peak_source": f"bf16 dense burst, {src}"}
 
     # Phase II of Algorithm 1 (pc_orient) on this skeleton: outside the metric's step,
-    # timed on its own (host wall time; pc_orient synchronises once per rule round)
+    # timed on its own (host wall time; pc_orient synchronises once)
     codes = np.empty((p, p), dtype=np.int8)
     fp.pc_orient(pc.h, p, codes)
     o_t = []
@@ -748,13 +752,17 @@ def run_many(args):
     dom = dominant_class(tim)
     di = cls.index(dom)
     flops_cls = list(st_t["flops_class"]) + [0.0]
-    dom_flops = flops_cls[di] if di > 0 else sum(2.0 * n_ * p_ * (p_ + 1) for n_, p_ in zip(ns, ps))
-    peak = FP64_PEAK_TFLOPS if dom in ("stage_a", "prec", "ci_complement") else FP32_PEAK_TFLOPS
+    # the correlation step: useful flops of the symmetric products against the tensor peak
+    dom_flops = flops_cls[di] if di > 0 else sum(float(n_) * p_ * (p_ + 1) for n_, p_ in zip(ns, ps))
+    bf16, _, src = measured_peaks()
+    peak = (bf16 if dom == "corr" else
+            FP64_PEAK_TFLOPS if dom in ("stage_a", "prec", "ci_complement") else FP32_PEAK_TFLOPS)
     achieved = dom_flops / (tim[dom][0] * 1e-3) / 1e12 if tim[dom][0] > 0 else 0.0
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "kernel": dom, "kernels": CLASS_KERNELS.get(dom, dom),
+    roofline = {"bound": "tensor" if dom == "corr" else "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak, "traffic": None, "kernel": dom, "kernels": CLASS_KERNELS.get(dom, dom),
                 "measured_on": "batched handle, timing step",
-                "peak_source": "nominal FP64 1.25 TFLOP/s" if peak == FP64_PEAK_TFLOPS else
+                "peak_source": f"bf16 dense burst, {src}" if dom == "corr" else
+                "nominal FP64 1.25 TFLOP/s" if peak == FP64_PEAK_TFLOPS else
                 "152 SMs x 128 FP32 lanes x 2 x 2.07 GHz", "class_ms": {c: tim[c][0] for c in cls},
                 "launch_groups": tim[dom][1], "largest_class": max(cls, key=lambda c: tim[c][0])}
 

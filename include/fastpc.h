@@ -189,7 +189,8 @@ pc_status pc_corr_get(pc_handle *h, float *C32, double *C64);
  * the Schur complement of Sec. 4.  Writes the skeleton into adj_out (p x p,
  * 0/1, symmetric, host or device; may be NULL) and the counters into stats
  * (host; may be NULL); a call that returns an error writes neither.  Sepsets
- * stay in the handle (pc_sepsets_*).  Requires a prior pc_corr.  Synchronises. */
+ * stay in the handle (pc_sepsets_*).  Requires a prior pc_corr.  Synchronises.
+ * PC_ERR_TIMEOUT when a bounded wait on the device expired (about 2 s). */
 pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats);
 
 /* pc_skeleton_many -- the skeleton searches of `count` independent problems

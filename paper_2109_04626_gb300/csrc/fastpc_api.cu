@@ -927,12 +927,21 @@ static pc_status split_product(pc_handle *h, const SplitBuffers &b, const void *
 
 // Does the correlation step form all FP64 correlations by the exact product from X itself
 // (C32 their rounding)?  Always for FP64 tests; FP32-first where the search needs all of
-// them (the reversed order) or they cost no more than the split-precision product with its
-// planes and the FP64 entries formed on demand: problems of p <= NL_PMAX, and batches of
-// instances of p <= EXACT_BATCH_PMAX, whose products fill the chip side by side
-// (64 instances of 50-400 variables and 2000-20000 samples: 4.5 ms for 3.1 with the
-// split-precision product, and in return the search takes 8-9 ms for 19-66, its FP64 tests
-// being decided on the spot instead of queued, their entries formed and re-read).
+// them (the reversed order), for problems of p <= NL_PMAX (in whose one-kernel search entries
+// on demand stand in the chain of a stage), and in batches of instances of p <= EXACT_BATCH_PMAX, whose products
+// fill the chip side by side.
+// Both sides (pc_corr and pc_skeleton, conventional order, sparse graphs of mean degree 8; exact /
+// split-precision with entries on demand, us):
+//   p =  60, n = 2000 / 20000:  152 /  235,   578 /  899
+//   p = 128:                    560 /  695,   815 / 1150
+//   p = 150:                    703 /  850,  1134 / 1355
+//   p = 300:                    950 / 1087,  1404 / 1545
+//   p = 500:                   1252 / 1422,  1850 / 1855
+//   8 instances, n = 8000: p = 200 1890 / 2099, 400 3470 / 3452, 512 4415 / 4200, 700 6257 / 5670
+// The line for one problem lies at NL_PMAX, although the exact product is still the better side up
+// to about p = 500.  The batch's lies above the 400 of equal times: strongly dependent data
+// queue FP64 tests that the other side pays dearly (64 dense instances of 50-400 variables: the
+// product 4.5 ms for 3.1, the search 8-9 ms for 19-66).
 static bool exact_corr(const pc_handle *h)
 {
     if (h->precision == 0) return true;

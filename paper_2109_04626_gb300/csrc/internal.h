@@ -74,7 +74,8 @@ struct StageConds {
     int has_comp, has_score, has_prec;  // which kernels the body has
 };
 // Batched handles whose instances have at most this many variables form all FP64
-// correlations at once (the exact product); larger ones form them on demand.
+// correlations at once (the exact product); larger ones form them on demand (both
+// sides measured at exact_corr).
 constexpr int EXACT_BATCH_PMAX = 512;
 constexpr int LANE_LMAX = 12;           // stages the lane-per-test kernel runs (FP32 modes)
 // Staged small-stage kernel: a node whose frozen degree is at most NODE_DMAX has

@@ -129,6 +129,9 @@ __device__ __forceinline__ bool pair_warped(const TestParams &tp, int l, int dg)
 }
 
 constexpr int PG1_PAIRS = 8, PG_PAIRS = 32;              // pairs of a group at stages 1 and 2
+// Sets of a stage-2 group that each warp walks for its own pairs, before the warps split the sets of
+// the pairs left.  128 / 256 / 512 (sparse graph of 1000 nodes, 500 nodes with a power law, 64 dense
+// instances; correlation and search, ms): 4.38 / 4.40 / 4.43, 1.79 / 1.79 / 1.80, 10.19 / 10.26 / 10.43.
 constexpr int PG_FIRST = 256;
 constexpr int PG_FLOATS = 12288;                         // rows corr[v, adj(u)] of a group: 48 KiB
 constexpr int PG_THREADS = 256;
@@ -1243,7 +1246,7 @@ __global__ void __launch_bounds__(NODE_THREADS, HI <= 2 ? 3 : (HI <= 4 ? 3 : (HI
 // lexicographic order, a lane per set.  The lane forms once what depends on u and S only
 // -- at stage 2 c = corr(s0, s1), x = 1 - c^2, the row of u eliminated by S, h11, and from
 // them the bound below -- and then tests the set against every pair of the group, with
-// corr(v, s0) and corr(v, s1): about 12 FP32 operations a test.
+// corr(v, s0) and corr(v, s1): 8 (stage 1) or 15 FP32 operations a test.
 //
 // Such a test decides only where the rule of fp32_trust certainly trusts FP32.  With
 // alpha_u^2 = A_u^2 / h11, alpha_v^2 = A_v^2 / h22 and eps = eps_c + 4 m eps32 that rule's
@@ -1818,6 +1821,8 @@ __device__ __forceinline__ void release_byte(unsigned char *flags, long long e)
 // pair, most of which an earlier set decides).  A queue of up to COLLECT_ALL tests lists them
 // all: the entries of a test on demand are a serial chain, 20000 samples each (stage 2 of the
 // 1000-node sparse graph, about 800 tests in all: the FP64 pass 315 us with the first tests only, 23 so).
+// Between 1024 and 16384 the limit makes no difference to that graph, to one of 500 nodes with a
+// power law or to 64 dense instances (0.3 %).
 constexpr ull COLLECT_ALL = 4096;
 __global__ void __launch_bounds__(256) c64_collect_kernel(GraphDev g, TestParams tp, const ull *queue,
                                                           const ull *qlen, ull qcap)
