@@ -1556,7 +1556,11 @@ static pc_status skeleton_enqueue(pc_handle *h)
     {
         Timed t(h, 5);
         CK(fpc::launch_level_degrees(g, s));
-        CK(fpc::launch_tail(g, tp, level_cap(h), 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, s));
+        // A split-precision product that did not finish leaves anything in its matrix, which may take any
+        // time to search: no stage of it (the exact product leaves NaN, which ends a search at once).
+        // On the device: a look at the word from the host before the search cost 50 us of it at p = 500.
+        CK(fpc::launch_tail(g, tp, level_cap(h), 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, h->tc_err,
+                            h->used_tc && !h->c32_rounded ? (h->nblk ? h->nblk : 1) : 0, s));
     }
     if (stage_a) {
         {
@@ -1574,7 +1578,7 @@ static pc_status skeleton_enqueue(pc_handle *h)
     }
     {
         Timed t(h, 5);
-        CK(fpc::launch_tail(g, tp, level_cap(h), 1, h->singular, stage_a, h->hcond, 0, fpc::StageConds{}, s));
+        CK(fpc::launch_tail(g, tp, level_cap(h), 1, h->singular, stage_a, h->hcond, 0, fpc::StageConds{}, nullptr, 0, s));
     }
     if (h->order == 1 && h->complement) {
         Timed t(h, 2);
@@ -1895,7 +1899,7 @@ static pc_status skeleton_pathpool_once(pc_handle *h, pc_stats *st, bool *overfl
         if (h->stage_a && n - p - 1 > 0) {
             // the closed-form stage l = p-2 on the complete graph (its only set is V\{u,v})
             CK(fpc::launch_level_degrees(g, s));
-            CK(fpc::launch_tail(g, tp, cap, 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, s));
+            CK(fpc::launch_tail(g, tp, cap, 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, nullptr, 0, s));
             CK(cudaMemcpyAsync(h->Pbuf, h->C64, (size_t)p * h->ldc * sizeof(double), cudaMemcpyDeviceToDevice, s));
             CK(fpc::launch_inverse_spd(h->Pbuf, p, h->ldc, h->work, h->singular, s));
             CK(fpc::launch_stage_a_decide(h->Pbuf, p, h->ldc, h->singular, g, tp, s));
@@ -1966,11 +1970,8 @@ extern "C" pc_status pc_skeleton(pc_handle *h, uint8_t *adj_out, pc_stats *stats
     pc_status r;
     // a device output is expanded right behind the search, before its one wait
     const bool early = adj_out && !h->path_pool && is_device_ptr(adj_out);
-    // (the exact product leaves NaN where it did not finish, which ends a search at once; the
-    // split-precision product leaves anything)
-    if (h->path_pool || !h->c32_rounded)
-        if (pc_status c = check_tc(h)) return c;
     if (h->path_pool) {
+        if (pc_status c = check_tc(h)) return c;
         r = skeleton_pathpool(h, &st);
     } else {
         h->adj_early = early ? adj_out : nullptr;

@@ -273,9 +273,10 @@ constexpr int LG_DIRECT = 24;          // direct-path stages a captured stage lo
 constexpr int DIRECT_MMAX = 160;       // largest (l+2) matrix one warp holds in shared memory
 cudaError_t launch_init_adj(GraphDev g, cudaStream_t s);
 cudaError_t launch_level_degrees(GraphDev g, cudaStream_t s);
+// err: nerr error words of the correlation product; one that is set halts the search with that error
 cudaError_t launch_tail(GraphDev g, TestParams tp, int cap, int mode, const int *stagea_singular,
                         int stagea_launched, cudaGraphConditionalHandle hc, int use_cond, StageConds sc,
-                        cudaStream_t s);
+                        const int *err, int nerr, cudaStream_t s);
 cudaError_t launch_head(GraphDev g, TestParams tp, double budget, int mmax_direct, StageConds sc, cudaStream_t s);
 cudaError_t launch_ci_direct(GraphDev g, TestParams tp, int mmax, const float *C32,
                              const double *C64, int ldc, cudaStream_t s);

@@ -312,8 +312,15 @@ __device__ void tail_body(GraphDev g, TestParams tp, int cap, int mode, const in
 
 __global__ void __launch_bounds__(1024) tail_kernel(GraphDev g, TestParams tp, int cap, int mode,
                                                     const int *stagea_singular, int stagea_launched,
-                                                    cudaGraphConditionalHandle hc, int use_cond, StageConds sc)
+                                                    cudaGraphConditionalHandle hc, int use_cond, StageConds sc,
+                                                    const int *err, int nerr)
 {
+    for (int i = threadIdx.x; i < nerr; i += blockDim.x)
+        if (err[i]) {
+            g.info->error = err[i];
+            g.info->halt = 1;
+        }
+    __syncthreads();
     tail_body(g, tp, cap, mode, stagea_singular, stagea_launched, hc, use_cond, sc, false);
 }
 
@@ -3518,9 +3525,10 @@ cudaError_t launch_degrees_tail(GraphDev g, TestParams tp, int cap, cudaGraphCon
 
 cudaError_t launch_tail(GraphDev g, TestParams tp, int cap, int mode, const int *stagea_singular,
                         int stagea_launched, cudaGraphConditionalHandle hc, int use_cond, StageConds sc,
-                        cudaStream_t s)
+                        const int *err, int nerr, cudaStream_t s)
 {
-    tail_kernel<<<1, stage_threads(g.p), 0, s>>>(g, tp, cap, mode, stagea_singular, stagea_launched, hc, use_cond, sc);
+    tail_kernel<<<1, stage_threads(g.p), 0, s>>>(g, tp, cap, mode, stagea_singular, stagea_launched, hc, use_cond, sc, err,
+                                                 nerr);
     note_launch();
     return cudaGetLastError();
 }

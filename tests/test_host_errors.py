@@ -170,13 +170,19 @@ def test_device_skeleton_of_a_failed_product(fp):
         assert (out == 1).all()
 
 
-def test_no_search_on_an_unfinished_split_product(fp):
-    """Its matrix holds anything where it did not finish, and a search of it can take any time: refused
-    before the first stage."""
-    with fp.PC(40, 150, 0.01, order=0) as pc:
-        fp.fail(0, 1)
-        pc.corr(np.zeros((40, 150)))
+@pytest.mark.parametrize("batch", [False, True])
+def test_no_search_on_an_unfinished_split_product(fp, batch):
+    """Its matrix holds anything where it did not finish, and a search of it can take any time: halted
+    on the device before the first stage."""
+    with _batch(fp, LARGE, graph=0) if batch else fp.PC(40, 150, 0.01, order=0, graph=0) as pc:
+        before = fp.load().fake_halted()
+        fp.fail(0, 2 if batch else 1)
+        for i, x in enumerate(LARGE) if batch else []:
+            pc.corr_block(i, x)
+        if not batch:
+            pc.corr(np.zeros((40, 150)))
         fp.fail()
         with pytest.raises(fp.PCError) as e:
             pc.skeleton()
         assert e.value.status == TIMEOUT
+        assert fp.load().fake_halted() == before + 1
