@@ -859,8 +859,10 @@ static pc_status alloc_planes(pc_handle *h, cudaStream_t s)
 // SMs idle at the sizes where a search takes less than a millisecond).  pc_corr joins the last
 // read of the caller's data; the product itself, which outlasts the exact one by 10-40 us at
 // p = 20-100 (joined there, p = 55, n = 5000: the search 179 -> 197 us, so 177), is joined where it
-// is read or written again (split_join), and under a capture at once.  Its planes, statistics, workspace and
-// matrix are one allocation, made at the first pc_corr.
+// is read or written again (split_join), and under a capture at once.  (In a process where the side
+// streams of many handles, or eight streams of its own, have run kernels, a captured search of
+// p = 500-1000 takes 25-40 us longer.)  Its planes, statistics, workspace and matrix are one
+// allocation, made at the first pc_corr.
 struct SplitBuffers {
     size_t plane, c32, sws, tws;
     uint16_t *hi, *lo;
@@ -1558,7 +1560,7 @@ static pc_status skeleton_enqueue(pc_handle *h)
         CK(fpc::launch_level_degrees(g, s));
         // A split-precision product that did not finish leaves anything in its matrix, which may take any
         // time to search: no stage of it (the exact product leaves NaN, which ends a search at once).
-        // On the device: a look at the word from the host before the search cost 50 us of it at p = 500.
+        // On the device: the host issues the search while the correlation step runs.
         CK(fpc::launch_tail(g, tp, level_cap(h), 2, h->singular, 0, h->hcond, 0, fpc::StageConds{}, h->tc_err,
                             h->used_tc && !h->c32_rounded ? (h->nblk ? h->nblk : 1) : 0, s));
     }
